@@ -111,10 +111,11 @@ cbct_status cbct_geometry_destroy(cbct_geometry *geom);
  * ray tracing): g_i = sum_j a_ij f_j, a_ij = length (mm) of ray i inside voxel j.
  * f: device [nz][ny][nx]; g: device [n_views][nv][nu]. FP32 arithmetic.
  * Uses the geometry's scratch (allocated on first use, grown when too small): the volume in
- * the projector's z-fastest layout and the grid's ray-trace table, 16 + 8 (nx + ny + 2)
- * bytes per (view, imager column). Every projection block copies its trace record with a
- * bounded wait; should that wait ever run out, the block's rows are written as NaN (the
- * call itself cannot see it; cbct_reconstruct reports it as TIMEOUT).
+ * the projector's z-fastest layout (z-lines padded to a multiple of 4 values) and the grid's
+ * ray-trace table, about 64 + 8 (nx + ny + 2) bytes per (view, imager column). A projection
+ * block waits for its asynchronous copies with a limit; should a wait ever run out, the
+ * block's rows are written as NaN (the call itself cannot see it; cbct_reconstruct reports
+ * it as TIMEOUT).
  */
 cbct_status cbct_project(const cbct_geometry *geom, const float *f, float *g,
                          cbct_stream_t stream);
@@ -228,8 +229,7 @@ cbct_status cbct_cgls(const cbct_geometry *geom, const float *y, float *x, int n
  * Uses the geometry's reconstruction workspace (allocated on first use; its size is
  * cbct_reconstruct_workspace_size). Synchronises the stream at the end.
  * Errors: INVALID_ARG, UNSUPPORTED, OUT_OF_MEMORY, CUDA, NONFINITE; TIMEOUT if a
- * projector block's bounded wait for its precomputed ray trace ran out (its rows are then
- * NaN).
+ * projector block's bounded wait for its copies ran out (its rows are then NaN).
  */
 cbct_status cbct_reconstruct(const float *y, const cbct_geometry *geom, float mu,
                              float lambda, int levels, const int *iters, float *f_out,
@@ -284,16 +284,16 @@ cbct_status cbct_count_nnz(const cbct_geometry *geom, int level, unsigned long l
  * allocation as a failure, or a latency-critical loop that cannot afford the device-wide
  * synchronisation an allocation may cause. The paper has no counterpart: this is an
  * interface variant, not a step of the method. Instead of the geometry's lazily
- * allocated scratch it uses one fixed scratch array of CBCT_PROJECT_STATIC_MAX_VOXELS
- * floats that the library places on every GPU that loads it, held until the process
- * exits. Volumes larger than that are rejected with CBCT_ERR_INVALID_ARG. The geometry
- * must have been created beforehand. The first call on a device looks up the array's
- * device address (cudaGetSymbolAddress) and keeps it for the life of the process; make
+ * allocated scratch it uses fixed scratch arrays (CBCT_PROJECT_STATIC_MAX_VOXELS floats for
+ * the volume, 8 MiB for ray traces, which a larger call goes through in batches) that the
+ * library places on every GPU that loads it, held until the process exits. Volumes larger than that are rejected with CBCT_ERR_INVALID_ARG. The geometry
+ * must have been created beforehand. The first call on a device looks up the arrays'
+ * device addresses (cudaGetSymbolAddress) and keeps them for the life of the process; make
  * that first call before any stream capture. A device reset (cudaDeviceReset) after the
- * first call is not supported: the kept address would no longer be valid. All calls
- * share the one array, so calls whose work overlaps on the GPU (different streams, or
+ * first call is not supported: the kept addresses would no longer be valid. All calls
+ * share the arrays, so calls whose work overlaps on the GPU (different streams, or
  * several host threads) race and must be serialised by the caller. Each call overwrites
- * the part of the array it uses before reading it, so no clearing is needed.
+ * the part of the arrays it uses before reading it, so no clearing is needed.
  */
 #define CBCT_PROJECT_STATIC_MAX_VOXELS 4194304
 cbct_status cbct_project_static(const cbct_geometry *geom, const float *f, float *g,
@@ -404,9 +404,9 @@ cbct_status cbct_server_destroy(cbct_server *srv);
 /*
  * Column groups of the projector (tuning and testing; not part of the paper's method).
  * Along each ray's transverse trace (Section 2.2.1's Siddon walk) the projector stages the
- * voxel columns in groups of 16, 24, 32, 40, 48, 56, 64, 80 or 96 and, by default, picks
- * the size per launch from an estimate of its per-group cost and of the blocks it keeps
- * resident per SM. Results of different group sizes agree to FP32 rounding (the sums are
+ * voxel columns in groups of 16, 24, 32, 40, 48, 56, 64, 80 or 96 (by its own choice it may
+ * tabulate two groups of 56 together) and, by default, picks the size per launch from an
+ * estimate of its per-table cost and of the blocks it keeps resident per SM. Results of different group sizes agree to FP32 rounding (the sums are
  * associated differently).
  *
  * cbct_set_project_group: process-wide; 0 restores the automatic choice, one of the sizes

@@ -12,8 +12,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libcbcttf.so")
-SOURCES = ["geometry.cu", "project.cu", "project_groups_16_32.cu", "project_groups_40_56.cu",
-           "project_groups_64_96.cu", "project_trace.cu", "backproject.cu", "tf.cu", "recon.cu", "project_static.cu",
+SOURCES = ["geometry.cu", "project.cu", "project_q4.cu", "project_q8.cu",
+           "project_trace.cu", "backproject.cu", "tf.cu", "recon.cu", "project_static.cu",
            "serve.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -1,10 +1,11 @@
 // Internal declarations of the cbcttf CUDA library (not part of the C ABI).
 //
 // Internal data layouts (the public ABI converts at its boundary):
-//   volumes inside the iteration are z-fastest, [ny][nx][nz], so that the projector's
-//   warps, whose lanes are adjacent imager rows, read adjacent z voxels of one (x, y)
-//   column; public volumes are x-fastest [nz][ny][nx]. Kernels that touch volumes take
-//   the element strides (sx, sy, sz) so they serve both layouts.
+//   volumes inside the iteration are z-fastest, [ny][nx][zp], so that a voxel column's
+//   z-line is contiguous; zp = nz rounded up to a multiple of 4, so that every line starts
+//   on a 16-byte boundary and is read in 16-byte pieces (the up to 3 padding values of a
+//   line are never part of a result). Public volumes are x-fastest [nz][ny][nx]. Kernels
+//   that touch volumes take the element strides (sx, sy, sz) so they serve both layouts.
 //   projection stacks are always [n_views][nv][nu].
 #pragma once
 
@@ -27,6 +28,7 @@ namespace cbct {
 // the source orbit lies in the plane z = 0 and the imager's v axis is z).
 struct GeomDev {
     int nx, ny, nz;
+    int zp;                 // floats per z-line of the internal layout: nz rounded up to 4
     float dx, dy, dz;
     float x0, y0, z0;       // volume corner, -n * d / 2
     int nu, nv, nviews;
@@ -180,28 +182,33 @@ int device_sm_count();
 // Launchers (all asynchronous on `st`; return CBCT_ERR_CUDA on launch failure).
 // Volume element (ix, iy, iz) lives at ix*sx + iy*sy + iz*sz.
 int project_num_blocks(const GeomDev &G);
-// Bytes past the end of a volume that the projector may read (its 16-byte staging copies
-// round the last z-line up): every volume buffer passed to launch_project is allocated with
-// at least this much slack, and its base is 16-byte aligned.
+// Elements of a volume in the internal layout.
+static inline size_t internal_elems(const GeomDev &G) { return (size_t)G.nx * G.ny * G.zp; }
+// Bytes past the end of a volume that the projector may read (the unpadded layout's last
+// z-line is read up to a multiple of 4 values): every volume buffer passed to
+// launch_project is allocated with at least this much slack, and its base is 16-byte aligned.
 constexpr size_t PROJECT_VOLUME_SLACK = 64;
 
 // Dynamic shared memory a projector block may use (opted in per kernel).
 constexpr size_t PROJECT_SMEM_LIMIT = 200 * 1024;
 
 // out holds `storage`-typed values (PM_COUNT: none); y is FP32; sc supplies kappa in
-// PM_Q_SCALED and, when given, receives bit 1 of its flags if a block's wait for its trace
-// record timed out (that block's rows are NaN). With FP32 storage the CGLS modes store
-// |D - S| r and |D - S| q. traces: the grid's trace table from launch_trace_table built with
-// the same sx, sy (the projector then copies each column's phase 1 instead of computing
-// it), or nullptr.
-cbct_status launch_project(const GeomDev &G, const float *f, long long sx, long long sy,
-                           long long sz, const float *y, void *out, int mode,
-                           double *partials, float count_thr, cudaStream_t st,
-                           int storage = ST_F32, Scalars *sc = nullptr, const void *traces = nullptr);
-// The projector's trace table of a grid (trace_table_bytes(G) bytes, 16-byte aligned):
-// phase 1 of every (view, imager column), column offsets for the strides sx, sy.
+// PM_Q_SCALED and, when given, receives bit 1 of its flags if a block's wait for its copies
+// ran out (its rows are NaN). With FP32 storage the CGLS modes store |D - S| r and |D - S| q.
+// f is in the internal layout with z-lines of zpitch floats: G.zp, or G.nz for a volume without
+// padding (PM_PLAIN with FP32 storage only; the same results from narrower loads). traces: the
+// trace table from launch_trace_table (PM_COUNT: none); only the (view, imager column) pairs
+// [col_first, col_first + ncols) are projected, whose records are its first (ncols = 0: all).
+// npartials, when given, receives the number of partial sums written, at most
+// project_num_blocks(G).
+cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const float *y, void *out, int mode,
+                           double *partials, float count_thr, cudaStream_t st, int storage, Scalars *sc,
+                           const void *traces, int *npartials = nullptr, int col_first = 0, int ncols = 0);
+// The projector's trace table of a grid (trace_table_bytes(G) bytes for all columns, 16-byte
+// aligned): the transverse trace of the (view, imager column) pairs [col_first, col_first + ncols)
+// (ncols = 0: all).
 size_t trace_table_bytes(const GeomDev &G);
-cbct_status launch_trace_table(const GeomDev &G, long long sx, long long sy, void *tab, cudaStream_t st);
+cbct_status launch_trace_table(const GeomDev &G, void *tab, cudaStream_t st, int col_first = 0, int ncols = 0);
 cbct_status trace_table_prepare();
 int backproject_num_blocks(const GeomDev &G);
 // Upper bound of backproject_num_blocks over every grid no larger than G's (any z chunk).
@@ -223,11 +230,12 @@ cbct_status launch_tf_analyze(int n0, int n1, int n2, const float *f, void *alph
 cbct_status launch_tf_synth_shrink(int n0, int n1, int n2, const void *alpha, float mu,
                                    int positivity, float *f, cudaStream_t st, int storage = ST_F32);
 // Fused f_new = H(W^T T_mu W x) and, if vout != nullptr, v = f_new + coef (f_new - f_old).
-cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, const float *x, float mu, int positivity,
+// p0 >= n0: elements from one row along axis 0 to the next, of every array.
+cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *x, float mu, int positivity,
                                    float *fnew, const float *fold, float coef, float *vout,
                                    cudaStream_t st);
-// Public x-fastest [nz][ny][nx] <-> internal z-fastest [ny][nx][nz] volume layout.
-cbct_status transpose(const float *in, float *out, int nx, int ny, int nz, bool to_internal,
+// Public x-fastest [nz][ny][nx] <-> internal z-fastest [ny][nx][zpitch] volume layout.
+cbct_status transpose(const float *in, float *out, int nx, int ny, int nz, int zpitch, bool to_internal,
                       cudaStream_t st);
 
 } // namespace cbct

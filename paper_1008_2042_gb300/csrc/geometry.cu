@@ -125,6 +125,7 @@ GeomDev level_geom(const cbct_geometry *g, int level)
     G.nx = (d.nx + s - 1) / s;
     G.ny = (d.ny + s - 1) / s;
     G.nz = (d.nz + s - 1) / s;
+    G.zp = (G.nz + 3) & ~3;
     double dx = d.dx * s, dy = d.dy * s, dz = d.dz * s;
     G.dx = (float)dx;
     G.dy = (float)dy;
@@ -389,10 +390,9 @@ extern "C" cbct_status cbct_count_nnz(const cbct_geometry *gc, int level, unsign
     if (st != CBCT_OK) return st;
     double *partials = (double *)g->d_scratch;
     float thr = 1e-3f * fminf(G.dx, fminf(G.dy, G.dz));
-    long long sz = 1, sx = G.nz, sy = (long long)G.nx * G.nz;
     // counting mode reads no volume
-    st = launch_project(G, nullptr, sx, sy, sz, nullptr, nullptr, PM_COUNT, partials, thr,
-                        (cudaStream_t)stream);
+    st = launch_project(G, nullptr, G.zp, nullptr, nullptr, PM_COUNT, partials, thr, (cudaStream_t)stream,
+                        ST_F32, nullptr, nullptr);
     if (st != CBCT_OK) return st;
     double *h = (double *)malloc(sizeof(double) * nb);
     if (!h) return set_error(CBCT_ERR_OUT_OF_MEMORY, "count_nnz: host allocation");

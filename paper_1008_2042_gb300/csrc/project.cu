@@ -3,6 +3,7 @@
 // itself is in project_kernel.cuh.
 #include <atomic>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -13,27 +14,44 @@ namespace cbct {
 
 int project_num_blocks(const GeomDev &G)
 {
-    const int rows = 2 * proj_threads(G);
+    const int rows = proj_rows_per_thread(G) * proj_threads(G);
     return G.nviews * G.nu * ((G.nv + rows - 1) / rows);
 }
 
-// the smallest group needs the least shared memory: a grid is accepted when it fits
-size_t project_smem_bytes(const GeomDev &G) { return project_smem(G, PROJECT_GROUP_SIZES[0]); }
-
-static const void *kernel_for(int sg, int mode, int storage)
+// The documented limit of the accepted grids: 16 bytes per possible segment (in groups of
+// 16) and per slab 16 staged values, 17 table entries and two totals. The kernel's own need
+// with the smallest group (project_smem) is below it for every grid.
+size_t project_smem_bytes(const GeomDev &G)
 {
-    switch (sg) {
-    case 16: return project_kernel<16>(mode, storage);
-    case 24: return project_kernel<24>(mode, storage);
-    case 32: return project_kernel<32>(mode, storage);
-    case 40: return project_kernel<40>(mode, storage);
-    case 48: return project_kernel<48>(mode, storage);
-    case 56: return project_kernel<56>(mode, storage);
-    case 64: return project_kernel<64>(mode, storage);
-    case 80: return project_kernel<80>(mode, storage);
-    case 96: return project_kernel<96>(mode, storage);
-    default: return nullptr;
+    const size_t segs = ((size_t)G.nx + G.ny + 2 + 15) / 16 * 16;
+    const size_t lists = ((size_t)G.nx + G.ny + 2 + 3) / 4 * 4, lines = 16 * (((size_t)G.nz + 9) / 4 * 4);
+    return 16 * segs + sizeof(float) * ((lines > lists ? lines : lists) + (size_t)G.nz * 19);
+}
+
+// Quads of slabs per warp in the table build, 4 or 8: with 8 there are half the parts, of twice
+// the columns, so fewer passes end in a scan (each pass costs about 8 instructions per column
+// and 60 around them), but the longest chain doubles. The split with the least total work plus
+// longest chain. Measured with groups of 80 (4 | 8): 18 quads on 6 warps 661 | 703 us, 16 quads
+// 206 | 187 us, 9 quads 315 | 355 us, 5 quads 185 | 211 us (the orders hold for the sizes used).
+static int quads_per_warp(const GeomDev &G, int threads, int sg)
+{
+    const int nq = G.zp / 4, warps = threads / 32;
+    int best = 8, best_cost = 1 << 30;
+    for (int qw = 8; qw >= 4; qw /= 2) {
+        if (nq > 16 * qw && qw < 8) break; // more parts take more shared memory for their offsets
+        const int passes = (nq + qw - 1) / qw, rounds = (passes + warps - 1) / warps;
+        const int cost = (passes + rounds) * (8 * ((sg * qw + 31) / 32) + 60);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = qw;
+        }
     }
+    return best;
+}
+
+static const void *kernel_for(int qw, int mode, int storage, int rows, int fill)
+{
+    return qw == 4 ? project_kernel<4>(mode, storage, rows, fill) : project_kernel<8>(mode, storage, rows, fill);
 }
 
 static int group_index(int sg)
@@ -43,17 +61,18 @@ static int group_index(int sg)
     return -1;
 }
 
-// per-device record of the shared-memory opt-in, one per (group size, mode, storage)
-static std::atomic<unsigned long long> g_optin[PROJECT_N_GROUP_SIZES][4][3];
+// per-device record of the shared-memory opt-in, one per instantiation
+static std::atomic<unsigned long long> g_optin[2][3][3][2][3];
 
-static cbct_status optin(int sg, int mode, int storage, const void **fn)
+static cbct_status optin(int qw, int mode, int storage, int rows, int fill, const void **fn)
 {
-    *fn = kernel_for(sg, mode, storage);
-    if (!*fn) return set_error(CBCT_ERR_UNSUPPORTED, "project: no kernel for group %d, mode %d", sg, mode);
+    *fn = kernel_for(qw, mode, storage, rows, fill);
+    if (!*fn) return set_error(CBCT_ERR_UNSUPPORTED, "project: no kernel for mode %d, storage %d", mode, storage);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return check_cuda(e, "project device");
-    std::atomic<unsigned long long> &done = g_optin[group_index(sg)][mode][storage == ST_BF16 ? 1 : storage == ST_F16 ? 2 : 0];
+    std::atomic<unsigned long long> &done =
+        g_optin[qw / 8][mode][storage == ST_BF16 ? 1 : storage == ST_F16 ? 2 : 0][rows - 1][fill];
     const unsigned long long bit = 1ull << (dev & 63);
     if (done.load() & bit) return CBCT_OK;
     e = cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PROJECT_SMEM_LIMIT);
@@ -64,69 +83,87 @@ static cbct_status optin(int sg, int mode, int storage, const void **fn)
 
 static std::atomic<int> g_forced_group{0}; // 0: automatic
 
-// The group size of a launch. Two effects compete (measured on GB300 over group sizes,
-// register budgets and seven grids): a group pays a fixed cost (barriers, the copy loop,
-// the running totals) that a larger group spreads over more columns, and a larger group
-// needs more shared memory, so fewer blocks stay resident to hide each other's latency.
-// Where each slab's prefix chain is split in two (threads >= 2 nz) the estimate
-//     (1 + GROUP_COST / sg) * (REF_WARPS / resident warps)^OCC_EXP
-// with GROUP_COST = 17 columns, REF_WARPS = 24 and OCC_EXP = 0.6 ranks the sizes as the
-// measurements do; without the split the chain's latency grows with the group and the
-// most resident blocks win. Resident blocks come from the occupancy query (registers,
-// threads and shared memory of that instantiation). Ties go to the larger group. Cached
-// per device, mode, storage, block size and the grid extents the shared memory depends on.
-constexpr double GROUP_COST = 17.0, REF_WARPS = 24.0, OCC_EXP = 0.6;
+static int fill_of(const GeomDev &G, int zpitch)
+{
+    return zpitch % 4 ? FILL_PACKED : G.zp <= TMA_BOX_MAX ? FILL_GATHER : FILL_BULK;
+}
 
-static cbct_status choose_group(const GeomDev &G, int threads, int mode, int storage, int *sg_out)
+struct GroupChoice {
+    int sg, qw, grid; // columns per group, quads per warp, resident blocks on the device
+    ProjPlan plan;
+    size_t smem;
+};
+
+// Tables of `groups` groups of sg columns; one line buffer where two do not fit.
+static bool make_plan(const GeomDev &G, int threads, int sg, int groups, GroupChoice *c)
+{
+    c->sg = sg;
+    c->qw = quads_per_warp(G, threads, sg * groups);
+    for (int nbuf = 2; nbuf >= 1; --nbuf) {
+        c->plan = project_plan(G, sg * groups, c->qw, nbuf);
+        c->smem = project_smem(G, c->plan, c->qw);
+        if (c->smem <= PROJECT_SMEM_LIMIT) return true;
+    }
+    return false;
+}
+
+// The group size of a launch. A table costs its block about as much as building and walking 60
+// columns (the waits, the barrier, the scans, the rows' set-up), which a larger table spreads
+// over more columns; but it takes more shared memory, so fewer blocks stay resident to fill
+// each other's waits:
+//     (1 + TABLE_COST / columns) * (REF_WARPS / resident warps)^OCC_EXP,
+// a tenth more where the build's accesses share banks, a twentieth more where it is not unrolled
+// (tables other than 80 and 112 columns). Measured (us, columns: 48 | 80 | 112):
+// the paper's finest grid 857 | 647 | 660 (4, 4, 3 blocks), its level 1 395 | 302 | 271, its level
+// 2 247 | 179 | 168, 256x256x64 240 | 186 | 201, 512x512x128 971 | 1014 | 1680 (4, 2, 1 blocks).
+constexpr double TABLE_COST = 60.0, REF_WARPS = 24.0, OCC_EXP = 0.6;
+
+static cbct_status choose_group(const GeomDev &G, int threads, int mode, int storage, int fill, GroupChoice *out)
 {
     const int forced = g_forced_group.load();
-    if (mode == PM_COUNT) {
-        *sg_out = PROJECT_GROUP_SIZES[0];
-        return CBCT_OK;
-    }
-    if (forced && project_smem(G, forced) <= PROJECT_SMEM_LIMIT) {
-        *sg_out = forced;
-        return CBCT_OK;
-    }
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return check_cuda(e, "project device");
-    using Key = std::tuple<int, int, int, int, int, int>;
+    using Key = std::tuple<int, int, int, int, int, int, int>;
     static std::mutex mu;
-    static std::map<Key, int> cache;
-    const Key key{dev, mode, storage, threads, G.nz, G.nx + G.ny};
+    static std::map<Key, GroupChoice> cache;
+    const Key key{dev, mode, storage, threads, G.nz, fill, forced};
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
         if (it != cache.end()) {
-            *sg_out = it->second;
+            *out = it->second;
             return CBCT_OK;
         }
     }
-    const bool split = threads >= 2 * G.nz;
-    int best = PROJECT_GROUP_SIZES[0];
+    GroupChoice best{}, c{};
+    const bool use_forced = forced && make_plan(G, threads, forced, 1, &c);
     double best_cost = 1e300;
-    for (int i = 0; i < PROJECT_N_GROUP_SIZES; ++i) {
-        const int sg = PROJECT_GROUP_SIZES[i];
-        const size_t smem = project_smem(G, sg);
-        if (smem > PROJECT_SMEM_LIMIT) break; // grows with sg
+    for (int i = 0; i <= PROJECT_N_GROUP_SIZES; ++i) {
+        const int groups = i < PROJECT_N_GROUP_SIZES ? 1 : 2, sg = groups == 1 ? PROJECT_GROUP_SIZES[i] : 56;
+        if ((use_forced && (sg != forced || groups > 1)) || !make_plan(G, threads, sg, groups, &c)) continue;
         const void *fn = nullptr;
-        cbct_status r = optin(sg, mode, storage, &fn);
+        cbct_status r = optin(c.qw, mode, storage, fill == FILL_GATHER ? proj_rows_per_thread(G) : 2, fill, &fn);
         if (r != CBCT_OK) return r;
         int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads + 32, c.smem);
         if (e != cudaSuccess) return check_cuda(e, "project occupancy");
         if (nb < 1) continue;
+        c.grid = nb * device_sm_count();
         const double warps = (double)nb * (threads / 32);
-        const double cost = split ? (1.0 + GROUP_COST / sg) * std::pow(REF_WARPS / warps, OCC_EXP) : 1.0 / warps;
+        const bool banks = c.qw == 4 && c.plan.nb * c.plan.pitch % 32 != 16;
+        const bool unrolled = c.plan.sg == 80 || c.plan.sg == 112;
+        const double cost = (1.0 + TABLE_COST / c.plan.sg) * std::pow(REF_WARPS / warps, OCC_EXP) * (banks ? 1.1 : 1.0) *
+                            (unrolled ? 1.0 : 1.05);
         if (cost <= best_cost) {
             best_cost = cost;
-            best = sg;
+            best = c;
         }
     }
+    if (!best.sg) return set_error(CBCT_ERR_UNSUPPORTED, "project: grid too large for the projector's shared memory (nx + ny and nz)");
     std::lock_guard<std::mutex> lk(mu);
     cache[key] = best;
-    *sg_out = best;
+    *out = best;
     return CBCT_OK;
 }
 
@@ -138,48 +175,99 @@ cbct_status project_set_group(int sg)
     return CBCT_OK;
 }
 
-cbct_status project_group_of(const GeomDev &G, int *sg) { return choose_group(G, proj_threads(G), PM_PLAIN, ST_F32, sg); }
+cbct_status project_group_of(const GeomDev &G, int *sg)
+{
+    GroupChoice c{};
+    const cbct_status st = choose_group(G, proj_threads(G), PM_PLAIN, ST_F32, fill_of(G, G.zp), &c);
+    *sg = c.sg;
+    return st;
+}
 
 cbct_status project_prepare()
 {
     cbct_status t = trace_table_prepare();
     if (t != CBCT_OK) return t;
-    for (int i = 0; i < PROJECT_N_GROUP_SIZES; ++i)
-        for (int mode = PM_PLAIN; mode <= PM_COUNT; ++mode)
-            for (int storage = ST_F32; storage <= ST_F16; ++storage) {
-                if (mode == PM_COUNT && (i > 0 || storage != ST_F32)) continue;
-                const void *fn = nullptr;
-                cbct_status r = optin(PROJECT_GROUP_SIZES[i], mode, storage, &fn);
-                if (r != CBCT_OK) return r;
-            }
+    for (int qw = 4; qw <= 8; qw *= 2)
+        for (int mode = PM_PLAIN; mode < PM_COUNT; ++mode)
+            for (int storage = ST_F32; storage <= ST_F16; ++storage)
+                for (int rows = 1; rows <= 2; ++rows)
+                    for (int fill = FILL_GATHER; fill <= FILL_BULK; ++fill) {
+                        const void *fn = nullptr;
+                        cbct_status r = optin(qw, mode, storage, rows, fill, &fn);
+                        if (r != CBCT_OK) return r;
+                    }
     return CBCT_OK;
 }
 
-cbct_status launch_project(const GeomDev &G, const float *f, long long sx, long long sy,
-                           long long sz, const float *y, void *out, int mode,
-                           double *partials, float count_thr, cudaStream_t st, int storage, Scalars *sc,
-                           const void *traces)
+// cuTensorMapEncodeTiled, from the driver the runtime has loaded (no link to libcuda).
+using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+static EncodeTiled encode_tiled()
 {
-    const int threads = proj_threads(G); // 2 rows each
-    dim3 grid((unsigned)(G.nviews * G.nu), (unsigned)((G.nv + 2 * threads - 1) / (2 * threads)));
+    static const EncodeTiled fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q);
+        if (e != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
+        return reinterpret_cast<EncodeTiled>(p);
+    }();
+    return fn;
+}
+
+// The volume as a matrix of nx ny lines of zp values; a box is one line of `pitch` slots (the
+// slots past zp are filled with zeros).
+static cbct_status line_map(const GeomDev &G, const float *f, int pitch, CUtensorMap *map)
+{
+    const EncodeTiled enc = encode_tiled();
+    if (!enc) return set_error(CBCT_ERR_CUDA, "project: the driver has no cuTensorMapEncodeTiled");
+    const cuuint64_t dims[2] = {(cuuint64_t)G.zp, (cuuint64_t)G.nx * G.ny}, strides[1] = {(cuuint64_t)G.zp * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)pitch, 1}, step[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(f), dims, strides, box, step,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return set_error(CBCT_ERR_CUDA, "project: tensor map of the volume (%d)", (int)r);
+    return CBCT_OK;
+}
+
+cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const float *y, void *out, int mode,
+                           double *partials, float count_thr, cudaStream_t st, int storage, Scalars *sc,
+                           const void *traces, int *npartials, int col_first, int ncols)
+{
     if (project_smem_bytes(G) > PROJECT_SMEM_LIMIT)
         return set_error(CBCT_ERR_UNSUPPORTED, "project: grid too large for the projector's shared memory (nx + ny and nz)");
-    if (sz != 1) return set_error(CBCT_ERR_INVALID_ARG, "project: the volume must be z-contiguous");
-    if (mode == PM_COUNT) storage = ST_F32;
-    int sg = 0;
-    cbct_status r = choose_group(G, threads, mode, storage, &sg);
+    if (mode == PM_COUNT) return launch_project_count(G, partials, count_thr, st);
+    const int threads = proj_threads(G), fill = fill_of(G, zpitch);
+    const int rows = fill == FILL_GATHER ? proj_rows_per_thread(G) : 2;
+    if (ncols == 0) ncols = G.nviews * G.nu;
+    // (views x columns < 2^31 / nv, so the items fit an int)
+    int nitems = ncols * ((G.nv + rows * threads - 1) / (rows * threads));
+    // the packed layout takes the padded one's plan: the same tables, hence the same sums
+    GroupChoice c{};
+    cbct_status r = choose_group(G, threads, mode, storage, fill_of(G, G.zp), &c);
     if (r != CBCT_OK) return r;
     const void *fn = nullptr;
-    r = optin(sg, mode, storage, &fn);
+    r = optin(c.qw, mode, storage, rows, fill, &fn);
     if (r != CBCT_OK) return r;
-    const size_t smem = project_smem(G, sg);
+    if (fill == FILL_PACKED) {
+        int nb = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads + 32, c.smem);
+        if (e != cudaSuccess) return check_cuda(e, "project occupancy");
+        c.grid = (nb > 0 ? nb : 1) * device_sm_count();
+    }
+    alignas(64) CUtensorMap map;
+    memset(&map, 0, sizeof(map));
+    if (fill == FILL_GATHER) {
+        r = line_map(G, f, c.plan.pitch, &map);
+        if (r != CBCT_OK) return r;
+    }
+    const int grid = nitems < c.grid ? nitems : c.grid;
+    if (npartials) *npartials = grid;
     GeomDev g = G;
-    int isx = (int)sx, isy = (int)sy;
-    const int4 *tr = mode == PM_COUNT ? nullptr : reinterpret_cast<const int4 *>(traces);
-    int tcap = trace_cap(G);
-    void *args[] = {&g, &f, &isx, &isy, &y, &out, &partials, &count_thr, &sc, &tr, &tcap};
+    const float *rec = static_cast<const float *>(traces);
+    void *args[] = {&g, &map, &f, &zpitch, &c.plan, &y, &out, &partials, &sc, &rec, &col_first, &ncols, &nitems};
     ProfToken tok = prof_start(CBCT_KERNEL_PROJECT, st);
-    cudaError_t e = cudaLaunchKernel(fn, grid, dim3((unsigned)threads), args, smem, st);
+    cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads + 32), args, c.smem, st);
     prof_stop(tok, st);
     note_launch();
     if (e != cudaSuccess) cudaGetLastError(); // the error is returned, not left pending

@@ -3,40 +3,89 @@
 //
 // GB300 mapping. All rays of one view that hit the same imager column u share their
 // transverse path through the (x, y) voxel columns; the imager row v only tilts them in
-// z. A block owns one (view, column) pair and its threads own the imager rows. The
-// block first computes the shared transverse Siddon trace once, cooperatively, into
-// shared memory (a parallel merge of the x-plane and y-plane crossing lists). Along that
-// trace a ray of row v stays in one z slab for long runs of columns (the cone is narrow),
-// and the block holds more rows than the volume has slabs. So, group by group of
-// columns, the block stages the columns' z-lines (contiguous in the iteration's
-// z-fastest layout) and forms per slab the running sum of voxel value x segment length;
-// a row's line integral over a run of columns in one slab is then the difference of two
-// table entries, and only the columns where it crosses a z plane are split explicitly.
-// Accumulation is FP32; the epilogue can
-// scale by |D - S|, form the CGLS residual and reduce squared norms in FP64 into one
-// partial per block; the output is stored as FP32, BF16 or FP16.
+// z. The path of every (view, column) is a record of the grid's trace table
+// (project_trace.cu). Along it the integral of slab k up to tau,
+//     C_k(tau) = int f(column at tau', slab k) dtau',
+// is piecewise linear, and a ray that leaves slab k for slab k' at tau contributes
+// C_k(tau) - C_k'(tau): a row does work only where it crosses a z plane (about five times
+// per ray at the paper's sizes), and the per-column work is done once per slab instead of
+// once per row. So, group by group of SG columns, a block tabulates C_k at the column
+// boundaries, and every row interpolates it at its crossings.
 //
-// This header holds the kernel template; it is instantiated for each group size in the
-// project_groups_*.cu units (compiled in parallel) and launched from project.cu.
+// A block is one producer warp and up to six consumer warps (whose threads own the imager
+// rows), and works through several (view, column) items. The producer brings each group's
+// z-lines by TMA, one group ahead and across items: the volume is a matrix of nx ny lines,
+// and one gather4 instruction fetches the lines of four columns, so the copies cost no
+// issue slots and no load/store wavefronts and their latency is hidden. The consumers turn
+// the lines into the table in place: each lane takes a quad of slabs (16-byte shared
+// accesses) and nb consecutive columns of the group; the 32 / QW parts of a quad sit in one
+// warp, which turns the parts' sums into offsets with shuffles. Pairs of slabs share one
+// instruction (fma.rn.f32x2; each half rounds like a scalar FMA).
+// Accumulation is FP32; the epilogue can scale by |D - S|, form the CGLS residual and
+// reduce squared norms in FP64 into one partial per block; the output is stored as FP32,
+// BF16 or FP16.
+//
+// This header holds the kernel template; it is instantiated for each QW in the
+// project_q*.cu units (compiled in parallel) and launched from project.cu.
 #pragma once
-#include <cfloat>
-
 #include "project.cuh"
 
 namespace cbct {
 
-// 16-byte asynchronous global -> shared copy (L2 only); both addresses 16-byte aligned
-__device__ __forceinline__ void cp_async16(float *smem_dst, const float *gsrc)
+// Two FP32 operations in one instruction, on pairs held as 64-bit registers; each half is
+// rounded like the scalar operation.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
 {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gsrc) : "memory");
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
-// One-shot bulk (TMA) copy of a block's trace record into shared memory, completed on an
-// mbarrier that one thread initialises, arms, feeds and waits on (the others wait at the
-// block barrier that follows, so no warp spins).
+// Shared-memory accesses by 32-bit address (byte offsets are added to it in one instruction).
+__device__ __forceinline__ ulonglong2 lds_quad(unsigned a)
+{
+    ulonglong2 v;
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts_quad(unsigned a, ulonglong2 v)
+{
+    asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(a), "l"(v.x), "l"(v.y) : "memory");
+}
+__device__ __forceinline__ f32x2 lds_pair(unsigned a)
+{
+    f32x2 v;
+    asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 lds_float2(unsigned a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float lds_float(unsigned a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// Bulk (TMA) copies into shared memory complete on mbarriers; the consumers give a buffer
+// back on another.
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count)
 {
@@ -47,33 +96,35 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, u
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(unsigned long long *bar)
+{
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+// one try: suspends the thread for up to about a millisecond while the phase is incomplete
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned parity)
 {
     unsigned ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
                  : "=r"(ok)
-                 : "r"(smem_u32(bar)), "r"(parity)
+                 : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u)
                  : "memory");
     return ok != 0;
 }
-// global -> shared bulk copy of `bytes` (a multiple of 16) between 16-byte-aligned addresses,
-// marked evict-first in L2: each record is read once per projection, and the volume lines
-// and the stack the projector and the next kernels reuse should stay
-__device__ __forceinline__ void bulk_copy_g2s(void *smem_dst, const void *gsrc, unsigned bytes, unsigned long long *bar)
+// Every wait ends: after PROJ_WAIT_CYCLES (about two seconds), or once another warp of the
+// block has given up, it returns false, and the block then ends with NaN results and bit 1
+// of the iteration's status word instead of a hang.
+constexpr long long PROJ_WAIT_CYCLES = 4000000000ll;
+__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, volatile int *give_up)
 {
-    unsigned long long policy;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(policy));
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n" ::"r"(
-            smem_u32(smem_dst)),
-        "l"(gsrc), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
-        : "memory");
+    bool ok = mbar_try_wait(bar, parity);
+    if (!ok) {
+        const long long t0 = clock64();
+        while (!(ok = mbar_try_wait(bar, parity)) && !*give_up)
+            if (clock64() - t0 > PROJ_WAIT_CYCLES) *give_up = 1;
+    }
+    __syncwarp();
+    return ok;
 }
-// tries of the record wait before a block gives up (each try may suspend the thread for a
-// while; together well over a second): a copy that never lands ends the block with NaN
-// results and bit 1 of the iteration's status word instead of a hang
-constexpr int PROJ_WAIT_TRIES = 1 << 22;
-
 // The transverse ray shared by every row of imager column iu in a view, and the tau
 // interval in which it crosses the volume's (x, y) footprint.
 struct ColumnRay {
@@ -102,10 +153,10 @@ __device__ __forceinline__ ColumnRay column_ray(const GeomDev &G, int view, int 
 // each plane family are increasing in tau, so every crossing's position in the merged order
 // is its own index plus the number of crossings of the other family before it. Writes, for
 // the nseg = nA + nB + 1 segments the ray spends in (x, y) voxel columns, sEnd[j] (the tau at
-// which segment j ends) and sCol[j] (its column's offset ix * sx + iy * sy); sA (nx + 1
+// which segment j ends) and sCol[j] (its column iy * nx + ix); sA (nx + 1
 // floats), sB (ny + 1) and s_cnt (4 per warp) are scratch. Returns (nA, nB, ix_e, iy_e): the
 // x- and y-plane crossings inside the volume and the column entered first.
-__device__ __forceinline__ int4 trace_column(const GeomDev &G, const ColumnRay &ray, int sx, int sy, float *sA,
+__device__ __forceinline__ int4 trace_column(const GeomDev &G, const ColumnRay &ray, float *sA,
                                              float *sB, unsigned *s_cnt, float *sEnd, int *sCol, int tid, int nthr)
 {
     const float dxr = ray.dxr, dyr = ray.dyr, qx = ray.qx, qy = ray.qy, inv_x = ray.inv_x, inv_y = ray.inv_y;
@@ -173,7 +224,7 @@ __device__ __forceinline__ int4 trace_column(const GeomDev &G, const ColumnRay &
         const int r = i + nb;
         const int cx = min(max(ix_e + sxs * (i + 1), 0), G.nx - 1), cy = min(max(iy_e + sys * nb, 0), G.ny - 1);
         sEnd[r] = t;
-        sCol[r + 1] = cx * sx + cy * sy;
+        sCol[r + 1] = cy * G.nx + cx;
     }
     for (int j = tid; j < nB; j += nthr) {
         const float t = LB[j];
@@ -186,342 +237,401 @@ __device__ __forceinline__ int4 trace_column(const GeomDev &G, const ColumnRay &
         const int r = j + na;
         const int cx = min(max(ix_e + sxs * na, 0), G.nx - 1), cy = min(max(iy_e + sys * (j + 1), 0), G.ny - 1);
         sEnd[r] = t;
-        sCol[r + 1] = cx * sx + cy * sy;
+        sCol[r + 1] = cy * G.nx + cx;
     }
     if (tid == 0) {
-        sCol[0] = ix_e * sx + iy_e * sy;
+        sCol[0] = iy_e * G.nx + ix_e;
         sEnd[nseg - 1] = tau_out;
     }
     return make_int4(nA, nB, ix_e, iy_e);
 }
 
 
-// One block per (view, imager column, chunk of rows), volume z-contiguous (sz = 1).
-// Phase 1 (whole block): the transverse Siddon trace of the column's rays — the
-// crossings with the x planes and with the y planes are each increasing in tau, so every
-// crossing's position in the merged order is its own index plus the number of crossings
-// of the other family before it (binary search); this yields the list of (x, y) voxel
-// columns the rays visit and the tau at which each is left. For every segment the block
-// also stores its length and where its column's z-line will sit in shared memory.
-// Phase 2, per group of SG segments: the block stages the group's z-lines and builds
-// the per-slab prefix table T[k][u] over the group's columns; then each thread (two
-// imager rows) adds, for each run of whole columns a row spends in one z slab, the
-// table difference, and splits exactly each column in which the row crosses a z plane.
-template <int MODE, typename TP, int SG>
-__global__ void __launch_bounds__(PROJ_THREADS, CBCT_PROJ_MIN_BLOCKS)
-k_project(GeomDev G, const float *__restrict__ f, int sx, int sy, const float *__restrict__ y,
-          TP *__restrict__ out, double *__restrict__ partials, float count_thr, Scalars *__restrict__ sc,
-          const int4 *__restrict__ traces, int trace_cap)
+// TMA gather of the z-lines of four columns (rows y.x .. y.w of the line matrix) into four
+// consecutive line slots; dst is a 128-byte aligned shared address.
+__device__ __forceinline__ void gather4_g2s(unsigned dst, const CUtensorMap *map, int4 y, unsigned long long *bar)
 {
-    extern __shared__ __align__(16) float smem[];
+    asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes "
+                 "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(dst),
+                 "l"(map), "r"(0), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w), "r"(smem_u32(bar))
+                 : "memory");
+}
+// one line by a bulk copy (bytes a multiple of 16, both addresses 16-byte aligned)
+__device__ __forceinline__ void bulk_g2s(unsigned dst, const float *src, int bytes, unsigned long long *bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+// one value by an asynchronous copy; copies_arrive: this thread's arrival once its copies landed
+__device__ __forceinline__ void copy4_async(unsigned dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_arrive(unsigned long long *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+// generic accesses of this thread to shared memory before, bulk copies into it after
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+// barrier of the n consumer threads that also tells whether any of them passed `v`
+__device__ __forceinline__ bool consumer_or(bool v, int n)
+{
+    unsigned r;
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, 1, %2, q;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(r)
+                 : "r"((unsigned)v), "r"(n)
+                 : "memory");
+    return r != 0;
+}
+
+// tau at which a row (1 / v = inv_v) in slab k leaves it; never if k is outside the volume
+__device__ __forceinline__ float next_crossing(const GeomDev &G, int k, float inv_v)
+{
+    return (unsigned)k < (unsigned)G.nz ? tau_zplane(plane_at(k + (inv_v > 0.0f), G.dz, G.z0), inv_v, G.tc) : P_INF;
+}
+
+// The table build of one lane's part of NB columns (an even number): lines at `at`, pitch lp4
+// bytes, the lengths of the columns in pairs at `al`; p becomes the part's sums.
+template <int NB>
+__device__ __forceinline__ void build_part(unsigned at, unsigned lp4, unsigned al, bool store, ulonglong2 &p)
+{
+#pragma unroll
+    for (int i0 = 0; i0 < NB; i0 += BUILD_BATCH) {
+        ulonglong2 v[BUILD_BATCH], l4[BUILD_BATCH / 2]; // lines; the lengths of two columns each
+#pragma unroll
+        for (int i = 0; i < BUILD_BATCH; ++i)
+            if (i0 + i < NB) v[i] = lds_quad(at + i * lp4);
+#pragma unroll
+        for (int i = 0; i < BUILD_BATCH / 2; ++i)
+            if (i0 + 2 * i < NB) l4[i] = lds_quad(al + 8 * i0 + 16 * i);
+#pragma unroll
+        for (int i = 0; i < BUILD_BATCH; ++i)
+            if (i0 + i < NB) {
+                const f32x2 l2 = i & 1 ? l4[i / 2].y : l4[i / 2].x;
+                p.x = fma2(v[i].x, l2, p.x);
+                p.y = fma2(v[i].y, l2, p.y);
+                if (store) sts_quad(at + i * lp4, p);
+            }
+        at += BUILD_BATCH * lp4;
+    }
+}
+
+// Items (view, imager column, chunk of rows) first_item + blockIdx.x, + gridDim.x, ...: item i is
+// chunk i / ncols of column col_first + i % ncols, whose record is rec[i % ncols].
+// Per group of sg segments of an item's trace the lines become the table in place,
+// T[c][k] = sum of f(column, slab k) * length over the columns of c's part up to and
+// including c, with the sums of the parts before in O[part][k] (O[PARTS] is the group's
+// total); then each consumer thread (R imager rows) adds, for every z crossing of its rows
+// inside the group, the interpolated table value of the slab left minus that of the slab
+// entered, and at the group's end the total of the slab the row is in (every group starts
+// from zero). One barrier of the consumers per group; two line buffers.
+// QW: quads of slabs per warp in the table build (PARTS = 32 / QW parts of nb columns each).
+// FILL_GATHER: lines by gather4; FILL_BULK: one bulk copy per line; FILL_PACKED: 4-byte copies
+// by the producer's lanes.
+template <int MODE, typename TP, int QW, int R, int FILL>
+__global__ void __launch_bounds__(PROJ_THREADS + 32, CBCT_PROJ_MIN_BLOCKS)
+k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__restrict__ f, int zpitch, ProjPlan pl,
+          const float *__restrict__ y, TP *__restrict__ out, double *__restrict__ partials, Scalars *__restrict__ sc,
+          const float *__restrict__ rec, int col_first, int ncols, int nitems)
+{
+    constexpr int PARTS = 32 / QW;
+    extern __shared__ __align__(128) float smem[];
     __shared__ double s_warp[PROJ_THREADS / 32];
-    __shared__ __align__(8) unsigned long long s_bar; // completion of the trace record's copy
-    const int cap = ((G.nx + G.ny + 2 + SG - 1) / SG) * SG;
-    float *sEnd = smem;                                    // tau at which segment j ends
-    int *sCol = reinterpret_cast<int *>(sEnd + cap);      // voxel-column offset of segment j
-    float2 *sSeg = reinterpret_cast<float2 *>(sCol + cap); // (line offset bits, length) of segment j
-    const int pitch = ((G.nz + 6 + 3) / 4) * 4;            // floats per staged line
-    const int quads = pitch / 4;                           // 16-byte pieces per line slot
-    float *sLine = reinterpret_cast<float *>(sSeg + cap);  // the staged z-lines of one group
-    float *sA = sLine;                                     // phase 1: x-plane crossings, in ray order
-    float *sB = sA + (G.nx + 1);                           // phase 1: y-plane crossings
-    const int lregion = max(SG * pitch, ((G.nx + G.ny + 2 + 3) / 4) * 4);
-    constexpr int TPITCH = SG + 1;                         // odd: the build's threads (slabs) hit distinct banks
-    float *sTab = sLine + lregion;                         // [nz][SG + 1] per-slab prefix table
-    float *sBase = sTab + G.nz * TPITCH;                   // [2][nz] running per-slab totals
-
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int view = blockIdx.x / G.nu;
-    const int iu = blockIdx.x - view * G.nu;
-
-    // ---- transverse ray, shared by every row ----
-    const ColumnRay ray = column_ray(G, view, iu);
-    const float dxr = ray.dxr, dyr = ray.dyr, qx = ray.qx, qy = ray.qy;
-    const float tau_in = ray.tau_in, tau_out = ray.tau_out;
-    const bool hit = ray.hit;
-    const int sxs = ray.sxs, sys = ray.sys;
-
-    // ---- phase 1: crossings of each plane family, then their merged order ----
-    int4 tr;
-    bool timed_out = false;
-    if (traces && hit) {
-        // phase 1 from the grid's trace table: the record's segment lists by one bulk copy
-        const int4 *rec = traces + (size_t)blockIdx.x * (1 + trace_cap / 2);
-        tr = __ldg(rec);
-        int bad = 0;
-        if (tid == 0) {
-            const unsigned bytes = 4u * (unsigned)((tr.x + tr.y + 1 + 3) & ~3);
-            mbar_init(&s_bar, 1u);
-            mbar_arrive_expect_tx(&s_bar, 2u * bytes);
-            bulk_copy_g2s(sEnd, rec + 1, bytes, &s_bar);
-            bulk_copy_g2s(sCol, reinterpret_cast<const float *>(rec + 1) + trace_cap, bytes, &s_bar);
-            bool landed = false;
-            for (int it = 0; it < PROJ_WAIT_TRIES && !(landed = mbar_try_wait(&s_bar, 0u)); ++it) {
-            }
-            bad = !landed;
+    __shared__ __align__(16) float s_hdr[2][TRACE_HDR / 2]; // headers of the items in work
+    __shared__ float s_gend[2];                              // tau at which a group ends
+    __shared__ __align__(8) unsigned long long s_full[2], s_empty[2];
+    __shared__ int s_give_up;
+    const int sg = pl.sg, lp = pl.pitch, bsh = pl.nbuf - 1; // group s uses buffer s & bsh, its use number s >> bsh
+    // a line of room (the line before a buffer's first may be read, not used), then [nbuf][sg][lp]
+    // lines, then table
+    float *sBuf = smem + (lp + 31) / 32 * 32;
+    float2 *sLen = reinterpret_cast<float2 *>(sBuf + pl.nbuf * sg * lp); // [nbuf][sg] (length, length) of a column's segment
+    float2 *sSeg = sLen + pl.nbuf * sg;                                  // [nbuf][sg] (tau at its start, 1 / length)
+    float *sOff = reinterpret_cast<float *>(sSeg + pl.nbuf * sg);        // [nbuf][PARTS + 1][zp] part offsets
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nthr = blockDim.x - 32, nwarps = nthr >> 5; // consumers; the last warp is the producer
+    const int tcap = trace_cap(G), rwords = trace_words(G);
+    if (tid == 0) {
+        s_give_up = 0;
+        for (int b = 0; b < 2; ++b) {
+            // the copies' transactions and the producer's own stores (and its lanes' 4-byte copies)
+            mbar_init(&s_full[b], FILL == FILL_PACKED ? 34u : 2u);
+            mbar_init(&s_empty[b], (unsigned)nwarps);
         }
-        timed_out = __syncthreads_or(bad) != 0;
-        if (timed_out && sc && tid == 0) atomicOr(&sc->flags, 2u);
-    } else {
-        // per-warp sums of phase 1 are parked in the segment records (written after it)
-        tr = trace_column(G, ray, sx, sy, sA, sB, reinterpret_cast<unsigned *>(sSeg), sEnd, sCol, tid, nthr);
-    }
-    const int nA = tr.x, nB = tr.y, ix_e = tr.z, iy_e = tr.w, nseg = nA + nB + 1;
-    const int col0 = ix_e * sx + iy_e * sy;
-    const float inv_dx = 1.0f / G.dx, inv_dy = 1.0f / G.dy;
-    for (int q = nseg + tid; q < cap; q += nthr) { // zero-length padding up to whole groups
-        sEnd[q] = tau_out;
-        sCol[q] = col0;
-    }
-    __syncthreads();
-    for (int q = tid; q < cap; q += nthr) {
-        const float st = q ? sEnd[q - 1] : tau_in;
-        // where the column's first voxel lands in its staged line
-        const int loff = (q % SG) * pitch + (sCol[q] & 3);
-        sSeg[q] = make_float2(__int_as_float(loff), sEnd[q] - st);
     }
     __syncthreads();
 
-    // ---- phase 2: per-row z state (two rows per thread: iv[0] and iv[1] = iv[0] + nthr) ----
-    constexpr int R = 2;
-    int iv[R], skz[R], kz[R];
-    float inv_v[R], tzn[R], L[R], acc[R];
-    bool ok[R], active[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        iv[r] = blockIdx.y * (R * nthr) + r * nthr + tid;
-        ok[r] = iv[r] < G.nv;
-        const float v = imager_v(G, iv[r]);
-        inv_v[r] = v != 0.0f ? __frcp_rn(v) : 1e30f;
-        skz[r] = v >= 0.0f ? 1 : -1;
-        kz[r] = (int)floorf((v * (G.tc + tau_in) - G.z0) / G.dz);
-        active[r] = hit && !timed_out && ok[r] && kz[r] >= 0 && kz[r] < G.nz;
-        tzn[r] = active[r] ? tau_zplane(plane_at(kz[r] + (skz[r] > 0), G.dz, G.z0), inv_v[r], G.tc) : P_INF;
-        if (active[r] && tzn[r] <= tau_in) { // the entry point already lies past that plane
-            kz[r] += skz[r];
-            active[r] = (unsigned)kz[r] < (unsigned)G.nz;
-            tzn[r] = active[r] ? tau_zplane(plane_at(kz[r] + (skz[r] > 0), G.dz, G.z0), inv_v[r], G.tc) : P_INF;
-        }
-        L[r] = ray_length(dxr, dyr, v);
-        acc[r] = 0.0f;
-    }
-
-    int cnt = 0;
-    if (hit && MODE == PM_COUNT) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float thr_tau = count_thr / L[r];
-            float s0 = tau_in;
-            for (int j = 0; j < nseg; ++j) {
-                const float e = sEnd[j];
-                float sl = s0;
-                while (tzn[r] < e) {
-                    cnt += (tzn[r] - sl) > thr_tau;
-                    sl = tzn[r];
-                    kz[r] += skz[r];
-                    active[r] = (unsigned)kz[r] < (unsigned)G.nz;
-                    tzn[r] = active[r] ? tau_zplane(plane_at(kz[r] + (skz[r] > 0), G.dz, G.z0), inv_v[r], G.tc) : P_INF;
-                }
-                if (active[r]) cnt += (e - sl) > thr_tau;
-                s0 = e;
+    if (warp == nwarps) {
+        // ---- producer: one group ahead of the consumers, through all items ----
+        int item = blockIdx.x, g = 0, nitem = 0, nseg = 0;
+        const float *r = nullptr;
+        int4 col = make_int4(0, 0, 0, 0);          // four columns of the next group ...
+        float4 end = make_float4(0.f, 0.f, 0.f, 0.f); // ... the tau at which they end ...
+        float start = 0.0f;                        // ... and where the first begins
+        float hdr = 0.0f;                          // lane's word of the item's header
+        auto next_columns = [&]() { // (past the trace's end: unused values of the record)
+            if (4 * lane < min(sg, tcap - g * sg)) {
+                const float *e = r + TRACE_HDR + g * sg + 4 * lane;
+                end = __ldg(reinterpret_cast<const float4 *>(e));
+                start = __ldg(e - 1);
+                col = __ldg(reinterpret_cast<const int4 *>(e + tcap));
             }
-        }
-    } else if (hit && !timed_out) {
-        // Per group of SG segments: stage the z-lines of its columns (16-byte cp.async into
-        // one buffer: a second buffer to copy the next group ahead would cost a resident
-        // block, which hides more latency than the early copy), build once for the block the
-        // per-slab prefix table over the group's columns,
-        //     T[k][u] = sum_{u' < u} f(column u', slab k) * length(u'),   u = 0..SG,
-        // and let every row add T[k][u1] - T[k][u0] for each run of whole columns it
-        // spends in slab k. Only the columns in which a row crosses a z plane are split,
-        // exactly, at the crossing. A block has far more rows than slabs, so the table
-        // does the per-column work once per slab instead of once per row.
-        const int nchunk = (nseg + SG - 1) / SG;
-        // 16-byte pieces of a group's lines: slot c = (line u, piece i), c = u * quads + i;
-        // thread tid takes c = tid, tid + nthr, ... (the same slots for every group)
-        const int u_0 = tid / quads, i_0 = tid - u_0 * quads;
-        const int du = nthr / quads, di = nthr - du * quads;
-        auto fill = [&](int chunk) {
-            float *dst = sLine;
-            const int *col = sCol + chunk * SG;
-            for (int u = u_0, i = i_0; u < SG;) {
-                const int c0 = col[u];
-                const int first = c0 & ~3, last = (c0 + G.nz + 3) & ~3; // 16-byte rounded line
-                if (first + 4 * i < last) cp_async16(dst + u * pitch + 4 * i, f + first + 4 * i);
-                u += du;
-                i += di;
-                if (i >= quads) {
-                    i -= quads;
-                    ++u;
-                }
-            }
-            cp_async_commit();
         };
-        const bool split = nthr >= 2 * G.nz;
-        // T[k][u]: the table entry, plus the first half's total for a second-half entry
-        auto tab = [&](int k, int u) {
-            const float *trow = sTab + k * TPITCH;
-            return split && u > SG / 2 ? trow[u] + trow[SG / 2] : trow[u];
+        auto next_item = [&]() {
+            r = rec + (size_t)(item % ncols) * rwords;
+            if (lane < TRACE_HDR / 2) hdr = __ldg(r + lane);
         };
-        float E[R] = {0.0f, 0.0f}; // running total where each row's current run starts
-        for (int k = tid; k < G.nz; k += nthr) sBase[k] = 0.0f; // published by the first barrier
-        float g0 = tau_in;
-        for (int ch = 0; ch < nchunk; ++ch) {
-            const int j = ch * SG;
-            if (ch) __syncthreads(); // every thread is done with the previous group's lines
-            fill(ch);
-            cp_async_wait<0>();
-            __syncthreads();
-            const float *lines = sLine;
-            // The group's prefix table. With threads to spare each slab's running sum is
-            // split into two chains of SG / 2 columns computed side by side; the second
-            // half's entries then hold sums from column SG / 2 on, and tab() adds the
-            // first half's total.
-            if (split) {
-                for (int task = tid; task < 2 * G.nz; task += nthr) {
-                    const int k = task >> 1, h = (task & 1) * (SG / 2);
-                    float *trow = sTab + k * TPITCH + h;
-                    float sum = 0.0f;
-                    if (!h) trow[0] = 0.0f;
-#pragma unroll 8
-                    for (int u = 0; u < SG / 2; ++u) {
-                        const float2 seg = sSeg[j + h + u]; // (line offset, length)
-                        sum = fmaf(lines[__float_as_int(seg.x) + k], seg.y, sum);
-                        trow[u + 1] = sum;
-                    }
+        next_item();
+        next_columns();
+        nseg = __shfl_sync(0xffffffffu, __float_as_int(hdr), 0);
+        for (int s = 0;; ++s) {
+            const int b = s & bsh, n = min(sg, nseg - g * sg), quads = (n + 3) / 4;
+            if (s > bsh && !mbar_wait(&s_empty[b], ((s >> bsh) - 1) & 1, &s_give_up)) break;
+            const unsigned dst = smem_u32(sBuf) + 4u * (unsigned)(b * sg * lp);
+            if (lane == 0)
+                mbar_arrive_expect_tx(&s_full[b], FILL == FILL_GATHER ? 16u * (unsigned)(quads * lp)
+                                                  : FILL == FILL_BULK ? 16u * (unsigned)(quads * G.zp) : 0u);
+            if (g == 0 && lane < TRACE_HDR / 2) s_hdr[nitem & 1][lane] = hdr;
+            __syncwarp();
+            const unsigned to = dst + (unsigned)lane * 16u * (unsigned)lp; // this lane's four line slots
+            if (FILL == FILL_GATHER) {
+                if (lane < quads) gather4_g2s(to, &lines, col, &s_full[b]);
+            } else if (FILL == FILL_BULK) {
+                if (lane < quads) {
+                    bulk_g2s(to, f + (size_t)col.x * zpitch, 4 * G.zp, &s_full[b]);
+                    bulk_g2s(to + 4 * lp, f + (size_t)col.y * zpitch, 4 * G.zp, &s_full[b]);
+                    bulk_g2s(to + 8 * lp, f + (size_t)col.z * zpitch, 4 * G.zp, &s_full[b]);
+                    bulk_g2s(to + 12 * lp, f + (size_t)col.w * zpitch, 4 * G.zp, &s_full[b]);
                 }
             } else {
-                for (int k = tid; k < G.nz; k += nthr) {
-                    float *trow = sTab + k * TPITCH;
-                    float sum = 0.0f;
-                    trow[0] = 0.0f;
-#pragma unroll 8
-                    for (int u = 0; u < SG; ++u) {
-                        const float2 seg = sSeg[j + u];
-                        sum = fmaf(lines[__float_as_int(seg.x) + k], seg.y, sum);
-                        trow[u + 1] = sum;
-                    }
+                for (int u = 0; u < n; ++u) {
+                    const int c4 = u & 3, cu = c4 == 0 ? col.x : c4 == 1 ? col.y : c4 == 2 ? col.z : col.w;
+                    const float *line = f + (size_t)__shfl_sync(0xffffffffu, cu, u >> 2) * zpitch;
+                    for (int k = lane; k < G.nz; k += 32) copy4_async(dst + 4 * (u * lp + k), line + k);
                 }
+                copies_arrive(&s_full[b]);
             }
-            __syncthreads();
-            const float gend = sEnd[j + SG - 1];
-            // running per-slab totals: C[k][j + u] = base[k] + T[k][u] is the sum over all
-            // columns of the trace before column j + u; one thread per slab carries it on
-            const float *bcur = sBase + (ch & 1) * G.nz;
-            float *bnext = sBase + ((ch + 1) & 1) * G.nz;
-            for (int k = tid; k < G.nz; k += nthr) bnext[k] = bcur[k] + tab(k, SG);
-            // A row does nothing in a group it crosses no z plane in. At a crossing it adds
-            // its run in the slab it leaves (a difference of running totals, plus the part
-            // of the crossing column before the plane) and books the rest of that column to
-            // the slab it enters; E remembers the running total where that slab's run of
-            // whole columns starts.
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                float a = acc[r];
-                int cpend = -1; // column of this row's previous crossing in this group
-                while (tzn[r] < gend) { // a z crossing inside this group (the row is active)
-                    const float t = tzn[r];
-                    // The segment holding the crossing: the x and y planes the ray has passed
-                    // at t, from its transverse position (no search). At a near tie this may
-                    // name the neighbouring segment, which only moves a rounding-sized piece
-                    // of length between two adjacent columns; it is kept monotone.
-                    int na = (int)floorf((fmaf(t, dxr, qx) - G.x0) * inv_dx) - ix_e;
-                    int nb = (int)floorf((fmaf(t, dyr, qy) - G.y0) * inv_dy) - iy_e;
-                    na = min(max(sxs > 0 ? na : -na, 0), nA);
-                    nb = min(max(sys > 0 ? nb : -nb, 0), nB);
-                    const int c = min(max(na + nb - j, max(cpend, 0)), SG - 1);
-                    const int lo = __float_as_int(sSeg[j + c].x);
-                    const float en = sEnd[j + c];
-                    const float fcur = lines[lo + kz[r]];
-                    if (c == cpend) // entered this slab in this same column: trim the booked rest
-                        a = fmaf(-fcur, en - t, a);
-                    else
-                        a += (bcur[kz[r]] + tab(kz[r], c)) - E[r] +
-                             fcur * fmaxf(t - (c ? sEnd[j + c - 1] : g0), 0.0f);
-                    cpend = c;
-                    kz[r] += skz[r];
-                    active[r] = (unsigned)kz[r] < (unsigned)G.nz;
-                    if (active[r]) {
-                        a = fmaf(lines[lo + kz[r]], en - t, a);
-                        E[r] = bcur[kz[r]] + tab(kz[r], c + 1);
-                    }
-                    tzn[r] = active[r] ? tau_zplane(plane_at(kz[r] + (skz[r] > 0), G.dz, G.z0), inv_v[r], G.tc) : P_INF;
-                }
-                acc[r] = a;
+            if (lane == quads - 1) s_gend[b] = end.w; // (a record's tail repeats its last segment)
+            if (lane < quads) {
+                const float l0 = end.x - start, l1 = end.y - end.x, l2 = end.z - end.y, l3 = end.w - end.z;
+                float4 *len = reinterpret_cast<float4 *>(sLen + b * sg + 4 * lane);
+                len[0] = make_float4(l0, l0, l1, l1);
+                len[1] = make_float4(l2, l2, l3, l3);
+                float4 *seg = reinterpret_cast<float4 *>(sSeg + b * sg + 4 * lane);
+                seg[0] = make_float4(start, __fdividef(1.0f, l0), end.x, __fdividef(1.0f, l1));
+                seg[1] = make_float4(end.y, __fdividef(1.0f, l2), end.z, __fdividef(1.0f, l3));
             }
-            g0 = gend;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_full[b]);
+            if (++g * sg >= nseg) {
+                g = 0;
+                ++nitem;
+                item += gridDim.x;
+                if (item >= nitems) break;
+                next_item();
+            }
+            next_columns();
+            if (g == 0) nseg = __shfl_sync(0xffffffffu, __float_as_int(hdr), 0);
         }
-        __syncthreads();
-        // the run each still-active row ends in: up to the end of the trace
-        const float *bend = sBase + (nchunk & 1) * G.nz;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (active[r]) acc[r] += bend[kz[r]] - E[r];
+        return;
     }
 
-    // ---- epilogue ----
-    if (timed_out) { // the trace record never arrived: NaN rows, reported through sc
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = __int_as_float(0x7fc00000);
-    }
-    double red = 0.0;
+    // ---- consumers ----
+    const int h = lane / QW, qs = lane - h * QW; // this lane's part and quad of a warp's QW quads
+    const int nq = G.zp >> 2;
+    const unsigned a_buf = smem_u32(sBuf), a_len = smem_u32(sLen), a_seg = smem_u32(sSeg), a_off = smem_u32(sOff);
+    const unsigned lp4 = 4 * lp, zp4 = 4 * G.zp, b_buf = sg * lp4, b_seg = 8 * sg, b_off = (PARTS + 1) * zp4;
+    const float inv_dz = 1.0f / G.dz;
     const float kappa = (MODE == PM_Q_SCALED) ? (float)sc->kappa : 1.0f;
     constexpr bool PRESCALE = sizeof(TP) == 4;
+    double red = 0.0;
+    bool lost = false; // a wait of the block ran out: NaN rows from here on
+    int s = 0, nitem = 0; // groups and items so far
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++nitem) {
+        const int chunk = item / ncols;
+        int kz[R];
+        float inv_v[R], tzn[R], acc[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (!ok[r]) continue;
-        const size_t idx = ((size_t)view * G.nv + iv[r]) * G.nu + iu;
-        const float q = acc[r] * L[r];
-        // FP32 storage keeps |D - S| folded into r and q (the adjoint then needs no
-        // per-sample rescale); 16-bit storage keeps the bare values
-        const float s = PRESCALE ? L[r] : 1.0f;
-        if (MODE == PM_PLAIN) {
-            store_from_float(out + idx, q);
-        } else if (MODE == PM_Q_SCALED) {
-            store_from_float(out + idx, q * s * kappa);
-            red += (double)q * (double)q;
-        } else if (MODE == PM_RESID) {
-            const float rr = __ldg(y + idx) - q;
-            store_from_float(out + idx, rr * s);
-            red += (double)rr * (double)rr;
+        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+        int nseg = 0;
+        float mx = 0.f, my = 0.f, cx = 0.f, cy = 0.f, dxy2 = 0.f;
+        for (int g = 0; !lost && (g == 0 || g * sg < nseg); ++g, ++s) {
+            const int j0 = g * sg, b = s & bsh;
+            lost = !mbar_wait(&s_full[b], (s >> bsh) & 1, &s_give_up);
+            if (g == 0) {
+                // the item's trace (see k_trace_table) and the rows' z state
+                const float4 a = *reinterpret_cast<const float4 *>(s_hdr[nitem & 1]);
+                const float4 d = *reinterpret_cast<const float4 *>(s_hdr[nitem & 1] + 4);
+                nseg = __float_as_int(a.x);
+                const float tau_in = a.y;
+                dxy2 = a.z;
+                mx = d.x;
+                my = d.y;
+                cx = d.z;
+                cy = d.w;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int iv = chunk * (R * nthr) + r * nthr + tid;
+                    const float v = imager_v(G, iv);
+                    inv_v[r] = v != 0.0f ? __frcp_rn(v) : 1e30f;
+                    kz[r] = (int)floorf((v * (G.tc + tau_in) - G.z0) * inv_dz);
+                    if (nseg == 0 || iv >= G.nv) kz[r] = -1;
+                    tzn[r] = next_crossing(G, kz[r], inv_v[r]);
+                    if (tzn[r] <= tau_in) { // the entry point already lies past that plane
+                        kz[r] += inv_v[r] > 0.0f ? 1 : -1;
+                        tzn[r] = next_crossing(G, kz[r], inv_v[r]);
+                    }
+                }
+            }
+            const int clast = min(sg, nseg - j0) - 1; // the group's last column
+            const unsigned aT = a_buf + b * b_buf, aO = a_off + b * b_off, aLen = a_len + b * b_seg, aSeg = a_seg + b * b_seg;
+            const int nb = pl.nb, inv_nb = pl.inv_nb;
+            for (int qg = warp; qg * QW < nq && !lost; qg += nwarps) {
+                const int q = min(qg * QW + qs, nq - 1);
+                const bool mine = qg * QW + qs < nq;
+                unsigned at = aT + h * nb * lp4 + 16 * q, al = aLen + 8 * h * nb;
+                ulonglong2 p = make_ulonglong2(0ull, 0ull); // running sums of the quad (all bits 0: 0.0f)
+                if (clast + 1 == 80 && nb == 80 / PARTS) {
+                    build_part<80 / PARTS>(at, lp4, al, mine, p);
+                } else if (clast + 1 == 112 && nb == 112 / PARTS) {
+                    build_part<112 / PARTS>(at, lp4, al, mine, p);
+                } else {
+                    const int n = min(nb, clast + 1 - h * nb); // columns of this lane's part
+                    for (int i = 0; i < n; ++i, at += lp4, al += 8) {
+                        const ulonglong2 v = lds_quad(at);
+                        const f32x2 l2 = lds_pair(al);
+                        p.x = fma2(v.x, l2, p.x);
+                        p.y = fma2(v.y, l2, p.y);
+                        if (mine) sts_quad(at, p);
+                    }
+                }
+                // sums of the parts before this one: shift by a part, then scan
+                ulonglong2 x;
+                x.x = __shfl_up_sync(0xffffffffu, p.x, QW);
+                x.y = __shfl_up_sync(0xffffffffu, p.y, QW);
+                if (h == 0) x = make_ulonglong2(0ull, 0ull);
+#pragma unroll
+                for (int d = QW; d < 32; d *= 2) {
+                    const f32x2 tx = __shfl_up_sync(0xffffffffu, x.x, d), ty = __shfl_up_sync(0xffffffffu, x.y, d);
+                    if (lane >= d) {
+                        x.x = add2(x.x, tx);
+                        x.y = add2(x.y, ty);
+                    }
+                }
+                const unsigned ao = aO + h * zp4 + 16 * q;
+                if (mine) sts_quad(ao, x);
+                if (mine && h == PARTS - 1) sts_quad(ao + zp4, make_ulonglong2(add2(x.x, p.x), add2(x.y, p.y))); // the group's total
+            }
+            lost = consumer_or(lost, nthr); // the table is built
+            if (lost) break;
+            const float gend = s_gend[b];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if ((unsigned)kz[r] >= (unsigned)G.nz) continue; // not in the volume, or out of it
+                const int dir = inv_v[r] > 0.0f ? 1 : -1;
+                float a = acc[r];
+                // The segment that holds a crossing: the x and y planes the ray has passed there,
+                // from its transverse position (no search). At a near tie this may name the
+                // neighbouring segment, which only moves a rounding-sized piece of length between
+                // two adjacent columns.
+                while (tzn[r] < gend) { // a z crossing inside this group
+                    const float t = tzn[r];
+                    const int c = min(max(floor_small(fmaf(t, mx, cx)) + floor_small(fmaf(t, my, cy)) - j0, 0), clast);
+                    const float2 sl = lds_float2(aSeg + 8 * c);
+                    const float w = __saturatef((t - sl.x) * sl.y); // (a 0 x inf of an empty segment saturates to 0)
+                    const int part = (c * inv_nb) >> 16;
+                    const bool first = c == part * nb; // of its part: the sums before it are zero
+                    const unsigned at = aT + c * lp4 + 4 * kz[r], ao = aO + part * zp4 + 4 * kz[r]; // slab left
+                    kz[r] += dir;
+                    const bool in = (unsigned)kz[r] < (unsigned)G.nz;
+                    const unsigned st = in ? 4 * dir : 0; // to the slab entered
+                    float d0 = lds_float(at - lp4), d1 = lds_float(at), o = lds_float(ao);
+                    const float e0 = lds_float(at - lp4 + st), e1 = lds_float(at + st), eo = lds_float(ao + st);
+                    d0 -= in ? e0 : 0.0f;
+                    d1 -= in ? e1 : 0.0f;
+                    o -= in ? eo : 0.0f;
+                    if (first) d0 = 0.0f;
+                    a += fmaf(w, d1 - d0, d0) + o;
+                    tzn[r] = next_crossing(G, kz[r], inv_v[r]);
+                }
+                if ((unsigned)kz[r] < (unsigned)G.nz) a += lds_float(aO + PARTS * zp4 + 4 * kz[r]);
+                acc[r] = a;
+            }
+            // this warp is done with the buffer
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_empty[b]);
+        }
+
+        // ---- epilogue of the item ----
+        const int column = col_first + item - chunk * ncols, view = column / G.nu, iu = column - view * G.nu;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int iv = chunk * (R * nthr) + r * nthr + tid;
+            if (iv >= G.nv) continue;
+            const size_t idx = ((size_t)view * G.nv + iv) * G.nu + iu;
+            const float v = imager_v(G, iv), len = sqrtf(fmaf(v, v, dxy2));
+            // rows whose lines never arrived are NaN (reported through sc)
+            const float q = lost ? __int_as_float(0x7fc00000) : acc[r] * len;
+            // FP32 storage keeps |D - S| folded into r and q (the adjoint then needs no
+            // per-sample rescale); 16-bit storage keeps the bare values
+            const float scl = PRESCALE ? len : 1.0f;
+            if (MODE == PM_PLAIN) {
+                store_from_float(out + idx, q);
+            } else if (MODE == PM_Q_SCALED) {
+                store_from_float(out + idx, q * scl * kappa);
+                red += (double)q * (double)q;
+            } else if (MODE == PM_RESID) {
+                const float rr = __ldg(y + idx) - q;
+                store_from_float(out + idx, rr * scl);
+                red += (double)rr * (double)rr;
+            }
         }
     }
-    if (MODE == PM_COUNT) red = (double)cnt;
+    if (lost) { // once more with a limit for the two groups that may still be in flight
+        if (tid == 0 && sc) atomicOr(&sc->flags, 2u);
+        int waiting = 0;
+        mbar_wait(&s_full[s & bsh], (s >> bsh) & 1, &waiting);
+        if (bsh) mbar_wait(&s_full[(s + 1) & 1], ((s + 1) >> 1) & 1, &waiting);
+    }
     if (MODE != PM_PLAIN) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) red += __shfl_down_sync(0xffffffffu, red, o);
-        if ((tid & 31) == 0) s_warp[tid >> 5] = red;
-        __syncthreads();
+        if (lane == 0) s_warp[warp] = red;
+        consumer_or(false, nthr);
         if (tid == 0) {
             double t = 0.0;
-            for (int w = 0; w < (nthr + 31) / 32; ++w) t += s_warp[w];
-            partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+            for (int w = 0; w < nwarps; ++w) t += s_warp[w];
+            partials[blockIdx.x] = t;
         }
     }
 }
 
-template <int MODE, typename TP, int SG> static const void *kernel_ptr()
+template <int MODE, typename TP, int QW> static const void *kernel_ptr(int rows, int fill)
 {
-    return reinterpret_cast<const void *>(&k_project<MODE, TP, SG>);
+    if (fill == FILL_GATHER)
+        return rows == 2 ? reinterpret_cast<const void *>(&k_project<MODE, TP, QW, 2, FILL_GATHER>)
+                         : reinterpret_cast<const void *>(&k_project<MODE, TP, QW, 1, FILL_GATHER>);
+    if (fill == FILL_BULK) return reinterpret_cast<const void *>(&k_project<MODE, TP, QW, 2, FILL_BULK>);
+    if constexpr (MODE == PM_PLAIN && sizeof(TP) == 4)
+        return reinterpret_cast<const void *>(&k_project<MODE, TP, QW, 2, FILL_PACKED>);
+    return nullptr;
 }
 
-template <int SG> const void *project_kernel(int mode, int storage)
+template <int QW> const void *project_kernel(int mode, int storage, int rows, int fill)
 {
-    if (mode == PM_COUNT) {
-        if constexpr (SG == PROJECT_GROUP_SIZES[0]) return kernel_ptr<PM_COUNT, float, SG>();
-        else return nullptr;
-    }
     const int s = storage == ST_BF16 ? 1 : storage == ST_F16 ? 2 : 0;
     switch (mode * 3 + s) {
-    case PM_PLAIN * 3 + 0: return kernel_ptr<PM_PLAIN, float, SG>();
-    case PM_PLAIN * 3 + 1: return kernel_ptr<PM_PLAIN, __nv_bfloat16, SG>();
-    case PM_PLAIN * 3 + 2: return kernel_ptr<PM_PLAIN, __half, SG>();
-    case PM_Q_SCALED * 3 + 0: return kernel_ptr<PM_Q_SCALED, float, SG>();
-    case PM_Q_SCALED * 3 + 1: return kernel_ptr<PM_Q_SCALED, __nv_bfloat16, SG>();
-    case PM_Q_SCALED * 3 + 2: return kernel_ptr<PM_Q_SCALED, __half, SG>();
-    case PM_RESID * 3 + 0: return kernel_ptr<PM_RESID, float, SG>();
-    case PM_RESID * 3 + 1: return kernel_ptr<PM_RESID, __nv_bfloat16, SG>();
-    case PM_RESID * 3 + 2: return kernel_ptr<PM_RESID, __half, SG>();
+    case PM_PLAIN * 3 + 0: return kernel_ptr<PM_PLAIN, float, QW>(rows, fill);
+    case PM_PLAIN * 3 + 1: return kernel_ptr<PM_PLAIN, __nv_bfloat16, QW>(rows, fill);
+    case PM_PLAIN * 3 + 2: return kernel_ptr<PM_PLAIN, __half, QW>(rows, fill);
+    case PM_Q_SCALED * 3 + 0: return kernel_ptr<PM_Q_SCALED, float, QW>(rows, fill);
+    case PM_Q_SCALED * 3 + 1: return kernel_ptr<PM_Q_SCALED, __nv_bfloat16, QW>(rows, fill);
+    case PM_Q_SCALED * 3 + 2: return kernel_ptr<PM_Q_SCALED, __half, QW>(rows, fill);
+    case PM_RESID * 3 + 0: return kernel_ptr<PM_RESID, float, QW>(rows, fill);
+    case PM_RESID * 3 + 1: return kernel_ptr<PM_RESID, __nv_bfloat16, QW>(rows, fill);
+    case PM_RESID * 3 + 2: return kernel_ptr<PM_RESID, __half, QW>(rows, fill);
     default: return nullptr;
     }
 }

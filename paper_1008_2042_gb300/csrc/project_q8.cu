@@ -1,0 +1,8 @@
+// Instantiations of the forward projector whose table build gives a warp eight quads of slabs.
+#include "project_kernel.cuh"
+
+namespace cbct {
+
+template const void *project_kernel<8>(int, int, int, int);
+
+} // namespace cbct

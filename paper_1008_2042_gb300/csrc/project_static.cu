@@ -16,6 +16,10 @@ namespace cbct {
 // may read past a volume's end. Every GPU that loads the library holds this array (16 MiB)
 // until the process exits.
 static __device__ __align__(256) float g_static_volume[CBCT_PROJECT_STATIC_MAX_VOXELS + PROJECT_VOLUME_SLACK / 4];
+// Fixed scratch for trace records (8 MiB): a call whose table is larger projects its (view,
+// imager column) pairs batch by batch. The largest record (nx + ny = 4096) is 33 KB.
+constexpr size_t STATIC_TRACE_BYTES = 8u << 20;
+static __device__ __align__(256) unsigned char g_static_traces[STATIC_TRACE_BYTES];
 
 // In host code `g_static_volume` names a host-side stand-in, not device memory, so the
 // device address is looked up once per device (with that device current) and cached for
@@ -23,8 +27,9 @@ static __device__ __align__(256) float g_static_volume[CBCT_PROJECT_STATIC_MAX_V
 constexpr int kMaxDevices = 64;
 static std::mutex g_static_mu;
 static float *g_static_ptr[kMaxDevices];
+static void *g_static_trace_ptr[kMaxDevices];
 
-static cbct_status static_volume_address(int device, float **out)
+static cbct_status static_addresses(int device, float **out, void **traces)
 {
     if (device < 0 || device >= kMaxDevices)
         return set_error(CBCT_ERR_UNSUPPORTED, "project_static: device ordinal %d not supported", device);
@@ -33,9 +38,14 @@ static cbct_status static_volume_address(int device, float **out)
         void *p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_static_volume);
         if (e != cudaSuccess) return check_cuda(e, "project_static: scratch address");
+        void *t = nullptr;
+        e = cudaGetSymbolAddress(&t, g_static_traces);
+        if (e != cudaSuccess) return check_cuda(e, "project_static: scratch address");
+        g_static_trace_ptr[device] = t;
         g_static_ptr[device] = static_cast<float *>(p);
     }
     *out = g_static_ptr[device];
+    *traces = g_static_trace_ptr[device];
     return CBCT_OK;
 }
 
@@ -61,11 +71,24 @@ extern "C" cbct_status cbct_project_static(const cbct_geometry *g, const float *
                          "project_static: volume of %lld voxels exceeds the fixed scratch of %d voxels", n,
                          (int)CBCT_PROJECT_STATIC_MAX_VOXELS);
     float *scratch = nullptr;
-    cbct_status st = static_volume_address(dev, &scratch);
+    void *traces = nullptr;
+    cbct_status st = static_addresses(dev, &scratch, &traces);
     if (st != CBCT_OK) return st;
     // the whole scratch region used is overwritten by the layout change before it is read
     cudaStream_t s = (cudaStream_t)stream;
-    st = transpose(f, scratch, G.nx, G.ny, G.nz, true, s);
+    // z-lines padded to a multiple of 4 as cbct_project's where the scratch holds them, else
+    // packed (narrower loads, the same sums)
+    const int zpitch = internal_elems(G) <= (size_t)CBCT_PROJECT_STATIC_MAX_VOXELS ? G.zp : G.nz;
+    st = transpose(f, scratch, G.nx, G.ny, G.nz, zpitch, true, s);
     if (st != CBCT_OK) return st;
-    return launch_project(G, scratch, G.nz, (long long)G.nx * G.nz, 1, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, s);
+    const int ncols = G.nviews * G.nu, batch = (int)(STATIC_TRACE_BYTES / (trace_table_bytes(G) / ncols));
+    for (int c0 = 0; c0 < ncols; c0 += batch) {
+        const int n = ncols - c0 < batch ? ncols - c0 : batch;
+        st = launch_trace_table(G, traces, s, c0, n);
+        if (st != CBCT_OK) return st;
+        st = launch_project(G, scratch, zpitch, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, s, ST_F32, nullptr, traces,
+                            nullptr, c0, n);
+        if (st != CBCT_OK) return st;
+    }
+    return CBCT_OK;
 }

@@ -171,10 +171,10 @@ __global__ void k_update_xp(float *__restrict__ x, float *__restrict__ p, const 
 }
 
 // ------------------------------------------------------------------------------------
-// Layout conversion: public x-fastest [z][y][x] <-> internal z-fastest [y][x][z]
+// Layout conversion: public x-fastest [z][y][x] <-> internal z-fastest [y][x][z], z-lines of zp floats
 // ------------------------------------------------------------------------------------
 
-__global__ void k_pub_to_int(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz)
+__global__ void k_pub_to_int(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz, int zp)
 {
     __shared__ float t[32][33];
     const int xb = blockIdx.x * 32, zb = blockIdx.y * 32, y = blockIdx.z;
@@ -185,17 +185,17 @@ __global__ void k_pub_to_int(const float *__restrict__ in, float *__restrict__ o
     __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
         const int x = xb + j, z = zb + threadIdx.x;
-        if (z < nz && x < nx) out[((size_t)y * nx + x) * nz + z] = t[threadIdx.x][j];
+        if (z < nz && x < nx) out[((size_t)y * nx + x) * zp + z] = t[threadIdx.x][j];
     }
 }
 
-__global__ void k_int_to_pub(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz)
+__global__ void k_int_to_pub(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz, int zp)
 {
     __shared__ float t[32][33];
     const int xb = blockIdx.x * 32, zb = blockIdx.y * 32, y = blockIdx.z;
     for (int j = threadIdx.y; j < 32; j += 8) {
         const int x = xb + j, z = zb + threadIdx.x;
-        if (z < nz && x < nx) t[j][threadIdx.x] = in[((size_t)y * nx + x) * nz + z];
+        if (z < nz && x < nx) t[j][threadIdx.x] = in[((size_t)y * nx + x) * zp + z];
     }
     __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
@@ -204,21 +204,22 @@ __global__ void k_int_to_pub(const float *__restrict__ in, float *__restrict__ o
     }
 }
 
-cbct_status transpose(const float *in, float *out, int nx, int ny, int nz, bool to_internal,
+cbct_status transpose(const float *in, float *out, int nx, int ny, int nz, int zpitch, bool to_internal,
                       cudaStream_t st)
 {
     dim3 grid((nx + 31) / 32, (nz + 31) / 32, ny), block(32, 8);
-    if (to_internal) CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_pub_to_int<<<grid, block, 0, st>>>(in, out, nx, ny, nz));
-    else CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_int_to_pub<<<grid, block, 0, st>>>(in, out, nx, ny, nz));
+    if (to_internal) CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_pub_to_int<<<grid, block, 0, st>>>(in, out, nx, ny, nz, zpitch));
+    else CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_int_to_pub<<<grid, block, 0, st>>>(in, out, nx, ny, nz, zpitch));
     return check_cuda(cudaGetLastError(), "transpose launch");
 }
 
 // ------------------------------------------------------------------------------------
-// Multigrid transfer (Section 2.2.3). layout 0: x-fastest, 1: z-fastest.
+// Multigrid transfer (Section 2.2.3). layout 0: x-fastest, 1: z-fastest with z-lines of p floats.
 // ------------------------------------------------------------------------------------
 
 struct Grid3 {
     int n[3];
+    int p;
     float h[3];
 };
 
@@ -235,9 +236,9 @@ __device__ __forceinline__ void unflatten(size_t i, const int n[3], int layout, 
     }
 }
 
-__device__ __forceinline__ size_t flatten(const int n[3], int layout, int x, int y, int z)
+__device__ __forceinline__ size_t flatten(const Grid3 &g, int layout, int x, int y, int z)
 {
-    return layout == 0 ? ((size_t)z * n[1] + y) * n[0] + x : ((size_t)y * n[0] + x) * n[2] + z;
+    return layout == 0 ? ((size_t)z * g.n[1] + y) * g.n[0] + x : ((size_t)y * g.n[0] + x) * g.p + z;
 }
 
 __global__ void k_prolong(Grid3 cg, const float *__restrict__ fc, Grid3 fg, float *__restrict__ ff, int layout)
@@ -263,9 +264,9 @@ __global__ void k_prolong(Grid3 cg, const float *__restrict__ fc, Grid3 fg, floa
             const int jx = (q & 1) ? i1[0] : i0[0], jy = (q & 2) ? i1[1] : i0[1], jz = (q & 4) ? i1[2] : i0[2];
             const float wt = ((q & 1) ? w[0] : 1.0f - w[0]) * ((q & 2) ? w[1] : 1.0f - w[1]) *
                              ((q & 4) ? w[2] : 1.0f - w[2]);
-            acc = fmaf(wt, __ldg(fc + flatten(cg.n, layout, jx, jy, jz)), acc);
+            acc = fmaf(wt, __ldg(fc + flatten(cg, layout, jx, jy, jz)), acc);
         }
-        ff[i] = acc;
+        ff[flatten(fg, layout, c[0], c[1], c[2])] = acc;
     }
 }
 
@@ -304,7 +305,7 @@ __global__ void k_restrict(Grid3 fg, const float *__restrict__ ff, Grid3 cg, flo
             double s = 0.0;
             for (int z = lo[2]; z <= hi[2]; ++z)
                 for (int y = lo[1]; y <= hi[1]; ++y)
-                    for (int x = lo[0]; x <= hi[0]; ++x) s += ff[flatten(fg.n, layout, x, y, z)];
+                    for (int x = lo[0]; x <= hi[0]; ++x) s += ff[flatten(fg, layout, x, y, z)];
             const double cnt = (double)(hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
             out = (float)(s / cnt);
         }
@@ -316,6 +317,7 @@ static Grid3 grid3(int nx, int ny, int nz, double dx, double dy, double dz)
 {
     Grid3 g;
     g.n[0] = nx; g.n[1] = ny; g.n[2] = nz;
+    g.p = (nz + 3) & ~3;
     g.h[0] = (float)dx; g.h[1] = (float)dy; g.h[2] = (float)dz;
     return g;
 }
@@ -357,7 +359,7 @@ static size_t max_partials(const cbct_geometry *g)
 static size_t work_layout(const cbct_geometry *g, char *base, Work *w)
 {
     const cbct_geometry_desc &d = g->desc;
-    const size_t N = (size_t)d.nx * d.ny * d.nz, M = (size_t)d.n_views * d.nv * d.nu;
+    const size_t N = internal_elems(level_geom(g, 0)), M = (size_t)d.n_views * d.nv * d.nu;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         char *p = base ? base + off : nullptr;
@@ -418,23 +420,24 @@ static cbct_status get_work(cbct_geometry *g, void *ws, size_t ws_bytes, Work *w
 static cbct_status run_cgls(const GeomDev &G, const float *y, float *x, int n_iter, const Work &w, int storage,
                             const void *traces, cudaStream_t st)
 {
-    const long long sz = 1, sx = G.nz, sy = (long long)G.nx * G.nz;
-    const size_t N = (size_t)G.nx * G.ny * G.nz, M = (size_t)G.nviews * G.nv * G.nu;
-    const int nbp = project_num_blocks(G), nbb = backproject_num_blocks(G);
+    const long long sz = 1, sx = G.zp, sy = (long long)G.nx * G.zp;
+    const size_t N = internal_elems(G), M = (size_t)G.nviews * G.nv * G.nu;
+    const int nbb = backproject_num_blocks(G);
+    int nbp = 0;
     // FP32 storage holds |D-S| r and |D-S| q; 16-bit storage holds r and kappa q and the
     // row prefix applies |D-S|. Only FP16 needs kappa (BF16 has FP32's exponent range).
     const int prescale = storage == ST_F32 ? 0 : 1;
     const int scale_q = storage == ST_F16 ? 1 : 0;
     // r = y - P x; s = P^T r; p = s; gamma = ||s||^2
-    TRY(launch_project(G, x, sx, sy, sz, y, w.R, PM_RESID, w.partials, 0.0f, st, storage, w.sc, traces));
+    TRY(launch_project(G, x, G.zp, y, w.R, PM_RESID, w.partials, 0.0f, st, storage, w.sc, traces, &nbp));
     TRY(finalize(w.partials, nbp, w.sc, FIN_RR, st));
     TRY(launch_row_prefix(G, w.R, w.PS, prescale, st, storage));
     TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, w.P, w.partials, st));
     TRY(finalize(w.partials, nbb, w.sc, FIN_GAMMA, st, scale_q));
     for (int l = 0; l < n_iter; ++l) {
         // q = P p, alpha = gamma / ||q||^2
-        TRY(launch_project(G, w.P, sx, sy, sz, nullptr, w.Q, PM_Q_SCALED, w.partials, 0.0f, st, storage, w.sc,
-                           traces));
+        TRY(launch_project(G, w.P, G.zp, nullptr, w.Q, PM_Q_SCALED, w.partials, 0.0f, st, storage, w.sc, traces,
+                           &nbp));
         TRY(finalize(w.partials, nbp, w.sc, FIN_ALPHA, st));
         if (l == n_iter - 1) { // last update: x only; s and p would not be used again
             CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_update_xp<<<vec_blocks(N), 256, 0, st>>>(x, w.P, w.S, w.sc, N, 0));
@@ -485,7 +488,7 @@ static cbct_status run_a2_iteration(const GeomDev &G, const float *y, float mu, 
     TRY(run_cgls(G, y, w.X, o.n_cgls, w, o.storage, traces, st));
     const double t_next = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
     const float c = o.momentum ? (float)((t - 1.0) / t_next) : 0.0f;
-    TRY(launch_tf_shrink_fused(G.nz, G.nx, G.ny, w.X, mu, o.positivity, *f_other, *f_cur, c, last ? nullptr : w.X2,
+    TRY(launch_tf_shrink_fused(G.nz, G.nx, G.ny, G.zp, w.X, mu, o.positivity, *f_other, *f_cur, c, last ? nullptr : w.X2,
                                st));
     std::swap(*f_cur, *f_other);
     std::swap(w.X, w.X2);
@@ -541,11 +544,10 @@ cbct_status reconstruct_cursor_step(ReconCursor *c, cudaStream_t st)
     Work &w = c->w;
     if (!c->started) {
         TRY(reset_scalars(w, st));
-        // the projector's trace table of every level, once per reconstruction (the iteration's
-        // volumes are z-contiguous: strides nz and nx nz)
+        // the projector's trace table of every level, once per reconstruction
         for (int lev = 0; lev < c->levels; ++lev) {
             const GeomDev G = level_geom(c->g, lev);
-            TRY(launch_trace_table(G, G.nz, (long long)G.nx * G.nz, w.TR[lev], st));
+            TRY(launch_trace_table(G, w.TR[lev], st));
         }
         c->f_cur = w.Fa;
         c->f_other = w.Fb;
@@ -557,12 +559,12 @@ cbct_status reconstruct_cursor_step(ReconCursor *c, cudaStream_t st)
     for (;;) {
         if (c->lev < 0) { // every level done: the volume back to the public layout
             const GeomDev G0 = level_geom(c->g, 0);
-            TRY(transpose(c->f_cur, c->f_out, G0.nx, G0.ny, G0.nz, false, st));
+            TRY(transpose(c->f_cur, c->f_out, G0.nx, G0.ny, G0.nz, G0.zp, false, st));
             c->finished = true;
             return CBCT_OK;
         }
         const GeomDev G = level_geom(c->g, c->lev);
-        const size_t N = (size_t)G.nx * G.ny * G.nz;
+        const size_t N = internal_elems(G);
         const int iters = c->iters[c->levels - 1 - c->lev];
         if (c->need_setup) {
             if (c->lev == c->levels - 1) {
@@ -647,16 +649,14 @@ extern "C" cbct_status cbct_project_ex(const cbct_geometry *gc, const float *f, 
     if (!valid_dtype(g_type)) return set_error(CBCT_ERR_INVALID_ARG, "project: unknown storage type %d", (int)g_type);
     cbct_geometry *g = const_cast<cbct_geometry *>(gc);
     const GeomDev G = level_geom(g, 0);
-    const size_t N = (size_t)G.nx * G.ny * G.nz;
-    const size_t vol_bytes = align256(sizeof(float) * N + PROJECT_VOLUME_SLACK);
+    const size_t vol_bytes = align256(sizeof(float) * internal_elems(G) + PROJECT_VOLUME_SLACK);
     TRY(ensure_scratch(g, vol_bytes + trace_table_bytes(G)));
     cudaStream_t st = (cudaStream_t)stream;
     float *fz = g->d_scratch;
     void *traces = reinterpret_cast<char *>(g->d_scratch) + vol_bytes;
-    TRY(transpose(f, fz, G.nx, G.ny, G.nz, true, st));
-    TRY(launch_trace_table(G, G.nz, (long long)G.nx * G.nz, traces, st));
-    return launch_project(G, fz, G.nz, (long long)G.nx * G.nz, 1, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, st,
-                          (int)g_type, nullptr, traces);
+    TRY(transpose(f, fz, G.nx, G.ny, G.nz, G.zp, true, st));
+    TRY(launch_trace_table(G, traces, st));
+    return launch_project(G, fz, G.zp, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, st, (int)g_type, nullptr, traces);
 }
 
 extern "C" cbct_status cbct_project(const cbct_geometry *gc, const float *f, float *g_out, cbct_stream_t stream)
@@ -781,10 +781,10 @@ extern "C" cbct_status cbct_cgls(const cbct_geometry *gc, const float *y, float 
     TRY(get_work(g, nullptr, 0, &w));
     TRY(reset_scalars(w, st));
     const GeomDev G = level_geom(g, 0);
-    TRY(transpose(x, w.Fa, G.nx, G.ny, G.nz, true, st));
-    TRY(launch_trace_table(G, G.nz, (long long)G.nx * G.nz, w.TR[0], st));
+    TRY(transpose(x, w.Fa, G.nx, G.ny, G.nz, G.zp, true, st));
+    TRY(launch_trace_table(G, w.TR[0], st));
     if (n_iter > 0) TRY(run_cgls(G, y, w.Fa, n_iter, w, ST_F32, w.TR[0], st));
-    TRY(transpose(w.Fa, x, G.nx, G.ny, G.nz, false, st));
+    TRY(transpose(w.Fa, x, G.nx, G.ny, G.nz, G.zp, false, st));
     return read_flags(w, st);
 }
 
@@ -858,5 +858,5 @@ extern "C" cbct_status cbct_tf_shrink(int nx, int ny, int nz, const float *f, fl
     if (!f || !out) return set_error(CBCT_ERR_INVALID_ARG, "tf_shrink: null pointer");
     if (f == out) return set_error(CBCT_ERR_INVALID_ARG, "tf_shrink: input and output must differ");
     if (!(mu >= 0.0f) || !std::isfinite(mu)) return set_error(CBCT_ERR_INVALID_ARG, "tf_shrink: mu must be finite and >= 0");
-    return launch_tf_shrink_fused(nx, ny, nz, f, mu, positivity, out, nullptr, 0.0f, nullptr, (cudaStream_t)stream);
+    return launch_tf_shrink_fused(nx, ny, nz, nx, f, mu, positivity, out, nullptr, 0.0f, nullptr, (cudaStream_t)stream);
 }

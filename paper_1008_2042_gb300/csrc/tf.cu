@@ -497,7 +497,7 @@ constexpr int FR_WARPS = FR_ROWS + 4;
 constexpr int FR_THREADS = 32 * FR_WARPS;
 
 __global__ void __launch_bounds__(FR_THREADS, FR_THREADS <= 320 ? 2 : 1)
-k_tf_shrink_fused(int n0, int n1, int n2, int chunk, const float *__restrict__ x, float mu, int positivity,
+k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__restrict__ x, float mu, int positivity,
                   float *__restrict__ fnew, const float *__restrict__ fold, float coef, float *__restrict__ vout)
 {
     __shared__ float s_t[2][FR_WARPS][3][32];              // axis-2 analysis of each row
@@ -507,9 +507,9 @@ k_tf_shrink_fused(int n0, int n1, int n2, int chunk, const float *__restrict__ x
     const int c_begin = blockIdx.z * chunk;
     const int c_end = min(n2, c_begin + chunk);
     if (c_begin >= c_end) return;
-    const size_t plane = (size_t)n0 * n1;
+    const size_t plane = (size_t)p0 * n1;
     const int pa = a_out + lane - 2, pb = b_out + w - 2;  // this lane's position (unwrapped)
-    const size_t inplane = (size_t)wrapi(pb, n1) * n0 + wrapi(pa, n0);
+    const size_t inplane = (size_t)wrapi(pb, n1) * p0 + wrapi(pa, n0);
     const bool coef_row = w >= 1 && w <= FR_ROWS + 2;     // rows whose coefficients are formed
     const bool out_row = w >= 2 && w <= FR_ROWS + 1 && pb < n1;
     const bool out_lane = lane >= 2 && lane < 2 + FR_OUT && pa < n0;
@@ -579,7 +579,7 @@ k_tf_shrink_fused(int n0, int n1, int n2, int chunk, const float *__restrict__ x
             if (cp >= c_begin + 1 && out_lane) {
                 float o = syn3(w_m2[0], w_m1[0], wv[0], w_m2[1], wv[1], w_m2[2], w_m1[2], wv[2]);
                 if (positivity && o < 0.0f) o = 0.0f;
-                const size_t idx = (size_t)(cp - 1) * plane + (size_t)pb * n0 + pa;
+                const size_t idx = (size_t)(cp - 1) * plane + (size_t)pb * p0 + pa;
                 fnew[idx] = o;
                 if (vout) vout[idx] = fmaf(coef, o - __ldg(fold + idx), o);
             }
@@ -597,7 +597,7 @@ k_tf_shrink_fused(int n0, int n1, int n2, int chunk, const float *__restrict__ x
 
 cbct_status tf_prepare() { return CBCT_OK; }
 
-cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, const float *x, float mu, int positivity, float *fnew,
+cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *x, float mu, int positivity, float *fnew,
                                    const float *fold, float coef, float *vout, cudaStream_t st)
 {
     int per_sm = 0;
@@ -607,7 +607,7 @@ cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, const float *x, float
     const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
     dim3 grid((n0 + FR_OUT - 1) / FR_OUT, (n1 + FR_ROWS - 1) / FR_ROWS, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
-               k_tf_shrink_fused<<<grid, dim3(32, FR_WARPS), 0, st>>>(n0, n1, n2, chunk, x, mu, positivity, fnew, fold,
+               k_tf_shrink_fused<<<grid, dim3(32, FR_WARPS), 0, st>>>(n0, n1, n2, p0, chunk, x, mu, positivity, fnew, fold,
                                                                       coef, vout));
     return check_cuda(cudaGetLastError(), "tf_shrink_fused launch");
 }
