@@ -14,67 +14,88 @@
 // a z plane inside the column (about 0.1 per plane at the paper's sizes) are evaluated
 // one by one. The factor |D - S| is folded into the table, which holds for every row m
 // the pair (prefix of the rows below m, value of row m): one 8-byte load per plane gives
-// both the window's prefix and its straddling row. Every crossing parameter
-// uses the same helper expressions as the projector, so both operators use the same
-// FP32 weights. No atomics: the result is independent of scheduling.
+// both the window's prefix and its straddling row. The crossing parameters come from the
+// same plane coordinates and reciprocals as the projector's, so both operators use the same
+// weights to FP32 rounding. No atomics: the result is independent of scheduling.
+//
+// What bounds it on the paper's finest grid (512x512x70, 40 views, 1.25 ms, 14 voxels per
+// thread): L1 data wavefronts 69-74% (the table's lines: lanes of a patch read about ten
+// sectors), issue slots 71%. Before the straddling row became one saturating multiply and
+// the chunks whole it took 1.63 ms; with the warps of a block on the same patch taking
+// turns at the views, 128x128x18 takes 104 us (200 before), 64x64x16 25 us (61).
 #include "cbct_internal.cuh"
 
-#include <type_traits>
+#include <cmath>
 
 namespace cbct {
 
-// Thread mapping: each warp takes an 8 x 4 patch of voxel columns, and a block of NT
-// threads stacks them into a 16 x (NT / 8) tile. Lanes whose columns are close in both x
-// and y read nearby table entries in every view (a voxel's imager column moves with x at
-// some views and with y at others): an 8 x 4 patch touches 10 sectors per table request
-// where a 32 x 1 row touched 16, and the warps of a block share their lines in L1. Larger
-// blocks share more of each view's table lines and pay where the grid is large (16-voxel
-// chunks on the paper's finest grid, kernel alone: 128 threads 1.80 ms, 256 1.72 ms, 512
-// (16 x 32 columns) 1.70 ms, 1024 1.72 ms); on coarser grids they leave too few blocks,
-// and 128 threads are kept.
-constexpr int BP_THREADS = 128;                 // the block size of the coarser grids
-constexpr int BP_BIG_THREADS = 512;             // with 16-voxel chunks
-constexpr int BP_WX = 8, BP_WY = 4;             // warp patch
-constexpr int BP_BX = 16;                       // block tile along x (two patches)
-template <int NT> constexpr int bp_by() { return BP_WY * (NT / 64); } // block tile along y
-constexpr int BP_BY = bp_by<BP_THREADS>();
+// Thread mapping: each warp takes an 8 x 4 patch of voxel columns and a block stacks patches two
+// wide. Lanes whose columns are close in both x and y read nearby table entries in every view
+// (a voxel's imager column moves with x at some views and with y at others): an 8 x 4 patch
+// touches 10 sectors per table request where a 32 x 1 row touched 16, and the warps of a
+// block share their lines in L1. Where the grid has too few columns to fill the chip, the
+// warps of a block also split the views: `slices` warps take the same patch and every
+// slices-th view each, and their sums are added in a fixed order through shared memory.
+constexpr int BP_WX = 8, BP_WY = 4; // warp patch
 
-// resident blocks per SM the register budget of the 16-voxel chunks is sized for (64
-// registers, no spills)
-#ifndef CBCT_BP_Z16_BLOCKS
-#define CBCT_BP_Z16_BLOCKS 8
-#endif
+// A launch: zc voxels per thread (an instantiation), warps per block and view slices per patch; a
+// block holds warps / slices patches, two wide. The last chunk of a
+// column ends at its top and so may overlap the one before, which keeps the voxels they share:
+// every chunk is whole, and the plane loop needs no test of where it ends.
+struct BpPlan {
+    int zc, warps, slices;
+    int bx, by; // columns of a block's tile
+    dim3 grid;
+};
+constexpr int BP_MAX_WARPS = 16;
+constexpr int BP_ZC[] = {8, 12, 14, 16, 18};
 
-// z voxels per thread. 16 halves the per-visit setup and the plane shared by two chunks,
-// but doubles a thread's work: it pays only where the grid still fills many waves of the
-// resident slots (at least six of 8 blocks per SM); measured 2.35 -> 2.26 ms for the paper's
-// 512x512x70 grid and 2.01 -> 1.87 ms for 512x512x128, while 256x256x64 (under two waves)
-// and 256x256x35 (a ragged last chunk) lose 1-4%. Otherwise 8, halved while the grid has
-// fewer than 4 blocks per SM.
-static int bp_zchunk(const GeomDev &G)
+// The voxels per thread that cover a column with the fewest planes (about one and a half more per
+// chunk for its first plane and set-up); measured at 512x512x70 (12 | 14 | 16 | 18): 1357 | 1254 | 1433 |
+// 1320 us, 256x256x35: 339 | 392 | 430 | 347 us. Where even 8 slices leave few warps, 8 voxels
+// (64x64x16: 24.6 us, with 16 32.8 us). Slices double until the chip has about 96 warps per
+// SM to draw from: 256x256x35 with 1 | 2 | 4 | 8 slices 403 | 354 | 339 | 356 us, 128x128x18 456 |
+// 240 | 131 | 104 us, 512x512x70 1254 | 1311 | 1393 | 1583 us (less of the table is shared in L1).
+static BpPlan bp_plan(const GeomDev &G)
 {
-    const long long tiles = (long long)((G.nx + BP_BX - 1) / BP_BX) * ((G.ny + BP_BY - 1) / BP_BY);
+    BpPlan p{};
+    const long long patches = (long long)((G.nx + BP_WX - 1) / BP_WX) * ((G.ny + BP_WY - 1) / BP_WY);
     const long long sms = device_sm_count();
-    if (tiles * ((G.nz + 15) / 16) >= 6LL * CBCT_BP_Z16_BLOCKS * sms) return 16;
-    const long long want = 4LL * sms;
-    int zc = 8;
-    while (zc > 1 && tiles * ((G.nz + zc - 1) / zc) < want) zc >>= 1;
-    return zc;
+    int chunks = 0, best = 1 << 30;
+    for (int zc : BP_ZC) {
+        const int n = (G.nz + zc - 1) / zc, cost = n * (2 * zc + 3);
+        if (cost < best) {
+            best = cost;
+            p.zc = zc;
+            chunks = n;
+        }
+    }
+    if (patches * chunks * 8 < 16 * sms) {
+        p.zc = BP_ZC[0];
+        chunks = (G.nz + p.zc - 1) / p.zc;
+    }
+    p.warps = BP_MAX_WARPS;
+    p.slices = 1;
+    while (p.slices < 8 && patches * chunks * p.slices < 96 * sms && 2 * p.slices <= G.nviews) p.slices *= 2;
+    const int patches_block = p.warps / p.slices;
+    p.bx = 2 * BP_WX;
+    p.by = patches_block / 2 * BP_WY;
+    p.grid = dim3((G.nx + p.bx - 1) / p.bx, (G.ny + p.by - 1) / p.by, chunks);
+    return p;
 }
+
+size_t prefix_table_bytes(const GeomDev &G) { return sizeof(float2) * (size_t)G.nviews * G.nu * ((size_t)G.nv + 1); }
 
 int backproject_max_blocks(const GeomDev &G)
 {
-    return ((G.nx + BP_BX - 1) / BP_BX) * ((G.ny + BP_BY - 1) / BP_BY) * G.nz; // one z voxel per thread
+    // the smallest tile is two patches (8 slices of 16 warps), the smallest chunk 8 voxels
+    return ((G.nx + 2 * BP_WX - 1) / (2 * BP_WX)) * ((G.ny + BP_WY - 1) / BP_WY) * ((G.nz + BP_ZC[0] - 1) / BP_ZC[0]);
 }
-
-// threads per block of a launch with z chunk zc
-static int bp_threads(int zc) { return zc >= 16 ? BP_BIG_THREADS : BP_THREADS; }
 
 int backproject_num_blocks(const GeomDev &G)
 {
-    const int zc = bp_zchunk(G);
-    const int by = bp_threads(zc) == BP_BIG_THREADS ? bp_by<BP_BIG_THREADS>() : BP_BY;
-    return ((G.nx + BP_BX - 1) / BP_BX) * ((G.ny + by - 1) / by) * ((G.nz + zc - 1) / zc);
+    const BpPlan p = bp_plan(G);
+    return (int)(p.grid.x * p.grid.y * p.grid.z);
 }
 
 // Rows whose ray, while inside the column (tau in [ta, tb], 1/(tc+ta) = A, 1/(tc+tb) = B),
@@ -90,259 +111,252 @@ __device__ __forceinline__ void straddle_rows(const GeomDev &G, float zp, float 
     hi = (int)floorf(fhi);
 }
 
-// The straddling row of a plane window [a, b) (b <= a + 1; table entry T = (P[a], g[a]))
-// split at the plane: its weighted value g (0 if the window is empty) times the part of
-// [ta, tb] below and above the plane z = zp.
-__device__ __forceinline__ void plane_split(const GeomDev &G, const float *s_invv, float2 T, int a, int b, float zp,
-                                            float ta, float tb, float &g, float &below, float &above)
+// The planes of one visit to a voxel column: the ray column's entries of the prefix table `tab`
+// (entry m at row_bytes * m, biased by ROUND_BIAS rows), 1 / v of the rows at shared address `iv`
+// (biased likewise), the column's interval [ta, tb] with A = 1 / (tc + ta), B = 1 / (tc + tb).
+constexpr int ROUND_BIAS = 0x4B400000; // bits of 1.5 * 2^23: what ceil by the FP adder leaves on top
+struct BpVisit {
+    const char *tab;
+    unsigned iv;
+    int row_bytes;
+    float ta, tb, A, B;
+};
+// The chunk: its lowest plane (and in rows at unit scale), the plane pitch in rows at unit scale,
+// the row coordinate of v = 0 minus the windows' margin, its voxels (ZC, or all nz < ZC).
+struct BpChunk {
+    float zbot, zs_bot, dzs, c0;
+    int nzc;
+};
+
+// Adds this visit's share of every voxel of the chunk. The rows that reach plane zp inside the
+// column lie in the window [zp B, zp A] of v (zp >= 0; [zp A, zp B] below) and are at most one
+// (the caller's `simple` test): row a, the first at or above the window's start. With the prefix
+// P[a] of the rows below, plane z is passed by
+//     (tb - ta) P[a_z] + below_z,   below_z = g_a * (part of [ta, tb] with row a below the plane),
+// and slab z receives the difference of its two planes,
+//     (tb - ta) ((P[a_{z+1}] - P[a_z]) + g_{z+1} f_{z+1} - g_z f_z),
+// with f the fraction of [ta, tb] that row a spends below the plane. f comes from the
+// crossing tau = zp / v - tc by one saturating multiply: where row a lies beyond the window, tau lies
+// beyond [ta, tb] on the side where f is 0, so no test of the window's end is needed.
+// SIDE +1 / -1: row a of every plane has v > 0 / v < 0 (it rises / falls); 0: tested per row.
+// CLAMP: windows may leave the imager (rows clamped to [0, nv]; entry nv has value 0).
+// FULL: the chunk has ZC voxels.
+template <int ZC, int SIDE, bool CLAMP, bool FULL>
+__device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, const BpChunk &c, float (&acc)[ZC])
 {
-    g = b > a ? T.y : 0.0f;
-    const float iw = s_invv[min(a, G.nv - 1)];
-    const float scl = fminf(fmaxf(tau_zplane(zp, iw, G.tc), ta), tb);
-    const float wlo = scl - ta, whi = tb - scl;
-    const bool up = iw > 0.0f; // z grows along the ray (v >= 0)
-    below = g * (up ? wlo : whi);
-    above = g * (up ? whi : wlo);
+    const float w = q.tb - q.ta, winv = __fdividef(1.0f, w);
+    const float sa = G.tc + q.ta, sb = G.tc + q.tb;
+    const float lo = SIDE < 0 ? q.A : q.B, x0 = fmaf(c.zs_bot, lo, c.c0), xs = c.dzs * lo;
+    auto plane = [&](int z, float &P, float &g, float &f) {
+        const float zp = fmaf((float)z, G.dz, c.zbot);
+        float x;
+        if (SIDE != 0) {
+            x = fmaf((float)z, xs, x0);
+        } else {
+            const float zs = fmaf((float)z, c.dzs, c.zs_bot);
+            x = fmaf(zs, zs >= 0.0f ? q.B : q.A, c.c0);
+        }
+        if (CLAMP) x = fminf(fmaxf(x, 0.0f), (float)G.nv);
+        const int a = __float_as_int(__fadd_ru(x, 12582912.0f)); // ROUND_BIAS + ceil(x)
+        const float2 T = __ldg(reinterpret_cast<const float2 *>(q.tab + (long long)a * q.row_bytes));
+        const float iw = lds_float(q.iv + 4u * (unsigned)a);
+        if (SIDE > 0) {
+            f = __saturatef(fmaf(zp, iw, -sa) * winv);
+        } else if (SIDE < 0) {
+            f = __saturatef(fmaf(-zp, iw, sb) * winv);
+        } else {
+            f = __saturatef(fmaf(zp, iw, -sa) * winv);
+            if (!(iw > 0.0f)) f = 1.0f - f;
+        }
+        P = T.x;
+        g = f > 0.0f ? T.y : 0.0f; // (a row outside the window is not touched, whatever its value)
+    };
+    float P0, g0, f0;
+    plane(0, P0, g0, f0);
+#pragma unroll
+    for (int z = 0; z < ZC; ++z) {
+        if (!FULL && z >= c.nzc) break;
+        float P1, g1, f1;
+        plane(z + 1, P1, g1, f1);
+        acc[z] = fmaf(w, fmaf(-g0, f0, fmaf(g1, f1, P1 - P0)), acc[z]);
+        P0 = P1;
+        g0 = g1;
+        f0 = f1;
+    }
 }
 
-// For a window on the imager (a <= nv - 1: the row exists; `in`: row a lies in the window,
-// i.e. b > a): the weighted value of the straddling row times the part of [ta, tb] that
-// lies below the plane z = zp (0 if the window is empty). UP = +1 / -1: the caller knows
-// that a row in the window has v > 0 / v < 0 (its ray rises / falls), so the direction
-// test is dropped; UP = 0 tests it.
-template <int UP>
-__device__ __forceinline__ float plane_below(const float *s_invv, float tc, float2 T, int a, bool in, float zp,
-                                             float ta, float tb)
-{
-    const float g = in ? T.y : 0.0f;
-    const float iw = s_invv[a];
-    const float scl = fminf(fmaxf(tau_zplane(zp, iw, tc), ta), tb);
-    const bool up = UP > 0 ? true : UP < 0 ? false : iw > 0.0f;
-    return g * (up ? scl - ta : tb - scl);
-}
-
-// Rows reaching plane zp inside the column lie in the window [a, b) of imager rows (at
-// most one row when the caller's `simple` test holds); a and b are clamped to [0, nv] so
-// that the table entry col[a * nu] exists (the table is [view][row 0..nv][column]).
-__device__ __forceinline__ void plane_window(const GeomDev &G, float zp, float A, float B, float c0, float c1,
-                                             int &a, int &b)
-{
-    const float v0 = zp * A, v1 = zp * B;
-    const float nvf = (float)G.nv;
-    const float fa = fminf(fmaxf(fmaf(fminf(v0, v1), G.inv_dv, c0), 0.0f), nvf);
-    const float fb = fminf(fmaxf(fmaf(fmaxf(v0, v1), G.inv_dv, c1), -1.0f), nvf - 1.0f);
-    a = ceil_small(fa);
-    b = floor_small(fb) + 1;
-}
-
-// Register budget of the 8-voxel chunks: 9 resident blocks of 128 threads (56 registers, no
-// spills) instead of the 5 that 88 registers allowed; measured 2.96 -> 2.34 ms for one P^T
-// of the paper grid through the public call, bit-identical results. Shorter chunks keep
-// the compiler's choice (fewer registers there cost more than they gain).
-#ifndef CBCT_BP_MIN_BLOCKS
-#define CBCT_BP_MIN_BLOCKS 9
-#endif
-template <int ZC, bool FLAT, int NT>
-__global__ void __launch_bounds__(NT, ZC >= 16 ? CBCT_BP_Z16_BLOCKS * 128 / NT : ZC >= 8 ? CBCT_BP_MIN_BLOCKS : 1)
-k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz,
+// Register budget: 64, two resident blocks of 512 threads.
+// FLAT: each lane walks its own list of candidates (view, imager column), so a warp runs for the
+// longest per-lane total instead of the widest shadow in every view: fewer idle lanes where
+// shadows are about one column wide.
+template <int ZC, bool FLAT>
+__global__ void __launch_bounds__(32 * BP_MAX_WARPS, 2)
+k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz, int slices,
               float *__restrict__ out2, double *__restrict__ partials)
 {
-    extern __shared__ float s_invv[]; // 1 / v per imager row
-    __shared__ double s_warp[NT / 32];
+    extern __shared__ float smem[]; // 1 / v per imager row (one more for entry nv); then the slices' sums
+    __shared__ double s_warp[BP_MAX_WARPS];
+    float *s_invv = smem, *s_sum = smem + G.nv + 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < G.nv; i += NT) {
+    for (int i = tid; i <= G.nv; i += blockDim.x) {
         const float v = imager_v(G, i);
         s_invv[i] = v != 0.0f ? __frcp_rn(v) : 1e30f;
     }
-    __syncthreads();
 
-    const int ix = blockIdx.x * BP_BX + (warp & 1) * BP_WX + lane % BP_WX;
-    const int iy = blockIdx.y * bp_by<NT>() + (warp >> 1) * BP_WY + lane / BP_WX;
-    const int iz0 = blockIdx.z * ZC;
+    const int npatch = (blockDim.x >> 5) / slices, slice = warp / npatch, patch = warp - slice * npatch;
+    const int bx = 2 * BP_WX, by = npatch / 2 * BP_WY;
+    const int ix = blockIdx.x * bx + (patch & 1) * BP_WX + lane % BP_WX;
+    const int iy = blockIdx.y * by + (patch >> 1) * BP_WY + lane / BP_WX;
+    const int iz0 = max(0, min((int)blockIdx.z * ZC, G.nz - ZC)), iz_own = blockIdx.z * ZC; // first voxel; first that is stored
     const bool ok = ix < G.nx && iy < G.ny;
     float acc[ZC];
 #pragma unroll
     for (int z = 0; z < ZC; ++z) acc[z] = 0.0f;
 
-    if (ok) {
-        const float xl = plane_at(ix, G.dx, G.x0), xh = plane_at(ix + 1, G.dx, G.x0);
-        const float yl = plane_at(iy, G.dy, G.y0), yh = plane_at(iy + 1, G.dy, G.y0);
-        float zp[ZC + 1], zs[ZC + 1];
-#pragma unroll
-        for (int z = 0; z <= ZC; ++z) {
-            zp[z] = plane_at(iz0 + z, G.dz, G.z0);
-            zs[z] = zp[z] * G.inv_dv;
-        }
-        const int nzc = min(ZC, G.nz - iz0); // valid voxels in this chunk
-        const float ztop = plane_at(iz0 + nzc, G.dz, G.z0), zs_top = ztop * G.inv_dv; // the chunk's top plane
-        const float zabs = fmaxf(fabsf(zp[0]), fabsf(ztop));
-        const size_t view_stride = ((size_t)G.nv + 1) * G.nu;
-        const float c0 = fmaf(-G.v_first, G.inv_dv, -1e-3f), c1 = fmaf(-G.v_first, G.inv_dv, 1e-3f);
+    const float xl = plane_at(ix, G.dx, G.x0), xh = plane_at(ix + 1, G.dx, G.x0);
+    const float yl = plane_at(iy, G.dy, G.y0), yh = plane_at(iy + 1, G.dy, G.y0);
+    BpChunk ch;
+    ch.nzc = min(ZC, G.nz);
+    ch.zbot = plane_at(iz0, G.dz, G.z0);
+    ch.zs_bot = ch.zbot * G.inv_dv;
+    ch.dzs = G.dz * G.inv_dv;
+    ch.c0 = fmaf(-G.v_first, G.inv_dv, -1e-3f);
+    const float ztop = plane_at(iz0 + ch.nzc, G.dz, G.z0), zs_top = ztop * G.inv_dv;
+    const float zabs = fmaxf(fabsf(ch.zbot), fabsf(ztop));
+    const float c1 = fmaf(-G.v_first, G.inv_dv, 1e-3f);
+    const size_t view_stride = ((size_t)G.nv + 1) * G.nu;
+    const unsigned iv0 = smem_u32(s_invv) - 4u * (unsigned)ROUND_BIAS;
 
-        // imager columns in the shadow of the voxel column in view k (its corners' u)
-        auto shadow = [&](int k, int &lo, int &hi) {
-            const float2 cs = G.cs[k];
-            float umin = 3.0e38f, umax = -3.0e38f;
+    // imager columns in the shadow of the voxel column in view k (its corners' u)
+    auto shadow = [&](int k, int &lo, int &hi) {
+        const float2 cs = G.cs[k];
+        float umin = 3.0e38f, umax = -3.0e38f;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float px = (c & 1) ? xh : xl, py = (c & 2) ? yh : yl;
-                const float a = fmaf(-px, cs.y, py * cs.x);
-                const float w = G.sad - fmaf(px, cs.x, py * cs.y);
-                const float u = G.sdd * __fdividef(a, w);
-                umin = fminf(umin, u);
-                umax = fmaxf(umax, u);
-            }
-            lo = max(0, (int)ceilf(fmaf(umin - G.u_first, G.inv_du, -1e-3f)));
-            hi = min(G.nu - 1, (int)floorf(fmaf(umax - G.u_first, G.inv_du, 1e-3f)));
-        };
-        // all rows of imager column iu in view k that cross this voxel column
-        auto visit = [&](int k, int iu) {
-                const float4 r4 = __ldg(G.ray4 + k * G.nu + iu); // (dxr, dyr, qx, qy)
-                const float2 r2 = __ldg(G.ray2 + k * G.nu + iu); // (1/dxr, 1/dyr)
-                const float t0 = tau_plane(xl, r4.z, r2.x), t1 = tau_plane(xh, r4.z, r2.x);
-                const float t2 = tau_plane(yl, r4.w, r2.y), t3 = tau_plane(yh, r4.w, r2.y);
-                const float ta = fmaxf(fminf(t0, t1), fminf(t2, t3));
-                const float tb = fminf(fmaxf(t0, t1), fmaxf(t2, t3));
-                if (!(tb > ta)) return;
-                const float A = __fdividef(1.0f, G.tc + ta), B = __fdividef(1.0f, G.tc + tb);
-                const float wfull = tb - ta;
-                const float2 *col = ps + (size_t)k * view_stride + iu; // prefix m at col[m * nu]
-                // Plane z = zp is reached by the rows with v between zp*A and zp*B. While that
-                // window is shorter than a row pitch and adjacent planes' windows are apart,
-                // every row crosses at most one plane inside the column (the usual case).
-                const float span = zabs * (A - B) * G.inv_dv;
-                const bool simple = span + 3e-3f < 1.0f && fmaf(G.dz * B, G.inv_dv, -span) > 3e-3f;
-                // row-window bounds at the lowest and highest plane of the chunk (monotone
-                // in the plane height, so these bound every plane's window)
-                const float fa_lo = fmaf(zs[0], zs[0] >= 0.0f ? B : A, c0);
-                const float fb_hi = fmaf(zs_top, zs_top >= 0.0f ? A : B, c1);
-                if (simple && fa_lo >= 0.0f && fb_hi <= (float)(G.nv - 1)) {
-                    // every window lies on the imager: no clamping. Slab z receives the rows
-                    // strictly between the windows of planes z and z + 1 at weight tb - ta,
-                    // P[a_{z+1}] - P[a_z] - g_z, the part of plane z's straddling row above
-                    // the plane, g_z (tb - ta) - below_z, and the part of plane z + 1's
-                    // straddling row below it, below_{z+1}; together
-                    //     (tb - ta) (P[a_{z+1}] - P[a_z]) + below_{z+1} - below_z.
-                    // The window of plane zp spans rows v in [zp B, zp A] above z = 0 and
-                    // [zp A, zp B] below; a chunk whose planes all lie on one side (all but
-                    // one chunk of a column) fixes that choice for the whole visit. Its
-                    // windows' rows then also share the sign of v (below: the test that
-                    // picks the side keeps every window a thousandth of a row pitch or more
-                    // away from v = 0), so the split needs no per-row direction test.
-                    auto planes = [&](auto side) {
-                        constexpr int S = decltype(side)::value; // +1 / -1: every plane at z > 0 / < 0
-                        auto bounds = [&](float zsv, float &lo_f, float &hi_f) {
-                            const bool pos = S > 0 || (S == 0 && zsv >= 0.0f);
-                            lo_f = pos ? B : A;
-                            hi_f = pos ? A : B;
-                        };
-                        // The window is [a, b) with a = ceil(xa), b = floor(xb) + 1; row a is in it
-                        // iff floor(xb) >= a, i.e. xb >= a (a is an integer), so b is not formed.
-                        float lo_f, hi_f;
-                        bounds(zs[0], lo_f, hi_f);
-                        int a = ceil_small(fmaf(zs[0], lo_f, c0));
-                        bool in = fmaf(zs[0], hi_f, c1) >= (float)a;
-                        float2 T = __ldg(col + a * G.nu); // (nv + 1) * nu < 2^31: 32-bit offsets
-                        float Pprev = T.x, bprev = plane_below<S>(s_invv, G.tc, T, a, in, zp[0], ta, tb);
-#pragma unroll
-                        for (int z = 0; z < ZC; ++z) {
-                            if (z >= nzc) break;
-                            bounds(zs[z + 1], lo_f, hi_f);
-                            a = ceil_small(fmaf(zs[z + 1], lo_f, c0));
-                            in = fmaf(zs[z + 1], hi_f, c1) >= (float)a;
-                            T = __ldg(col + a * G.nu);
-                            const float below = plane_below<S>(s_invv, G.tc, T, a, in, zp[z + 1], ta, tb);
-                            acc[z] += fmaf(wfull, T.x - Pprev, below - bprev);
-                            Pprev = T.x;
-                            bprev = below;
-                        }
-                    };
-                    // Side +1: the window of the lowest plane, hence of every plane, starts
-                    // at a row with v / dv >= zs[0] B - 1e-3 > 0; side -1: every window ends
-                    // at a row with v / dv <= zs_top B + 1e-3 < 0. Otherwise (a chunk that
-                    // meets or nearly meets z = 0) both the side and the direction are
-                    // decided per plane, which gives the same bounds for the planes at z >= 0.
-                    if (zs[0] * B > 2e-3f) planes(std::integral_constant<int, 1>());
-                    else if (zs_top * B < -2e-3f) planes(std::integral_constant<int, -1>());
-                    else planes(std::integral_constant<int, 0>());
-                } else if (simple) {
-                    // windows may leave the imager: clamped to [0, nv]
-                    int a, b;
-                    plane_window(G, zp[0], A, B, c0, c1, a, b);
-                    float2 T = __ldg(col + a * G.nu);
-                    float g, below, above;
-                    plane_split(G, s_invv, T, a, b, zp[0], ta, tb, g, below, above);
-                    acc[0] += above;
-                    float Pprev = T.x, gprev = g;
-#pragma unroll
-                    for (int z = 0; z < ZC; ++z) {
-                        if (z >= nzc) break;
-                        plane_window(G, zp[z + 1], A, B, c0, c1, a, b);
-                        T = __ldg(col + a * G.nu);
-                        plane_split(G, s_invv, T, a, b, zp[z + 1], ta, tb, g, below, above);
-                        acc[z] = fmaf(wfull, (T.x - Pprev) - gprev, acc[z]) + below;
-                        if (z + 1 < ZC && z + 1 < nzc) acc[z + 1] += above;
-                        Pprev = T.x;
-                        gprev = g;
-                    }
-                } else {
-                    int lo_p, hi_p;
-                    straddle_rows(G, zp[0], A, B, lo_p, hi_p);
-#pragma unroll
-                    for (int z = 0; z < ZC; ++z) {
-                        if (z >= nzc) break;
-                        int lo_n, hi_n;
-                        straddle_rows(G, zp[z + 1], A, B, lo_n, hi_n);
-                        float a = acc[z];
-                        const int f0 = max(hi_p + 1, 0), f1 = min(lo_n - 1, G.nv - 1);
-                        if (f0 <= f1) {
-                            const float P1 = __ldg(col + (f1 + 1) * G.nu).x, P0 = __ldg(col + f0 * G.nu).x;
-                            a = fmaf(wfull, P1 - P0, a);
-                        }
-                        // rows that cross a z plane inside the column: exact overlap
-                        const int r0 = max(lo_p, 0), r1 = min(hi_n, G.nv - 1);
-                        for (int iv = r0; iv <= r1; ++iv) {
-                            if (iv == f0 && f0 <= f1) { // already counted
-                                iv = f1;
-                                continue;
-                            }
-                            const float iw = s_invv[iv];
-                            const float s0 = tau_zplane(zp[z], iw, G.tc), s1 = tau_zplane(zp[z + 1], iw, G.tc);
-                            const float lo = fmaxf(ta, fminf(s0, s1)), hi = fminf(tb, fmaxf(s0, s1));
-                            if (hi > lo) a = fmaf(__ldg(col + iv * G.nu).y, hi - lo, a);
-                        }
-                        acc[z] = a;
-                        lo_p = lo_n;
-                        hi_p = hi_n;
-                    }
-                }
-        };
-        if (FLAT) {
-            // Each lane walks its own list of candidates (view, imager column) across all
-            // views in one loop, so a warp runs for the longest per-lane total instead of the
-            // widest shadow in every view: fewer idle lanes where shadows are ~1 column wide.
-            int k = -1, iu = 0, iu_hi = -1;
-            for (;;) {
-                while (iu > iu_hi && k < G.nviews) // next view with a non-empty shadow
-                    if (++k < G.nviews) shadow(k, iu, iu_hi);
-                if (k >= G.nviews) break;
-                visit(k, iu++);
+        for (int c = 0; c < 4; ++c) {
+            const float px = (c & 1) ? xh : xl, py = (c & 2) ? yh : yl;
+            const float a = fmaf(-px, cs.y, py * cs.x);
+            const float w = G.sad - fmaf(px, cs.x, py * cs.y);
+            const float u = G.sdd * __fdividef(a, w);
+            umin = fminf(umin, u);
+            umax = fmaxf(umax, u);
+        }
+        lo = max(0, (int)ceilf(fmaf(umin - G.u_first, G.inv_du, -1e-3f)));
+        hi = min(G.nu - 1, (int)floorf(fmaf(umax - G.u_first, G.inv_du, 1e-3f)));
+    };
+    // all rows of imager column iu in view k that cross this voxel column
+    auto visit = [&](int k, int iu) {
+        const float4 r4 = __ldg(G.ray4 + k * G.nu + iu); // (dxr, dyr, qx, qy)
+        const float2 r2 = __ldg(G.ray2 + k * G.nu + iu); // (1/dxr, 1/dyr)
+        const float t0 = tau_plane(xl, r4.z, r2.x), t1 = tau_plane(xh, r4.z, r2.x);
+        const float t2 = tau_plane(yl, r4.w, r2.y), t3 = tau_plane(yh, r4.w, r2.y);
+        const float ta = fmaxf(fminf(t0, t1), fminf(t2, t3));
+        const float tb = fminf(fmaxf(t0, t1), fmaxf(t2, t3));
+        if (!(tb > ta)) return;
+        const float A = __fdividef(1.0f, G.tc + ta), B = __fdividef(1.0f, G.tc + tb);
+        const size_t entry = (size_t)k * view_stride + iu; // row m's entry: ps[entry + m * nu]
+        // Plane z = zp is reached by the rows with v between zp*A and zp*B. While that
+        // window is shorter than a row pitch and adjacent planes' windows are apart,
+        // every row crosses at most one plane inside the column (the usual case).
+        const float span = zabs * (A - B) * G.inv_dv;
+        if (span + 3e-3f < 1.0f && fmaf(G.dz * B, G.inv_dv, -span) > 3e-3f) {
+            BpVisit q;
+            q.iv = iv0;
+            q.ta = ta;
+            q.tb = tb;
+            q.A = A;
+            q.B = B;
+            // row-window bounds at the lowest and highest plane of the chunk (monotone
+            // in the plane height, so these bound every plane's window)
+            const bool inside = fmaf(ch.zs_bot, ch.zs_bot >= 0.0f ? B : A, ch.c0) >= 0.0f &&
+                                fmaf(zs_top, zs_top >= 0.0f ? A : B, c1) <= (float)(G.nv - 1);
+            // Side +1: the window of the lowest plane, hence of every plane, starts at a row
+            // with v / dv >= zs B - 1e-3 > 0, and so does every row at or above a window's start;
+            // side -1: every window ends more than a row below v = 0, so that the first row
+            // above a window's start has v < 0 even where it lies beyond the window.
+            const int side = !inside ? 0 : ch.zs_bot * B > 2e-3f ? 1 : zs_top * B < -1.002f ? -1 : 0;
+            q.row_bytes = 8 * G.nu;
+            q.tab = reinterpret_cast<const char *>(ps + entry) - (long long)ROUND_BIAS * q.row_bytes;
+            if (ch.nzc == ZC) {
+                if (side > 0) bp_planes<ZC, 1, false, true>(G, q, ch, acc);
+                else if (side < 0) bp_planes<ZC, -1, false, true>(G, q, ch, acc);
+                else bp_planes<ZC, 0, true, true>(G, q, ch, acc);
+            } else {
+                bp_planes<ZC, 0, true, false>(G, q, ch, acc);
             }
         } else {
-            for (int k = 0; k < G.nviews; ++k) {
-                int lo, hi;
-                shadow(k, lo, hi);
-                for (int iu = lo; iu <= hi; ++iu) visit(k, iu);
+            const float2 *col = ps + entry;
+            const float wfull = tb - ta;
+            int lo_p, hi_p;
+            straddle_rows(G, ch.zbot, A, B, lo_p, hi_p);
+#pragma unroll
+            for (int z = 0; z < ZC; ++z) {
+                if (z >= ch.nzc) break;
+                const float z0 = plane_at(iz0 + z, G.dz, G.z0), z1 = plane_at(iz0 + z + 1, G.dz, G.z0);
+                int lo_n, hi_n;
+                straddle_rows(G, z1, A, B, lo_n, hi_n);
+                float a = acc[z];
+                const int f0 = max(hi_p + 1, 0), f1 = min(lo_n - 1, G.nv - 1);
+                if (f0 <= f1) {
+                    const float P1 = __ldg(col + (f1 + 1) * G.nu).x, P0 = __ldg(col + f0 * G.nu).x;
+                    a = fmaf(wfull, P1 - P0, a);
+                }
+                // rows that cross a z plane inside the column: exact overlap
+                const int r0 = max(lo_p, 0), r1 = min(hi_n, G.nv - 1);
+                for (int iv = r0; iv <= r1; ++iv) {
+                    if (iv == f0 && f0 <= f1) { // already counted
+                        iv = f1;
+                        continue;
+                    }
+                    const float iw = s_invv[iv];
+                    const float s0 = tau_zplane(z0, iw, G.tc), s1 = tau_zplane(z1, iw, G.tc);
+                    const float lo = fmaxf(ta, fminf(s0, s1)), hi = fminf(tb, fmaxf(s0, s1));
+                    if (hi > lo) a = fmaf(__ldg(col + iv * G.nu).y, hi - lo, a);
+                }
+                acc[z] = a;
+                lo_p = lo_n;
+                hi_p = hi_n;
             }
+        }
+    };
+
+    __syncthreads();
+    if (ok && FLAT) {
+        // (the lane's list goes on across all views of its slice)
+        int k = slice - slices, iu = 0, iu_hi = -1;
+        for (;;) {
+            while (iu > iu_hi && k < G.nviews) // next view with a non-empty shadow
+                if ((k += slices) < G.nviews) shadow(k, iu, iu_hi);
+            if (k >= G.nviews) break;
+            visit(k, iu++);
+        }
+    } else if (ok) {
+        for (int k = slice; k < G.nviews; k += slices) {
+            int lo, hi;
+            shadow(k, lo, hi);
+            for (int iu = lo; iu <= hi; ++iu) visit(k, iu);
         }
     }
 
+    // the slices' sums, in the slices' order
+    if (slices > 1) {
+        const int per = npatch * 32, at = patch * 32 + lane;
+        if (slice > 0)
+#pragma unroll
+            for (int z = 0; z < ZC; ++z)
+                s_sum[((slice - 1) * ZC + z) * per + at] = acc[z];
+        __syncthreads();
+        if (slice == 0)
+            for (int q = 0; q + 1 < slices; ++q)
+#pragma unroll
+                for (int z = 0; z < ZC; ++z)
+                    acc[z] += s_sum[(q * ZC + z) * per + at];
+    }
     double red = 0.0;
-    if (ok) {
+    if (ok && slice == 0) {
         const long long base = (long long)ix * sx + (long long)iy * sy;
 #pragma unroll
         for (int z = 0; z < ZC; ++z) {
-            if (iz0 + z < G.nz) {
+            if (iz0 + z >= iz_own && iz0 + z < G.nz) {
                 const long long o = base + (long long)(iz0 + z) * sz;
                 out[o] = acc[z];
                 if (out2) out2[o] = acc[z];
@@ -357,40 +371,55 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
         __syncthreads();
         if (tid == 0) {
             double t = 0.0;
-            for (int w = 0; w < NT / 32; ++w) t += s_warp[w];
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_warp[w];
             partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = t;
         }
     }
 }
 
+static const void *bp_kernel(int zc, bool flat)
+{
+    switch (zc) {
+    case 18: return flat ? (const void *)&k_backproject<18, true> : (const void *)&k_backproject<18, false>;
+    case 16: return flat ? (const void *)&k_backproject<16, true> : (const void *)&k_backproject<16, false>;
+    case 14: return flat ? (const void *)&k_backproject<14, true> : (const void *)&k_backproject<14, false>;
+    case 12: return flat ? (const void *)&k_backproject<12, true> : (const void *)&k_backproject<12, false>;
+    default: return flat ? (const void *)&k_backproject<8, true> : (const void *)&k_backproject<8, false>;
+    }
+}
+
+// The shared-memory opt-in of every instantiation, once per device: at most 33 KB of rows (nv <= 8192)
+// and 34 KB of the slices' sums (7/8 of 512 threads, 18 voxels).
+cbct_status backproject_prepare()
+{
+    static std::atomic<unsigned long long> done[sizeof(BP_ZC) / sizeof(int)][2];
+    for (int i = 0; i < (int)(sizeof(BP_ZC) / sizeof(int)); ++i)
+        for (int flat = 0; flat < 2; ++flat) {
+            const cudaError_t e = smem_optin_once(bp_kernel(BP_ZC[i], flat != 0), 72 * 1024, done[i][flat]);
+            if (e != cudaSuccess) return check_cuda(e, "backproject attribute");
+        }
+    return CBCT_OK;
+}
+
 cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, long long sx, long long sy,
                                long long sz, float *out2, double *partials, cudaStream_t st)
 {
-    const int zc = bp_zchunk(G);
-    const int nt = bp_threads(zc);
-    const int by = nt == BP_BIG_THREADS ? bp_by<BP_BIG_THREADS>() : BP_BY;
-    dim3 block(nt);
-    dim3 grid((G.nx + BP_BX - 1) / BP_BX, (G.ny + by - 1) / by, (G.nz + zc - 1) / zc);
-    const size_t smem = sizeof(float) * G.nv;
-    const int isx = (int)sx, isy = (int)sy, isz = (int)sz;
-    ProfToken tok = prof_start(CBCT_KERNEL_BACKPROJECT, st);
+    BpPlan p = bp_plan(G);
     // flatten the candidate loop where a voxel column's shadow spans about one imager
     // column (its diagonal, magnified at the rotation axis, below 1.5 pixels)
     const bool flat = sqrtf(G.dx * G.dx + G.dy * G.dy) * (G.sdd / G.sad) < 1.5f * G.du;
-#define CBCT_BP_LAUNCH(Z, NT)                                                                                    \
-    if (flat) k_backproject<Z, true, NT><<<grid, block, smem, st>>>(G, ps, out, isx, isy, isz, out2, partials);    \
-    else k_backproject<Z, false, NT><<<grid, block, smem, st>>>(G, ps, out, isx, isy, isz, out2, partials)
-    switch (zc) {
-    case 16: CBCT_BP_LAUNCH(16, BP_BIG_THREADS); break;
-    case 8: CBCT_BP_LAUNCH(8, BP_THREADS); break;
-    case 4: CBCT_BP_LAUNCH(4, BP_THREADS); break;
-    case 2: CBCT_BP_LAUNCH(2, BP_THREADS); break;
-    default: CBCT_BP_LAUNCH(1, BP_THREADS); break;
-    }
-#undef CBCT_BP_LAUNCH
+    const cbct_status r = backproject_prepare();
+    if (r != CBCT_OK) return r;
+    const size_t smem = sizeof(float) * ((size_t)G.nv + 1 + (size_t)(p.slices - 1) * p.zc * (p.warps / p.slices) * 32);
+    GeomDev g = G;
+    int isx = (int)sx, isy = (int)sy, isz = (int)sz;
+    void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials};
+    ProfToken tok = prof_start(CBCT_KERNEL_BACKPROJECT, st);
+    const cudaError_t e = cudaLaunchKernel(bp_kernel(p.zc, flat), p.grid, dim3(32u * p.warps), args, smem, st);
     prof_stop(tok, st);
     note_launch();
-    return check_cuda(cudaGetLastError(), "backproject launch");
+    if (e != cudaSuccess) cudaGetLastError(); // the error is returned, not left pending
+    return check_cuda(e, "backproject launch");
 }
 
 // Prefix sums over imager rows of every (view k, imager column iu), stored row-major like

@@ -81,6 +81,15 @@ __device__ __forceinline__ float imager_v(const GeomDev &G, int iv) { return fma
 __device__ __forceinline__ int ceil_small(float x) { return __float_as_int(__fadd_ru(x, 12582912.0f)) - 0x4B400000; }
 __device__ __forceinline__ int floor_small(float x) { return __float_as_int(__fadd_rd(x, 12582912.0f)) - 0x4B400000; }
 
+// Shared memory by 32-bit address.
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ float lds_float(unsigned a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
 // Length of ray (d) per unit tau: |D - S|.
 __device__ __forceinline__ float ray_length(float dxr, float dyr, float v)
 {
@@ -120,7 +129,7 @@ static inline size_t storage_bytes(int storage) { return storage == ST_F32 ? 4 :
 // Opts a kernel into more than 48 KB of dynamic shared memory. The attribute belongs to
 // the function on one device, so it is set once per device (`done` holds one bit each).
 template <typename Kernel>
-inline cudaError_t smem_optin_once(Kernel *fn, int bytes, std::atomic<unsigned long long> &done)
+inline cudaError_t smem_optin_once(Kernel fn, int bytes, std::atomic<unsigned long long> &done)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -214,8 +223,9 @@ int backproject_num_blocks(const GeomDev &G);
 // Upper bound of backproject_num_blocks over every grid no larger than G's (any z chunk).
 int backproject_max_blocks(const GeomDev &G);
 // ps: per-(view, imager column) prefix sums over rows of the |D - S|-weighted stack,
-// [n_views][nv + 1][nu] float2 (prefix of the rows below m, value of row m), built by
-// launch_row_prefix.
+// [n_views][nv + 1][nu] float2 (prefix of the rows below m, value of row m), prefix_table_bytes(G)
+// bytes, built by launch_row_prefix.
+size_t prefix_table_bytes(const GeomDev &G);
 cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, long long sx,
                                long long sy, long long sz, float *out2, double *partials,
                                cudaStream_t st);
@@ -301,5 +311,6 @@ void reconstruct_cursor_destroy(ReconCursor *c);
 // Sets every kernel attribute the launchers would otherwise set on first use (shared
 // memory opt-ins) on the current device, so that later launches can be graph-captured.
 cbct_status project_prepare();
+cbct_status backproject_prepare();
 cbct_status tf_prepare();
 }

@@ -8,6 +8,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "async.cuh"
 #include "project.cuh"
 
 namespace cbct {
@@ -199,11 +200,7 @@ cbct_status project_prepare()
     return CBCT_OK;
 }
 
-// cuTensorMapEncodeTiled, from the driver the runtime has loaded (no link to libcuda).
-using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static EncodeTiled encode_tiled()
+EncodeTiled encode_tiled()
 {
     static const EncodeTiled fn = [] {
         void *p = nullptr;

@@ -28,6 +28,7 @@
 // This header holds the kernel template; it is instantiated for each QW in the
 // project_q*.cu units (compiled in parallel) and launched from project.cu.
 #pragma once
+#include "async.cuh"
 #include "project.cuh"
 
 namespace cbct {
@@ -71,60 +72,7 @@ __device__ __forceinline__ f32x2 lds_pair(unsigned a)
     asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ float2 lds_float2(unsigned a)
-{
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float lds_float(unsigned a)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
 
-// Bulk (TMA) copies into shared memory complete on mbarriers; the consumers give a buffer
-// back on another.
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar)
-{
-    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
-}
-// one try: suspends the thread for up to about a millisecond while the phase is incomplete
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned parity)
-{
-    unsigned ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok)
-                 : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u)
-                 : "memory");
-    return ok != 0;
-}
-// Every wait ends: after PROJ_WAIT_CYCLES (about two seconds), or once another warp of the
-// block has given up, it returns false, and the block then ends with NaN results and bit 1
-// of the iteration's status word instead of a hang.
-constexpr long long PROJ_WAIT_CYCLES = 4000000000ll;
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, volatile int *give_up)
-{
-    bool ok = mbar_try_wait(bar, parity);
-    if (!ok) {
-        const long long t0 = clock64();
-        while (!(ok = mbar_try_wait(bar, parity)) && !*give_up)
-            if (clock64() - t0 > PROJ_WAIT_CYCLES) *give_up = 1;
-    }
-    __syncwarp();
-    return ok;
-}
 // The transverse ray shared by every row of imager column iu in a view, and the tau
 // interval in which it crosses the volume's (x, y) footprint.
 struct ColumnRay {
@@ -272,8 +220,6 @@ __device__ __forceinline__ void copies_arrive(unsigned long long *bar)
 {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
-// generic accesses of this thread to shared memory before, bulk copies into it after
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 // barrier of the n consumer threads that also tells whether any of them passed `v`
 __device__ __forceinline__ bool consumer_or(bool v, int n)
 {

@@ -343,8 +343,6 @@ struct Work {
     Scalars *sc;
 };
 
-static size_t prefix_elems(const cbct_geometry_desc &d) { return (size_t)d.n_views * d.nu * ((size_t)d.nv + 1); }
-
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 static size_t max_partials(const cbct_geometry *g)
@@ -370,7 +368,7 @@ static size_t work_layout(const cbct_geometry *g, char *base, Work *w)
     float *X = (float *)take(VB), *X2 = (float *)take(VB), *P = (float *)take(VB), *S = (float *)take(VB);
     float *Fa = (float *)take(VB), *Fb = (float *)take(VB);
     void *R = take(4 * M), *Q = take(4 * M); // sized for FP32, the widest storage type
-    float2 *PS = (float2 *)take(sizeof(float2) * prefix_elems(d));
+    float2 *PS = (float2 *)take(prefix_table_bytes(level_geom(g, 0)));
     void *TR[MAX_LEVELS];
     for (int lev = 0; lev < MAX_LEVELS; ++lev) TR[lev] = take(trace_table_bytes(level_geom(g, lev)));
     double *partials = (double *)take(sizeof(double) * max_partials(g));
@@ -672,7 +670,7 @@ extern "C" cbct_status cbct_backproject_ex(const cbct_geometry *gc, const void *
     if (!valid_dtype(g_type)) return set_error(CBCT_ERR_INVALID_ARG, "backproject: unknown storage type %d", (int)g_type);
     cbct_geometry *g = const_cast<cbct_geometry *>(gc);
     const GeomDev G = level_geom(g, 0);
-    TRY(ensure_scratch(g, sizeof(float2) * prefix_elems(g->desc)));
+    TRY(ensure_scratch(g, prefix_table_bytes(G)));
     cudaStream_t st = (cudaStream_t)stream;
     float2 *ps = reinterpret_cast<float2 *>(g->d_scratch);
     TRY(launch_row_prefix(G, gin, ps, 1, st, (int)g_type));

@@ -484,6 +484,7 @@ extern "C" cbct_status cbct_server_create(const cbct_server_opts *opts, cbct_ser
                                                        : N_CLASSES;
     // kernels' shared-memory opt-ins, so that nothing is set while a stream is captured
     SRV_TRY(project_prepare());
+    SRV_TRY(backproject_prepare());
     SRV_TRY(tf_prepare());
     cudaMemPoolProps props;
     std::memset(&props, 0, sizeof(props));
