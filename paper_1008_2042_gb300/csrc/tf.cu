@@ -470,118 +470,192 @@ namespace cbct {
 // The 27 coefficients never leave the SM: HBM traffic is one read of x (halo re-reads hit
 // L2) and the writes of f_new (and v, with one read of f_old).
 //
-// A warp covers 32 consecutive positions of one row along axis 0: the 28 output positions
-// of its tile and two halo positions on either side (the coefficients of the outputs'
-// neighbours need x one position further out). A block stacks FR_ROWS + 4 such warps along
-// axis 1 (its output rows, the two rows of coefficients around them and the two rows of x
-// those need) and marches along axis 2. Per plane every lane
+// A warp covers 32 consecutive positions along axis 0 (28 outputs and two halo positions on
+// either side: the coefficients of the outputs' neighbours need x one position further out)
+// of two adjacent rows, whose values a lane holds as pairs and treats with one instruction
+// (fma.rn.f32x2 and its kind: each half rounds like the scalar operation). A block stacks
+// FR_WARPS such pairs along axis 1, the first and last of them halo rows, and marches along
+// axis 2. Per plane every lane
 //   1. analyses along axis 2 from the three x planes it holds in registers (the next plane
 //      is loaded while this one is computed),
-//   2. along axis 1 from its neighbour rows' values through shared memory,
-//   3. along axis 0 from its neighbour lanes by shuffles, giving its position's 27
+//   2. along axis 1: each row's neighbour is the pair's other row or, through shared memory,
+//      the adjacent warp's near row,
+//   3. along axis 0 from its neighbour lanes by shuffles, giving its positions' 27
 //      coefficients, which it shrinks in registers (Eq. (2)),
 // and then synthesises back as the shrink + synthesis kernel does: shares of neighbouring
-// lanes by shuffles, of neighbouring rows through shared memory, of neighbouring planes in
-// registers, finishing the output plane one behind the analysed one.
+// lanes by shuffles, of neighbouring rows within the pair or through shared memory, of
+// neighbouring planes in registers, finishing the output plane one behind the analysed one.
+//
+// Bound by instruction issue (57%), the packed-FP32 pipe and the shuffles; 16 warps (118
+// registers) per SM. 512x512x70: 334 us (one row per warp, 22 warps: 377 us), z-fastest as in
+// the iteration 363 us (421 us); 12 warps with more registers 484 us.
 // ------------------------------------------------------------------------------------
-// Output rows per block along axis 1. Each block recomputes the coefficients of two halo
-// rows, so taller blocks waste less; one block of 22 warps per SM (80 registers, 47.6 KB of
-// shared memory) measured 0.418 ms on the iteration's 512x512x70 grid against 0.471 ms for two
-// blocks of 6 rows (10 warps each).
-#ifndef CBCT_FR_ROWS
-#define CBCT_FR_ROWS 18
-#endif
-constexpr int FR_ROWS = CBCT_FR_ROWS;
-constexpr int FR_OUT = 28;                       // output positions per warp along axis 0
-constexpr int FR_WARPS = FR_ROWS + 4;
+constexpr int FR_WARPS = 16;
+constexpr int FR_ROWS = 2 * FR_WARPS - 4; // output rows per block along axis 1
+constexpr int FR_OUT = 28;                // output positions per warp along axis 0
 constexpr int FR_THREADS = 32 * FR_WARPS;
 
-__global__ void __launch_bounds__(FR_THREADS, FR_THREADS <= 320 ? 2 : 1)
+// Two FP32 values in one 64-bit register: .x the even row's, .y the odd row's.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pk(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return b;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 splat(float v) { return pk(v, v); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, splat(-1.0f), a); } // a - b, rounded once
+
+// The frame with plain taps: [1, 2, 1], [1, 0, -1] and [1, -2, 1] stand for 4 h_0, (4 / sqrt(2)) h_1
+// and -4 h_2, so that a triple takes four operations. A coefficient with j factors h_1 is then 64 /
+// sqrt(2)^j times the frame's (its sign is its own on both ways), the squared norm is the sum of
+// 2^j A^2 over 4096, and synthesis counts the middle tap triple twice and divides by 4096: all
+// powers of two, which round nothing.
+__device__ __forceinline__ void ana3_plain(f32x2 p, f32x2 c, f32x2 n, f32x2 &o0, f32x2 &o1, f32x2 &o2)
+{
+    const f32x2 s = add2(n, p);
+    o0 = fma2(splat(2.0f), c, s);
+    o1 = sub2(n, p);
+    o2 = fma2(splat(-2.0f), c, s);
+}
+// shares of a triple: to p + 1, half of that to p itself, to p - 1
+__device__ __forceinline__ void syn_shares_plain(f32x2 a0, f32x2 a1, f32x2 a2, f32x2 &up, f32x2 &half, f32x2 &dn)
+{
+    const f32x2 q = add2(a0, a2);
+    up = fma2(splat(2.0f), a1, q);
+    dn = fma2(splat(-2.0f), a1, q);
+    half = sub2(a0, a2);
+}
+
+__global__ void __launch_bounds__(FR_THREADS, 1)
 k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__restrict__ x, float mu, int positivity,
                   float *__restrict__ fnew, const float *__restrict__ fold, float coef, float *__restrict__ vout)
 {
-    __shared__ float s_t[2][FR_WARPS][3][32];              // axis-2 analysis of each row
-    __shared__ float s_up[2][FR_ROWS + 2][3][32], s_dn[2][FR_ROWS + 2][3][32]; // axis-1 synthesis shares
+    __shared__ f32x2 s_t[2][FR_WARPS][3][32];                      // axis-2 analysis of each pair
+    __shared__ float s_up[2][FR_WARPS][3][32], s_dn[2][FR_WARPS][3][32]; // axis-1 synthesis shares to the pairs beside
     const int lane = threadIdx.x, w = threadIdx.y;
     const int a_out = blockIdx.x * FR_OUT, b_out = blockIdx.y * FR_ROWS;
     const int c_begin = blockIdx.z * chunk;
     const int c_end = min(n2, c_begin + chunk);
     if (c_begin >= c_end) return;
     const size_t plane = (size_t)p0 * n1;
-    const int pa = a_out + lane - 2, pb = b_out + w - 2;  // this lane's position (unwrapped)
-    const size_t inplane = (size_t)wrapi(pb, n1) * p0 + wrapi(pa, n0);
-    const bool coef_row = w >= 1 && w <= FR_ROWS + 2;     // rows whose coefficients are formed
-    const bool out_row = w >= 2 && w <= FR_ROWS + 1 && pb < n1;
+    const int pa = a_out + lane - 2, pb = b_out + 2 * w - 2;  // this lane's position and first row (unwrapped)
+    const size_t in0 = (size_t)wrapi(pb, n1) * p0 + wrapi(pa, n0), in1 = (size_t)wrapi(pb + 1, n1) * p0 + wrapi(pa, n0);
+    const bool out_pair = w >= 1 && w <= FR_WARPS - 2 && pb < n1;
     const bool out_lane = lane >= 2 && lane < 2 + FR_OUT && pa < n0;
-    const float *src = x + inplane;
+    const int wu = w > 0 ? w - 1 : 0, wd = w < FR_WARPS - 1 ? w + 1 : w; // (the outermost halo rows' coefficients are not used)
+    auto load = [&](int c) {
+        const float *src = x + (size_t)wrapi(c, n2) * plane;
+        return pk(__ldg(src + in0), __ldg(src + in1));
+    };
 
-    // x of this position at planes cp - 1, cp, cp + 1 (cp: the analysed plane)
-    float xm = __ldg(src + (size_t)wrapi(c_begin - 2, n2) * plane);
-    float x0 = __ldg(src + (size_t)wrapi(c_begin - 1, n2) * plane);
-    float xp = __ldg(src + (size_t)wrapi(c_begin, n2) * plane);
-    float w_m2[3] = {0.f, 0.f, 0.f}, w_m1[3] = {0.f, 0.f, 0.f}; // axis-2 synthesis inputs at cp-2, cp-1
+    // x of these positions at planes cp - 1, cp, cp + 1 (cp: the analysed plane)
+    f32x2 xm = load(c_begin - 2), x0 = load(c_begin - 1), xp = load(c_begin);
+    f32x2 w_m2[3] = {0ull, 0ull, 0ull}, w_m1[3] = {0ull, 0ull, 0ull}; // axis-2 synthesis inputs at cp-2, cp-1
     int buf = 0;
     for (int cp = c_begin - 1; cp <= c_end; ++cp, buf ^= 1) {
-        const float xn = cp < c_end ? __ldg(src + (size_t)wrapi(cp + 2, n2) * plane) : 0.0f;
+        const f32x2 xn = cp < c_end ? load(cp + 2) : 0ull;
         // 1. analysis along axis 2
-        float t[3];
-        ana3(xm, x0, xp, t[0], t[1], t[2]);
+        f32x2 t[3];
+        ana3_plain(xm, x0, xp, t[0], t[1], t[2]);
 #pragma unroll
         for (int n = 0; n < 3; ++n) s_t[buf][w][n][lane] = t[n];
         __syncthreads();
-        float midn[3] = {0.f, 0.f, 0.f};
-        if (coef_row) { // warp-uniform
-            // 2. along axis 1: u[m][n]
-            float u[3][3];
+        // 2. along axis 1: u[m][n]
+        f32x2 u[3][3];
 #pragma unroll
-            for (int n = 0; n < 3; ++n)
-                ana3(s_t[buf][w - 1][n][lane], t[n], s_t[buf][w + 1][n][lane], u[0][n], u[1][n], u[2][n]);
-            // 3. along axis 0: alpha[l + 3m + 9n]
-            float al[27];
+        for (int n = 0; n < 3; ++n) {
+            const float above = hi2(s_t[buf][wu][n][lane]), below = lo2(s_t[buf][wd][n][lane]);
+            ana3_plain(pk(above, lo2(t[n])), t[n], pk(hi2(t[n]), below), u[0][n], u[1][n], u[2][n]);
+        }
+        // 3. along axis 0: alpha[l + 3m + 9n]
+        f32x2 al[27];
 #pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int n = 0; n < 3; ++n) {
-                    const float pv = __shfl_up_sync(0xffffffffu, u[m][n], 1);
-                    const float nv = __shfl_down_sync(0xffffffffu, u[m][n], 1);
-                    ana3(pv, u[m][n], nv, al[3 * m + 9 * n], al[1 + 3 * m + 9 * n], al[2 + 3 * m + 9 * n]);
-                }
-            // vector shrinkage, Eq. (2)
-            float s2 = 0.0f;
-#pragma unroll
-            for (int ch = 1; ch < 27; ++ch) s2 = fmaf(al[ch], al[ch], s2);
-            const float nrm = sqrtf(s2);
-            const float scale = nrm > mu ? 1.0f - mu / nrm : 0.0f;
-#pragma unroll
-            for (int ch = 1; ch < 27; ++ch) al[ch] *= scale;
-            // synthesis along axis 0 (lanes), then the shares along axis 1
-            float us[9];
-#pragma unroll
-            for (int mn = 0; mn < 9; ++mn) {
-                float up, mid, dn;
-                syn_shares(al[3 * mn], al[3 * mn + 1], al[3 * mn + 2], up, mid, dn);
-                us[mn] = __shfl_up_sync(0xffffffffu, up, 1) + mid + __shfl_down_sync(0xffffffffu, dn, 1);
-            }
+        for (int m = 0; m < 3; ++m)
 #pragma unroll
             for (int n = 0; n < 3; ++n) {
-                float up, dn;
-                syn_shares(us[3 * n], us[3 * n + 1], us[3 * n + 2], up, midn[n], dn);
-                s_up[buf][w - 1][n][lane] = up;
-                s_dn[buf][w - 1][n][lane] = dn;
+                const f32x2 pv = __shfl_up_sync(0xffffffffu, u[m][n], 1);
+                const f32x2 nv = __shfl_down_sync(0xffffffffu, u[m][n], 1);
+                ana3_plain(pv, u[m][n], nv, al[3 * m + 9 * n], al[1 + 3 * m + 9 * n], al[2 + 3 * m + 9 * n]);
             }
+        // vector shrinkage, Eq. (2): squares summed by their number j of factors h_1
+        f32x2 sj[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+        for (int ch = 1; ch < 27; ++ch) {
+            const int j = (ch % 3 == 1) + (ch / 3 % 3 == 1) + (ch / 9 == 1);
+            sj[j] = fma2(al[ch], al[ch], sj[j]);
+        }
+        const f32x2 s2 = fma2(splat(2.0f), fma2(splat(2.0f), fma2(splat(2.0f), sj[3], sj[2]), sj[1]), sj[0]);
+        const float na = sqrtf(lo2(s2)), nb = sqrtf(hi2(s2)), mu64 = 64.0f * mu;
+        const f32x2 scale = pk(na > mu64 ? 1.0f - mu64 / na : 0.0f, nb > mu64 ? 1.0f - mu64 / nb : 0.0f);
+#pragma unroll
+        for (int ch = 1; ch < 27; ++ch) al[ch] = mul2(al[ch], scale);
+        // synthesis along axis 0 (lanes), then the shares along axis 1
+        f32x2 us[9];
+#pragma unroll
+        for (int mn = 0; mn < 9; ++mn) {
+            f32x2 up, half, dn;
+            syn_shares_plain(al[3 * mn], al[3 * mn + 1], al[3 * mn + 2], up, half, dn);
+            us[mn] = add2(fma2(splat(2.0f), half, __shfl_up_sync(0xffffffffu, up, 1)), __shfl_down_sync(0xffffffffu, dn, 1));
+        }
+        f32x2 up[3], half[3], dn[3];
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {
+            syn_shares_plain(us[3 * n], us[3 * n + 1], us[3 * n + 2], up[n], half[n], dn[n]);
+            s_up[buf][w][n][lane] = hi2(up[n]);
+            s_dn[buf][w][n][lane] = lo2(dn[n]);
         }
         __syncthreads();
-        if (out_row) {
-            float wv[3];
+        if (out_pair) {
+            f32x2 wv[3];
 #pragma unroll
-            for (int n = 0; n < 3; ++n) wv[n] = s_up[buf][w - 2][n][lane] + midn[n] + s_dn[buf][w][n][lane];
+            for (int n = 0; n < 3; ++n)
+                wv[n] = add2(fma2(splat(2.0f), half[n], pk(s_up[buf][wu][n][lane], lo2(up[n]))),
+                             pk(hi2(dn[n]), s_dn[buf][wd][n][lane]));
             // synthesis along axis 2: plane cp - 1 from planes cp - 2, cp - 1, cp
             if (cp >= c_begin + 1 && out_lane) {
-                float o = syn3(w_m2[0], w_m1[0], wv[0], w_m2[1], wv[1], w_m2[2], w_m1[2], wv[2]);
-                if (positivity && o < 0.0f) o = 0.0f;
                 const size_t idx = (size_t)(cp - 1) * plane + (size_t)pb * p0 + pa;
-                fnew[idx] = o;
-                if (vout) vout[idx] = fmaf(coef, o - __ldg(fold + idx), o);
+                const f32x2 ends = add2(add2(w_m2[0], w_m2[2]), add2(wv[0], wv[2]));
+                const f32x2 o2 = fma2(splat(2.0f), add2(sub2(w_m1[0], w_m1[2]), sub2(w_m2[1], wv[1])), ends);
+                float o[2] = {lo2(o2) * (1.0f / 4096.0f), hi2(o2) * (1.0f / 4096.0f)};
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (pb + r >= n1) break; // an odd number of rows
+                    if (positivity && o[r] < 0.0f) o[r] = 0.0f;
+                    const size_t at = idx + (size_t)r * p0;
+                    fnew[at] = o[r];
+                    if (vout) vout[at] = fmaf(coef, o[r] - __ldg(fold + at), o[r]);
+                }
             }
 #pragma unroll
             for (int n = 0; n < 3; ++n) {
