@@ -92,12 +92,6 @@ int backproject_max_blocks(const GeomDev &G)
     return ((G.nx + 2 * BP_WX - 1) / (2 * BP_WX)) * ((G.ny + BP_WY - 1) / BP_WY) * ((G.nz + BP_ZC[0] - 1) / BP_ZC[0]);
 }
 
-int backproject_num_blocks(const GeomDev &G)
-{
-    const BpPlan p = bp_plan(G);
-    return (int)(p.grid.x * p.grid.y * p.grid.z);
-}
-
 // Rows whose ray, while inside the column (tau in [ta, tb], 1/(tc+ta) = A, 1/(tc+tb) = B),
 // reaches the plane z = zp: v (tc + tau) = zp for some tau, i.e. v between zp*A and zp*B.
 // Returned as a widened integer row range (may extend outside [0, nv-1]).
@@ -192,7 +186,7 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
 template <int ZC, bool FLAT>
 __global__ void __launch_bounds__(32 * BP_MAX_WARPS, 2)
 k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz, int slices,
-              float *__restrict__ out2, double *__restrict__ partials)
+              float *__restrict__ out2, double *__restrict__ partials, Scalars *__restrict__ sc, int fin_op, int scale_q)
 {
     extern __shared__ float smem[]; // 1 / v per imager row (one more for entry nv); then the slices' sums
     __shared__ double s_warp[BP_MAX_WARPS];
@@ -369,10 +363,25 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
         for (int o = 16; o > 0; o >>= 1) red += __shfl_down_sync(0xffffffffu, red, o);
         if ((tid & 31) == 0) s_warp[tid >> 5] = red;
         __syncthreads();
+        const unsigned blocks = gridDim.x * gridDim.y * gridDim.z;
+        bool last = false;
         if (tid == 0) {
             double t = 0.0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_warp[w];
             partials[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = t;
+            last = last_to_arrive(sc, blocks);
+        }
+        if (__syncthreads_or(last)) {
+            double t = sum_partials(partials, blocks, tid, blockDim.x);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if ((tid & 31) == 0) s_warp[tid >> 5] = t;
+            __syncthreads();
+            if (tid == 0) {
+                double sum = 0.0;
+                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += s_warp[w];
+                apply_sum(sc, sum, fin_op, scale_q);
+            }
         }
     }
 }
@@ -402,7 +411,8 @@ cbct_status backproject_prepare()
 }
 
 cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, long long sx, long long sy,
-                               long long sz, float *out2, double *partials, cudaStream_t st)
+                               long long sz, float *out2, double *partials, cudaStream_t st, Scalars *sc, int fin_op,
+                               int scale_q)
 {
     BpPlan p = bp_plan(G);
     // flatten the candidate loop where a voxel column's shadow spans about one imager
@@ -413,7 +423,7 @@ cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, l
     const size_t smem = sizeof(float) * ((size_t)G.nv + 1 + (size_t)(p.slices - 1) * p.zc * (p.warps / p.slices) * 32);
     GeomDev g = G;
     int isx = (int)sx, isy = (int)sy, isz = (int)sz;
-    void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials};
+    void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials, &sc, &fin_op, &scale_q};
     ProfToken tok = prof_start(CBCT_KERNEL_BACKPROJECT, st);
     const cudaError_t e = cudaLaunchKernel(bp_kernel(p.zc, flat), p.grid, dim3(32u * p.warps), args, smem, st);
     prof_stop(tok, st);
@@ -444,9 +454,11 @@ __device__ __forceinline__ void comp_add(float &s, float &c, float v)
     s = t;
 }
 
-template <typename T>
+// UPDATE: g is the CGLS residual r and first becomes r - alpha q (q stored as kappa q; FP32
+// arithmetic, one rounding to the storage type), which saves a pass over r and q of its own.
+template <typename T, bool UPDATE>
 __global__ void __launch_bounds__(32 * PREFIX_WARPS)
-k_row_prefix(GeomDev G, const T *__restrict__ g, float2 *__restrict__ ps, int prescale)
+k_row_prefix(GeomDev G, T *g, const T *__restrict__ q, const Scalars *__restrict__ sc, float2 *__restrict__ ps, int prescale)
 {
     __shared__ float2 s_tot[PREFIX_WARPS][32];
     const int lane = threadIdx.x, w = threadIdx.y;
@@ -460,13 +472,30 @@ k_row_prefix(GeomDev G, const T *__restrict__ g, float2 *__restrict__ ps, int pr
         dxr = r4.x;
         dyr = r4.y;
     }
-    const T *src = g + (size_t)k * G.nv * G.nu + iu;
+    const float step = UPDATE ? (float)(sc->alpha / sc->kappa) : 0.0f;
+    const size_t first = (size_t)k * G.nv * G.nu + iu;
+    T *src = g + first;
     float ts = 0.0f, tc = 0.0f;
     if (ok)
-        for (int iv = r0; iv < r1; ++iv) {
-            float val = load_as_float(src + (size_t)iv * G.nu);
-            if (prescale) val *= ray_length(dxr, dyr, imager_v(G, iv));
-            comp_add(ts, tc, val);
+        for (int i0 = r0; i0 < r1; i0 += 4) { // four rows at a time: their loads go out together
+            float val[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const size_t at = (size_t)min(i0 + i, r1 - 1) * G.nu;
+                val[i] = UPDATE ? as_float(src[at]) : load_as_float(src + at);
+                if (UPDATE) val[i] = fmaf(-step, load_as_float(q + first + at), val[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i0 + i >= r1) break;
+                if (UPDATE) {
+                    T *at = src + (size_t)(i0 + i) * G.nu;
+                    store_from_float(at, val[i]);
+                    val[i] = as_float(*at);
+                }
+                if (prescale) val[i] *= ray_length(dxr, dyr, imager_v(G, i0 + i));
+                comp_add(ts, tc, val[i]);
+            }
         }
     s_tot[w][lane] = make_float2(ts, tc);
     __syncthreads();
@@ -478,8 +507,9 @@ k_row_prefix(GeomDev G, const T *__restrict__ g, float2 *__restrict__ ps, int pr
     }
     if (!ok) return;
     float2 *dst = ps + (size_t)k * ((size_t)G.nv + 1) * G.nu + iu; // entry m at dst[m * nu]
+#pragma unroll 4
     for (int iv = r0; iv < r1; ++iv) {
-        float val = load_as_float(src + (size_t)iv * G.nu);
+        float val = UPDATE ? as_float(src[(size_t)iv * G.nu]) : load_as_float(src + (size_t)iv * G.nu);
         if (prescale) val *= ray_length(dxr, dyr, imager_v(G, iv));
         dst[(size_t)iv * G.nu] = make_float2(rs + rc, val);
         comp_add(rs, rc, val);
@@ -487,19 +517,30 @@ k_row_prefix(GeomDev G, const T *__restrict__ g, float2 *__restrict__ ps, int pr
     if (w == PREFIX_WARPS - 1) dst[(size_t)G.nv * G.nu] = make_float2(rs + rc, 0.0f); // all rows
 }
 
-cbct_status launch_row_prefix(const GeomDev &G, const void *g, float2 *ps, int prescale, cudaStream_t st, int storage)
+template <typename T>
+static void row_prefix(const GeomDev &G, void *g, const void *q, const Scalars *sc, float2 *ps, int prescale, cudaStream_t st)
 {
-    dim3 grid((G.nu + 31) / 32, G.nviews), block(32, PREFIX_WARPS);
-    if (storage == ST_BF16)
+    const dim3 grid((G.nu + 31) / 32, G.nviews), block(32, PREFIX_WARPS);
+    if (q)
         CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_row_prefix<__nv_bfloat16><<<grid, block, 0, st>>>(G, static_cast<const __nv_bfloat16 *>(g), ps, prescale));
-    else if (storage == ST_F16)
-        CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_row_prefix<__half><<<grid, block, 0, st>>>(G, static_cast<const __half *>(g), ps, prescale));
+                   k_row_prefix<T, true><<<grid, block, 0, st>>>(G, static_cast<T *>(g), static_cast<const T *>(q), sc, ps, prescale));
     else
         CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_row_prefix<float><<<grid, block, 0, st>>>(G, static_cast<const float *>(g), ps, prescale));
+                   k_row_prefix<T, false><<<grid, block, 0, st>>>(G, static_cast<T *>(g), nullptr, nullptr, ps, prescale));
+}
+
+cbct_status launch_update_prefix(const GeomDev &G, void *r, const void *q, const Scalars *sc, float2 *ps, int prescale,
+                                 cudaStream_t st, int storage)
+{
+    if (storage == ST_BF16) row_prefix<__nv_bfloat16>(G, r, q, sc, ps, prescale, st);
+    else if (storage == ST_F16) row_prefix<__half>(G, r, q, sc, ps, prescale, st);
+    else row_prefix<float>(G, r, q, sc, ps, prescale, st);
     return check_cuda(cudaGetLastError(), "row prefix launch");
+}
+
+cbct_status launch_row_prefix(const GeomDev &G, const void *g, float2 *ps, int prescale, cudaStream_t st, int storage)
+{
+    return launch_update_prefix(G, const_cast<void *>(g), nullptr, nullptr, ps, prescale, st, storage); // (g is only read)
 }
 
 // The paper's own backprojector, Eq. (3): voxel-driven, for every view the imager value at

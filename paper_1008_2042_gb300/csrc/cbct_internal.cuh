@@ -107,6 +107,9 @@ template <> __device__ __forceinline__ float load_as_float<__nv_bfloat16>(const 
     return __bfloat162float(__ldg(p));
 }
 template <> __device__ __forceinline__ float load_as_float<__half>(const __half *p) { return __half2float(__ldg(p)); }
+__device__ __forceinline__ float as_float(float v) { return v; }
+__device__ __forceinline__ float as_float(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float as_float(__half v) { return __half2float(v); }
 template <typename T> __device__ __forceinline__ void store_from_float(T *p, float v);
 template <> __device__ __forceinline__ void store_from_float<float>(float *p, float v) { *p = v; }
 template <> __device__ __forceinline__ void store_from_float<__nv_bfloat16>(__nv_bfloat16 *p, float v)
@@ -150,10 +153,45 @@ struct Scalars {
     double rr;       // ||r||^2 (monitoring)
     double kappa;    // q is stored as kappa * q, kappa = 1 / sqrt(gamma): keeps FP16 in range
     unsigned int flags; // bit 0: a reduction was not finite; bit 1: a projector block's wait timed out
-    unsigned int pad;
+    unsigned int arrived; // blocks of the running reduction that have written their partial sum (0 between kernels)
 };
 
-enum FinalizeOp { FIN_GAMMA = 0, FIN_ALPHA = 1, FIN_BETA = 2, FIN_RR = 3 };
+// What the sum of a kernel's partials becomes. scale_q: q is about to be stored in FP16, so keep
+// kappa = 1 / sqrt(gamma) (||kappa p|| >= 1 and kappa q stays O(1)); otherwise kappa = 1.
+enum FinalizeOp { FIN_NONE = -1, FIN_GAMMA = 0, FIN_ALPHA = 1, FIN_BETA = 2, FIN_RR = 3 };
+
+// After thread 0 of a block has stored partials[block]: true in the block that is the last of
+// `blocks` to do so (thread 0 only).
+__device__ __forceinline__ bool last_to_arrive(Scalars *sc, unsigned blocks)
+{
+    __threadfence();
+    return atomicAdd(&sc->arrived, 1u) == blocks - 1u;
+}
+// The last block's share: thread t of nthr sums partials t, t + nthr, ... (a fixed order, so the
+// result does not depend on scheduling).
+__device__ __forceinline__ double sum_partials(const double *partials, unsigned n, int t, int nthr)
+{
+    __threadfence();
+    double v = 0.0;
+    for (unsigned i = t; i < n; i += nthr) v += __ldcg(partials + i);
+    return v;
+}
+// Thread 0 of the last block: the scalars of CGLS from the whole sum.
+__device__ __forceinline__ void apply_sum(Scalars *sc, double sum, int op, int scale_q)
+{
+    if (!isfinite(sum)) atomicOr(&sc->flags, 1u);
+    if (op == FIN_GAMMA || op == FIN_BETA) {
+        if (op == FIN_BETA) sc->beta = sc->gamma > 0.0 ? sum / sc->gamma : 0.0;
+        sc->gamma = sum;
+        sc->kappa = (scale_q && sum > 0.0 && isfinite(sum)) ? 1.0 / sqrt(sum) : 1.0;
+    } else if (op == FIN_ALPHA) {
+        sc->delta = sum;
+        sc->alpha = (sc->gamma > 0.0 && sum > 0.0) ? sc->gamma / sum : 0.0;
+    } else {
+        sc->rr = sum;
+    }
+    sc->arrived = 0u;
+}
 
 // Projector epilogues (q = |D - S| * sum of f * dtau is the projection of the ray).
 enum ProjectMode {
@@ -208,29 +246,32 @@ constexpr size_t PROJECT_SMEM_LIMIT = 200 * 1024;
 // padding (PM_PLAIN with FP32 storage only; the same results from narrower loads). traces: the
 // trace table from launch_trace_table (PM_COUNT: none); only the (view, imager column) pairs
 // [col_first, col_first + ncols) are projected, whose records are its first (ncols = 0: all).
-// npartials, when given, receives the number of partial sums written, at most
-// project_num_blocks(G).
+// In the CGLS modes the last block to finish also sums the blocks' partials (at most
+// project_num_blocks(G) of them) into sc: ||y - q||^2 (PM_RESID), ||q||^2 and alpha (PM_Q_SCALED).
 cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const float *y, void *out, int mode,
                            double *partials, float count_thr, cudaStream_t st, int storage, Scalars *sc,
-                           const void *traces, int *npartials = nullptr, int col_first = 0, int ncols = 0);
+                           const void *traces, int col_first = 0, int ncols = 0);
 // The projector's trace table of a grid (trace_table_bytes(G) bytes for all columns, 16-byte
 // aligned): the transverse trace of the (view, imager column) pairs [col_first, col_first + ncols)
 // (ncols = 0: all).
 size_t trace_table_bytes(const GeomDev &G);
 cbct_status launch_trace_table(const GeomDev &G, void *tab, cudaStream_t st, int col_first = 0, int ncols = 0);
 cbct_status trace_table_prepare();
-int backproject_num_blocks(const GeomDev &G);
-// Upper bound of backproject_num_blocks over every grid no larger than G's (any z chunk).
+// Upper bound of the blocks of an adjoint launch over every grid no larger than G's.
 int backproject_max_blocks(const GeomDev &G);
 // ps: per-(view, imager column) prefix sums over rows of the |D - S|-weighted stack,
 // [n_views][nv + 1][nu] float2 (prefix of the rows below m, value of row m), prefix_table_bytes(G)
-// bytes, built by launch_row_prefix.
+// bytes, built by launch_row_prefix. With partials, the last block to finish sums them into sc by
+// fin_op (FinalizeOp).
 size_t prefix_table_bytes(const GeomDev &G);
 cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, long long sx,
                                long long sy, long long sz, float *out2, double *partials,
-                               cudaStream_t st);
+                               cudaStream_t st, Scalars *sc = nullptr, int fin_op = FIN_NONE, int scale_q = 0);
 cbct_status launch_row_prefix(const GeomDev &G, const void *g, float2 *ps, int prescale,
                               cudaStream_t st, int storage = ST_F32);
+// The same of the CGLS residual after its update r -= alpha q, which is written back to r.
+cbct_status launch_update_prefix(const GeomDev &G, void *r, const void *q, const Scalars *sc, float2 *ps, int prescale,
+                                 cudaStream_t st, int storage);
 cbct_status launch_backproject_eq3(const GeomDev &G, const float *g, float *f, float pref,
                                    cudaStream_t st);
 

@@ -229,7 +229,7 @@ static cbct_status line_map(const GeomDev &G, const float *f, int pitch, CUtenso
 
 cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const float *y, void *out, int mode,
                            double *partials, float count_thr, cudaStream_t st, int storage, Scalars *sc,
-                           const void *traces, int *npartials, int col_first, int ncols)
+                           const void *traces, int col_first, int ncols)
 {
     if (project_smem_bytes(G) > PROJECT_SMEM_LIMIT)
         return set_error(CBCT_ERR_UNSUPPORTED, "project: grid too large for the projector's shared memory (nx + ny and nz)");
@@ -259,7 +259,6 @@ cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const f
         if (r != CBCT_OK) return r;
     }
     const int grid = nitems < c.grid ? nitems : c.grid;
-    if (npartials) *npartials = grid;
     GeomDev g = G;
     const float *rec = static_cast<const float *>(traces);
     void *args[] = {&g, &map, &f, &zpitch, &c.plan, &y, &out, &partials, &sc, &rec, &col_first, &ncols, &nitems};

@@ -546,10 +546,24 @@ k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__r
         for (int o = 16; o > 0; o >>= 1) red += __shfl_down_sync(0xffffffffu, red, o);
         if (lane == 0) s_warp[warp] = red;
         consumer_or(false, nthr);
+        bool last = false;
         if (tid == 0) {
             double t = 0.0;
             for (int w = 0; w < nwarps; ++w) t += s_warp[w];
             partials[blockIdx.x] = t;
+            last = last_to_arrive(sc, gridDim.x);
+        }
+        if (consumer_or(last, nthr)) {
+            double t = sum_partials(partials, gridDim.x, tid, nthr);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if (lane == 0) s_warp[warp] = t;
+            consumer_or(false, nthr);
+            if (tid == 0) {
+                double sum = 0.0;
+                for (int w = 0; w < nwarps; ++w) sum += s_warp[w];
+                apply_sum(sc, sum, MODE == PM_RESID ? FIN_RR : FIN_ALPHA, 0);
+            }
         }
     }
 }

@@ -87,7 +87,7 @@ extern "C" cbct_status cbct_project_static(const cbct_geometry *g, const float *
         st = launch_trace_table(G, traces, s, c0, n);
         if (st != CBCT_OK) return st;
         st = launch_project(G, scratch, zpitch, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, s, ST_F32, nullptr, traces,
-                            nullptr, c0, n);
+                            c0, n);
         if (st != CBCT_OK) return st;
     }
     return CBCT_OK;

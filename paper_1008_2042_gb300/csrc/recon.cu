@@ -2,8 +2,8 @@
 // (Section 2.2.3), plus the public entry points that wrap the operators.
 //
 // The whole iteration stays on the device: CGLS inner products are reduced in FP64 into
-// device-resident scalars (one partial per producer block, then one finalising block
-// in a fixed order, so results are deterministic), and the vector updates read their
+// device-resident scalars (one partial per producer block, summed in a fixed order by the
+// producer's last block, so results are deterministic), and the vector updates read their
 // step sizes from there. The host only enqueues kernels; it reads one status word at
 // the end. The A2 momentum coefficients do not depend on the data and are computed on
 // the host.
@@ -21,41 +21,6 @@ namespace cbct {
 // Reductions and vector updates
 // ------------------------------------------------------------------------------------
 
-// scale_q: q is about to be stored in FP16, so keep kappa = 1 / sqrt(gamma) (||kappa p|| >= 1
-// and kappa q stays O(1)); otherwise kappa = 1.
-__global__ void __launch_bounds__(1024) k_finalize(const double *__restrict__ partials, int n,
-                                                   Scalars *sc, int op, int scale_q)
-{
-    __shared__ double s[32];
-    double t = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) t += partials[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += s[w];
-        if (!isfinite(sum)) sc->flags |= 1u;
-        if (op == FIN_GAMMA || op == FIN_BETA) {
-            if (op == FIN_BETA) sc->beta = sc->gamma > 0.0 ? sum / sc->gamma : 0.0;
-            sc->gamma = sum;
-            sc->kappa = (scale_q && sum > 0.0 && isfinite(sum)) ? 1.0 / sqrt(sum) : 1.0;
-        } else if (op == FIN_ALPHA) {
-            sc->delta = sum;
-            sc->alpha = (sc->gamma > 0.0 && sum > 0.0) ? sc->gamma / sum : 0.0;
-        } else {
-            sc->rr = sum;
-        }
-    }
-}
-
-static cbct_status finalize(const double *partials, int n, Scalars *sc, int op, cudaStream_t st, int scale_q = 0)
-{
-    CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_finalize<<<1, 1024, 0, st>>>(partials, n, sc, op, scale_q));
-    return check_cuda(cudaGetLastError(), "finalize launch");
-}
-
 static int vec_blocks(size_t n)
 {
     const size_t per = 256 * 4;
@@ -63,77 +28,6 @@ static int vec_blocks(size_t n)
     const size_t cap = 16ull * device_sm_count();
     if (b > cap) b = cap;
     return b < 1 ? 1 : (int)b;
-}
-
-// Four consecutive values as FP32 (one 16-byte or 8-byte load) and back.
-__device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void store4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
-__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p)
-{
-    const uint2 raw = *reinterpret_cast<const uint2 *>(p);
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
-{
-    uint2 raw;
-    *reinterpret_cast<__nv_bfloat162 *>(&raw.x) = __floats2bfloat162_rn(v.x, v.y);
-    *reinterpret_cast<__nv_bfloat162 *>(&raw.y) = __floats2bfloat162_rn(v.z, v.w);
-    *reinterpret_cast<uint2 *>(p) = raw;
-}
-__device__ __forceinline__ float4 load4(const __half *p)
-{
-    const uint2 raw = *reinterpret_cast<const uint2 *>(p);
-    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&raw.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&raw.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ void store4(__half *p, float4 v)
-{
-    uint2 raw;
-    *reinterpret_cast<__half2 *>(&raw.x) = __floats2half2_rn(v.x, v.y);
-    *reinterpret_cast<__half2 *>(&raw.y) = __floats2half2_rn(v.z, v.w);
-    *reinterpret_cast<uint2 *>(p) = raw;
-}
-
-// r -= alpha q, with q stored as kappa q: r -= (alpha / kappa) q_stored. FP32 arithmetic,
-// r and q in the storage type T (both buffers 256-byte aligned).
-template <typename T>
-__global__ void k_update_r(T *__restrict__ r, const T *__restrict__ q, const Scalars *sc, size_t n)
-{
-    const float a = (float)(sc->alpha / sc->kappa);
-    const size_t n4 = n / 4;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-        float4 rv = load4(r + 4 * i);
-        const float4 qv = load4(q + 4 * i);
-        rv.x = fmaf(-a, qv.x, rv.x);
-        rv.y = fmaf(-a, qv.y, rv.y);
-        rv.z = fmaf(-a, qv.z, rv.z);
-        rv.w = fmaf(-a, qv.w, rv.w);
-        store4(r + 4 * i, rv);
-    }
-    for (size_t i = 4 * n4 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float rv = fmaf(-a, load_as_float(q + i), load_as_float(r + i));
-        store_from_float(r + i, rv);
-    }
-}
-
-static cbct_status launch_update_r(void *r, const void *q, const Scalars *sc, size_t n, int storage, cudaStream_t st)
-{
-    if (storage == ST_BF16)
-        CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_update_r<<<vec_blocks(n), 256, 0, st>>>(static_cast<__nv_bfloat16 *>(r),
-                                                             static_cast<const __nv_bfloat16 *>(q), sc, n));
-    else if (storage == ST_F16)
-        CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_update_r<<<vec_blocks(n), 256, 0, st>>>(static_cast<__half *>(r), static_cast<const __half *>(q),
-                                                             sc, n));
-    else
-        CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_update_r<<<vec_blocks(n), 256, 0, st>>>(static_cast<float *>(r), static_cast<const float *>(q), sc, n));
-    return check_cuda(cudaGetLastError(), "update launch");
 }
 
 // x += alpha p; and if with_p: p = s + beta p
@@ -419,34 +313,26 @@ static cbct_status run_cgls(const GeomDev &G, const float *y, float *x, int n_it
                             const void *traces, cudaStream_t st)
 {
     const long long sz = 1, sx = G.zp, sy = (long long)G.nx * G.zp;
-    const size_t N = internal_elems(G), M = (size_t)G.nviews * G.nv * G.nu;
-    const int nbb = backproject_num_blocks(G);
-    int nbp = 0;
+    const size_t N = internal_elems(G);
     // FP32 storage holds |D-S| r and |D-S| q; 16-bit storage holds r and kappa q and the
     // row prefix applies |D-S|. Only FP16 needs kappa (BF16 has FP32's exponent range).
     const int prescale = storage == ST_F32 ? 0 : 1;
     const int scale_q = storage == ST_F16 ? 1 : 0;
     // r = y - P x; s = P^T r; p = s; gamma = ||s||^2
-    TRY(launch_project(G, x, G.zp, y, w.R, PM_RESID, w.partials, 0.0f, st, storage, w.sc, traces, &nbp));
-    TRY(finalize(w.partials, nbp, w.sc, FIN_RR, st));
+    TRY(launch_project(G, x, G.zp, y, w.R, PM_RESID, w.partials, 0.0f, st, storage, w.sc, traces));
     TRY(launch_row_prefix(G, w.R, w.PS, prescale, st, storage));
-    TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, w.P, w.partials, st));
-    TRY(finalize(w.partials, nbb, w.sc, FIN_GAMMA, st, scale_q));
+    TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, w.P, w.partials, st, w.sc, FIN_GAMMA, scale_q));
     for (int l = 0; l < n_iter; ++l) {
         // q = P p, alpha = gamma / ||q||^2
-        TRY(launch_project(G, w.P, G.zp, nullptr, w.Q, PM_Q_SCALED, w.partials, 0.0f, st, storage, w.sc, traces,
-                           &nbp));
-        TRY(finalize(w.partials, nbp, w.sc, FIN_ALPHA, st));
+        TRY(launch_project(G, w.P, G.zp, nullptr, w.Q, PM_Q_SCALED, w.partials, 0.0f, st, storage, w.sc, traces));
         if (l == n_iter - 1) { // last update: x only; s and p would not be used again
             CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_update_xp<<<vec_blocks(N), 256, 0, st>>>(x, w.P, w.S, w.sc, N, 0));
             TRY(check_cuda(cudaGetLastError(), "update launch"));
             break;
         }
-        TRY(launch_update_r(w.R, w.Q, w.sc, M, storage, st));
-        // s = P^T r, beta = ||s||^2 / gamma
-        TRY(launch_row_prefix(G, w.R, w.PS, prescale, st, storage));
-        TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, nullptr, w.partials, st));
-        TRY(finalize(w.partials, nbb, w.sc, FIN_BETA, st, scale_q));
+        // r -= alpha q; s = P^T r, beta = ||s||^2 / gamma
+        TRY(launch_update_prefix(G, w.R, w.Q, w.sc, w.PS, prescale, st, storage));
+        TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, nullptr, w.partials, st, w.sc, FIN_BETA, scale_q));
         // x += alpha p; p = s + beta p
         CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_update_xp<<<vec_blocks(N), 256, 0, st>>>(x, w.P, w.S, w.sc, N, 1));
         TRY(check_cuda(cudaGetLastError(), "update launch"));

@@ -172,10 +172,6 @@ constexpr int SY_OUT = 30;                       // output positions per warp al
 constexpr int SY_WARPS = SY_ROWS + 2;
 constexpr int SY_THREADS = 32 * SY_WARPS;
 
-__device__ __forceinline__ float raw_to_float(float v) { return v; }
-__device__ __forceinline__ float raw_to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float raw_to_float(__half v) { return __half2float(v); }
-
 // shares of a filter triple (a0, a1, a2): to p + 1, to p, to p - 1
 __device__ __forceinline__ void syn_shares(float a0, float a1, float a2, float &up, float &mid, float &dn)
 {
@@ -216,7 +212,7 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
     for (int cp = c_begin - 1; cp <= c_end; ++cp, buf ^= 1) {
         float a[27];
 #pragma unroll
-        for (int ch = 0; ch < 27; ++ch) a[ch] = raw_to_float(nxt[ch]);
+        for (int ch = 0; ch < 27; ++ch) a[ch] = as_float(nxt[ch]);
         if (cp < c_end) fetch(cp + 1);
         // vector shrinkage, Eq. (2)
         float s2 = 0.0f;
