@@ -8,8 +8,8 @@
 //
 // GB300 mapping. Every kernel marches along axis 2 so that each input value is read from
 // DRAM once and each output written once, with warps reading and writing rows along the
-// contiguous axis. The analysis W owns a 32 x 8 tile of the (axis 0, axis 1) plane and
-// keeps three planes of it in shared memory (with a one-voxel halo). The shrink +
+// contiguous axis. The analysis W marches a tile of the (axis 0, axis 1) plane that is read
+// through shared memory (with a one-voxel halo). The shrink +
 // synthesis and the fused step give each lane whole positions and pass neighbour values by
 // warp shuffles (axis 0), a shared exchange (axis 1) and registers (axis 2); they are
 // described at their kernels. The public transforms are bandwidth bound: 4 B in + 108 B
@@ -27,24 +27,90 @@ __device__ __forceinline__ int wrapi(int i, int n)
     return i < 0 ? i + n : i;
 }
 
+// Two FP32 values in one 64-bit register; each half rounds like the scalar operation.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pk(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v)
+{
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return b;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 splat(float v) { return pk(v, v); }
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, splat(-1.0f), a); } // a - b, rounded once
+
 // Analysis along one axis for the window (f(x-1), f(x), f(x+1)) = (p, c, n):
 // alpha_l(x) = h_l[-1] f(x+1) + h_l[0] f(x) + h_l[1] f(x-1).
 __device__ __forceinline__ void ana3(float p, float c, float n, float &o0, float &o1, float &o2)
 {
     const float s = n + p;
     o0 = fmaf(0.25f, s, 0.5f * c);
-    o1 = R2_4 * (n - p);
+    o1 = __fmul_rn(R2_4, n - p); // (not contracted into the next pass: the packed form's bits)
     o2 = fmaf(-0.25f, s, 0.5f * c);
 }
 
-// Synthesis along one axis: sum_l sum_k h_l[k] a_l(x + k) from the three channels at
-// x-1 (P*), x (C*), x+1 (N*).
-__device__ __forceinline__ float syn3(float P0, float C0, float N0, float P1, float N1, float P2,
-                                      float C2, float N2)
+__device__ __forceinline__ void ana3(f32x2 p, f32x2 c, f32x2 n, f32x2 &o0, f32x2 &o1, f32x2 &o2)
 {
-    return fmaf(0.25f, (P0 + N0) - (P2 + N2), fmaf(0.5f, C0 + C2, R2_4 * (P1 - N1)));
+    const f32x2 s = add2(n, p), h = mul2(splat(0.5f), c);
+    o0 = fma2(splat(0.25f), s, h);
+    o1 = mul2(splat(R2_4), sub2(n, p));
+    o2 = fma2(splat(-0.25f), s, h);
 }
 
+// Two adjacent values of the contiguous axis as stored.
+template <typename T> struct Pair;
+template <> struct Pair<float> {
+    using T2 = float2;
+    static __device__ __forceinline__ f32x2 get(T2 v) { return pk(v.x, v.y); }
+    static __device__ __forceinline__ T2 put(f32x2 v) { return make_float2(lo2(v), hi2(v)); }
+};
+template <> struct Pair<__nv_bfloat16> {
+    using T2 = __nv_bfloat162;
+    static __device__ __forceinline__ f32x2 get(T2 v)
+    {
+        const float2 f = __bfloat1622float2(v);
+        return pk(f.x, f.y);
+    }
+    static __device__ __forceinline__ T2 put(f32x2 v) { return __floats2bfloat162_rn(lo2(v), hi2(v)); }
+};
+template <> struct Pair<__half> {
+    using T2 = __half2;
+    static __device__ __forceinline__ f32x2 get(T2 v)
+    {
+        const float2 f = __half22float2(v);
+        return pk(f.x, f.y);
+    }
+    static __device__ __forceinline__ T2 put(f32x2 v) { return __floats2half2_rn(lo2(v), hi2(v)); }
+};
 
 template <typename TA_T>
 __global__ void __launch_bounds__(TF_THREADS)
@@ -125,6 +191,89 @@ k_tf_analyze(int n0, int n1, int n2, int chunk, const float *__restrict__ f, TA_
     }
 }
 
+// The same with two adjacent positions per lane (an even n0, so that every pair is aligned): one
+// store of a pair per channel, packed arithmetic with the bits of the general kernel's, and the axis-0
+// and axis-1 passes of each plane done once (those of the two planes before stay in registers).
+// Bound by the 27 written channels: 512x512x70 FP32 334 us (6.2 TB/s; one position per lane and three
+// planes in shared memory 360 us), BF16 198 us (240), 256x256x64 74 (76) and 44 us (62). Blocks of
+// 4 rows and 102 registers, five per SM; with 80 registers 336 | 245 us, blocks of 8 rows 330 | 221 us but
+// 84 us at 256x256x64 FP32 (the last wave), 2 rows 341 | 256 us. An odd n0 takes the general kernel.
+constexpr int AP_B = 4, AP_THREADS = 32 * AP_B, AP_BLOCKS = 5;
+template <typename T>
+__global__ void __launch_bounds__(AP_THREADS, AP_BLOCKS)
+k_tf_analyze_pair(int n0, int n1, int n2, int chunk, const float *__restrict__ f, T *__restrict__ alpha)
+{
+    using P = Pair<T>;
+    using T2 = typename P::T2;
+    constexpr int W = 66, SIZE = W * (AP_B + 2), PER = (SIZE + AP_THREADS - 1) / AP_THREADS;
+    __shared__ __align__(8) float s[2][SIZE]; // a plane of the tile with its halo
+    const int a0 = blockIdx.x * 64, b0 = blockIdx.y * AP_B;
+    const int c_begin = blockIdx.z * chunk;
+    const int c_end = min(n2, c_begin + chunk);
+    if (c_begin >= c_end) return;
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    const size_t plane = (size_t)n0 * n1, N = plane * n2;
+
+    int off[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int pos = tid + k * AP_THREADS, r = pos / W, q = pos - r * W;
+        off[k] = pos < SIZE ? wrapi(b0 + r - 1, n1) * n0 + wrapi(a0 + q - 1, n0) : -1;
+    }
+    float nxt[PER];
+    auto fetch = [&](int c) {
+        const float *src = f + (size_t)wrapi(c, n2) * plane;
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (off[k] >= 0) nxt[k] = __ldg(src + off[k]);
+    };
+    fetch(c_begin - 1);
+    const int pa = a0 + 2 * threadIdx.x, pb = b0 + threadIdx.y;
+    const bool inside = pa < n0 && pb < n1;
+    f32x2 um[3][3], u0[3][3]; // [m][l] of planes cp - 2 and cp - 1
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) um[m][l] = u0[m][l] = 0ull;
+    int buf = 0;
+    for (int cp = c_begin - 1; cp <= c_end; ++cp, buf ^= 1) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (off[k] >= 0) s[buf][tid + k * AP_THREADS] = nxt[k];
+        __syncthreads();
+        if (cp < c_end) fetch(cp + 1);
+        f32x2 t[3][3], up[3][3];
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb) {
+            const float2 *row = reinterpret_cast<const float2 *>(&s[buf][(threadIdx.y + bb) * W + 2 * threadIdx.x]);
+            const float2 v0 = row[0], v1 = row[1];
+            ana3(pk(v0.x, v0.y), pk(v0.y, v1.x), pk(v1.x, v1.y), t[bb][0], t[bb][1], t[bb][2]);
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) ana3(t[0][l], t[1][l], t[2][l], up[0][l], up[1][l], up[2][l]);
+        if (inside && cp > c_begin) {
+            T2 *q = reinterpret_cast<T2 *>(alpha + (size_t)(cp - 1) * plane + (size_t)pb * n0 + pa);
+            const size_t ch = N / 2; // (N is even)
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
+                    f32x2 w[3];
+                    ana3(um[m][l], u0[m][l], up[m][l], w[0], w[1], w[2]);
+#pragma unroll
+                    for (int n = 0; n < 3; ++n) __stcs(q + (l + 3 * m + 9 * n) * ch, P::put(w[n]));
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                um[m][l] = u0[m][l];
+                u0[m][l] = up[m][l];
+            }
+    }
+}
+
 // Planes per block along axis 2 (shrink + synthesis and the fused step): the split whose blocks fill whole
 // waves of the resident slots best, counting the two extra planes each block recomputes
 // at its start (a block's cost grows with chunk + 2).
@@ -162,27 +311,23 @@ static int fused_chunk(long long tiles, int n2, int slots)
 // two shuffles per channel group, axis 1 between warps through shared memory (one
 // barrier per plane, double buffered), and axis 2 between planes in registers.
 // HBM traffic: 27 coefficients read and one value written per voxel; the halo positions
-// (32/30 along axis 0, (SY_ROWS + 2)/SY_ROWS along axis 1) are re-read from L2.
+// (32/30 along axis 0, (SY_ROWS + 2)/SY_ROWS along axis 1) are re-read from L2, and a warp's
+// row touches five sectors of each channel, not four. 512x512x70 FP32: 411 us, 2.10 GB from
+// DRAM (5.3 TB/s), 3.58 GB from L2 (8.8 TB/s), issue 60%. Two positions per lane 420 us, 16 or 20 warps
+// in one block 414 | 411 us, a second plane of coefficients under way 413 us.
 // ------------------------------------------------------------------------------------
-#ifndef CBCT_SY_ROWS
-#define CBCT_SY_ROWS 8
-#endif
-constexpr int SY_ROWS = CBCT_SY_ROWS;
+constexpr int SY_ROWS = 8;
 constexpr int SY_OUT = 30;                       // output positions per warp along axis 0
 constexpr int SY_WARPS = SY_ROWS + 2;
 constexpr int SY_THREADS = 32 * SY_WARPS;
 
-// shares of a filter triple (a0, a1, a2): to p + 1, to p, to p - 1
-__device__ __forceinline__ void syn_shares(float a0, float a1, float a2, float &up, float &mid, float &dn)
-{
-    const float q = 0.25f * (a0 - a2);
-    up = fmaf(R2_4, a1, q);
-    dn = fmaf(-R2_4, a1, q);
-    mid = 0.5f * (a0 + a2);
-}
+// Each pass leaves out a factor 1/4 of its taps, which rounds nothing: shares a_0 - a_2 +- sqrt(2) a_1 and
+// 2 (a_0 + a_2), and 64 times the result. The shrinkage factor is applied to a triple's sum and difference.
+// Kernels for pairs of positions take the same operations and leave the same bits.
+constexpr float SYN_R = 4.0f * R2_4;
 
 template <typename TA_T>
-__global__ void __launch_bounds__(SY_THREADS, SY_THREADS <= 320 ? 2 : 1)
+__global__ void __launch_bounds__(SY_THREADS, 2)
 k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ alpha, float mu,
                   int positivity, float *__restrict__ f)
 {
@@ -220,33 +365,34 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
         for (int ch = 1; ch < 27; ++ch) s2 = fmaf(a[ch], a[ch], s2);
         const float nrm = sqrtf(s2);
         const float scale = nrm > mu ? 1.0f - mu / nrm : 0.0f;
-#pragma unroll
-        for (int ch = 1; ch < 27; ++ch) a[ch] *= scale;
+        const float sc2 = scale + scale, scr = SYN_R * scale, scn = -SYN_R * scale;
         // axis 0 (lanes): u[m + 3n] = sum over l and the lane's neighbours
         float u[9];
 #pragma unroll
         for (int mn = 0; mn < 9; ++mn) {
-            float up, mid, dn;
-            syn_shares(a[3 * mn], a[3 * mn + 1], a[3 * mn + 2], up, mid, dn);
-            u[mn] = __shfl_up_sync(0xffffffffu, up, 1) + mid + __shfl_down_sync(0xffffffffu, dn, 1);
+            const float a0 = a[3 * mn], a2 = mn ? a[3 * mn + 2] : __fmul_rn(scale, a[3 * mn + 2]); // (channel 0 is not shrunk)
+            const float q = mn ? __fmul_rn(scale, a0 - a2) : a0 - a2;
+            const float up = fmaf(scr, a[3 * mn + 1], q), dn = fmaf(scn, a[3 * mn + 1], q);
+            u[mn] = fmaf(mn ? sc2 : 2.0f, a0 + a2, __shfl_up_sync(0xffffffffu, up, 1)) + __shfl_down_sync(0xffffffffu, dn, 1);
         }
         // axis 1 (warps): shares of rows to the rows above and below through shared memory
-        float midn[3];
+        float mid[3];
 #pragma unroll
         for (int n = 0; n < 3; ++n) {
-            float up, dn;
-            syn_shares(u[3 * n], u[3 * n + 1], u[3 * n + 2], up, midn[n], dn);
-            s_up[buf][w][n][lane] = up;
-            s_dn[buf][w][n][lane] = dn;
+            const float q = u[3 * n] - u[3 * n + 2];
+            mid[n] = u[3 * n] + u[3 * n + 2];
+            s_up[buf][w][n][lane] = fmaf(SYN_R, u[3 * n + 1], q);
+            s_dn[buf][w][n][lane] = fmaf(-SYN_R, u[3 * n + 1], q);
         }
         __syncthreads();
         if (out_row) {
             float wv[3];
 #pragma unroll
-            for (int n = 0; n < 3; ++n) wv[n] = s_up[buf][w - 1][n][lane] + midn[n] + s_dn[buf][w + 1][n][lane];
+            for (int n = 0; n < 3; ++n) wv[n] = fmaf(2.0f, mid[n], s_up[buf][w - 1][n][lane]) + s_dn[buf][w + 1][n][lane];
             // axis 2 (planes): plane cp - 1 from planes cp - 2, cp - 1, cp
             if (cp >= c_begin + 1 && out_lane) {
-                float o = syn3(w_m2[0], w_m1[0], wv[0], w_m2[1], wv[1], w_m2[2], w_m1[2], wv[2]);
+                const float ends = (w_m2[0] + wv[0]) - (w_m2[2] + wv[2]);
+                float o = (fmaf(2.0f, w_m1[0] + w_m1[2], SYN_R * (w_m2[1] - wv[1])) + ends) * (1.0f / 64.0f);
                 if (positivity && o < 0.0f) o = 0.0f;
                 f[(size_t)(cp - 1) * plane + (size_t)pb * n0 + pa] = o;
             }
@@ -262,13 +408,16 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
 template <typename TA_T>
 static cbct_status launch_tf_analyze_t(int n0, int n1, int n2, const float *f, TA_T *alpha, cudaStream_t st)
 {
+    const bool pair = n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & (2 * sizeof(TA_T) - 1)) == 0;
+    const auto kernel = pair ? k_tf_analyze_pair<TA_T> : k_tf_analyze<TA_T>;
+    const int ta = pair ? 64 : TA, tb = pair ? AP_B : TB;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_analyze<TA_T>, TF_THREADS, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * tb, 0);
     if (e != cudaSuccess) return check_cuda(e, "tf_analyze occupancy");
-    const long long tiles = (long long)((n0 + TA - 1) / TA) * ((n1 + TB - 1) / TB);
+    const long long tiles = (long long)((n0 + ta - 1) / ta) * ((n1 + tb - 1) / tb);
     const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
-    dim3 grid((n0 + TA - 1) / TA, (n1 + TB - 1) / TB, (n2 + chunk - 1) / chunk);
-    CBCT_TIMED(CBCT_KERNEL_TF_ANALYZE, st, k_tf_analyze<<<grid, dim3(TA, TB), 0, st>>>(n0, n1, n2, chunk, f, alpha));
+    dim3 grid((n0 + ta - 1) / ta, (n1 + tb - 1) / tb, (n2 + chunk - 1) / chunk);
+    CBCT_TIMED(CBCT_KERNEL_TF_ANALYZE, st, kernel<<<grid, dim3(32, tb), 0, st>>>(n0, n1, n2, chunk, f, alpha));
     return check_cuda(cudaGetLastError(), "tf_analyze launch");
 }
 
@@ -287,33 +436,20 @@ cbct_status launch_tf_analyze(int n0, int n1, int n2, const float *f, void *alph
 // extent n0 is even, which the launcher requires; an even n0 also keeps a pair from
 // straddling the periodic wrap).
 constexpr int SP_OUT = 60;
-// output rows per block: one block of 16 warps per SM (128 registers, 48 KB of shared
-// memory) measured 0.338 ms at 512x512x70 BF16 against 0.352 ms for two blocks of 6 rows
-#ifndef CBCT_SP_ROWS
-#define CBCT_SP_ROWS 14
-#endif
-constexpr int SP_ROWS = CBCT_SP_ROWS;
-constexpr int SP_WARPS = SP_ROWS + 2;
-constexpr int SP_THREADS = 32 * SP_WARPS;
+// Output rows per block: one block of 16 warps per SM (126 registers, 48 KB of shared memory)
+// takes 313 us at 512x512x70 BF16 in packed arithmetic (329 us position by position), two blocks of
+// 6 rows 329 us, 10 warps 366 us; 18 and 20 warps spill (507 us), and so does a second plane of
+// coefficients under way (383 us).
+constexpr int SP_ROWS = 14, SP_WARPS = SP_ROWS + 2;
 
-template <typename T16> struct Pair16;
-template <> struct Pair16<__nv_bfloat16> {
-    using T2 = __nv_bfloat162;
-    static __device__ __forceinline__ float2 f2(T2 v) { return __bfloat1622float2(v); }
-};
-template <> struct Pair16<__half> {
-    using T2 = __half2;
-    static __device__ __forceinline__ float2 f2(T2 v) { return __half22float2(v); }
-};
-
-template <typename T16>
-__global__ void __launch_bounds__(SP_THREADS, SP_THREADS <= 256 ? 2 : 1)
-k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T16 *__restrict__ alpha, float mu, int positivity,
+template <typename T>
+__global__ void __launch_bounds__(32 * SP_WARPS, 1)
+k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T *__restrict__ alpha, float mu, int positivity,
                        float *__restrict__ f)
 {
-    using P = Pair16<T16>;
+    using P = Pair<T>;
     using T2 = typename P::T2;
-    __shared__ float2 s_up[2][SP_WARPS][3][32], s_dn[2][SP_WARPS][3][32];
+    __shared__ f32x2 s_up[2][SP_WARPS][3][32], s_dn[2][SP_WARPS][3][32];
     const int lane = threadIdx.x, w = threadIdx.y;
     const int a_out = blockIdx.x * SP_OUT, b_out = blockIdx.y * SP_ROWS;
     const int c_begin = blockIdx.z * chunk;
@@ -334,9 +470,7 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T16 *__restrict_
         for (int ch = 0; ch < 27; ++ch) nxt[ch] = src[(size_t)ch * stride];
     };
     fetch(c_begin - 1);
-    float2 w_m2[3], w_m1[3];
-#pragma unroll
-    for (int n = 0; n < 3; ++n) w_m2[n] = w_m1[n] = make_float2(0.f, 0.f);
+    f32x2 w_m2[3] = {0ull, 0ull, 0ull}, w_m1[3] = {0ull, 0ull, 0ull}; // axis-2 inputs at planes cp-2, cp-1
     int buf = 0;
     for (int cp = c_begin - 1; cp <= c_end; ++cp, buf ^= 1) {
         T2 cur[27];
@@ -344,57 +478,46 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T16 *__restrict_
         for (int ch = 0; ch < 27; ++ch) cur[ch] = nxt[ch];
         if (cp < c_end) fetch(cp + 1);
         // vector shrinkage, Eq. (2), for both positions
-        float2 s2 = make_float2(0.f, 0.f);
+        f32x2 s2 = 0ull;
 #pragma unroll
         for (int ch = 1; ch < 27; ++ch) {
-            const float2 a = P::f2(cur[ch]);
-            s2.x = fmaf(a.x, a.x, s2.x);
-            s2.y = fmaf(a.y, a.y, s2.y);
+            const f32x2 a = P::get(cur[ch]);
+            s2 = fma2(a, a, s2);
         }
-        const float na = sqrtf(s2.x), nb = sqrtf(s2.y);
-        const float sa = na > mu ? 1.0f - mu / na : 0.0f, sb = nb > mu ? 1.0f - mu / nb : 0.0f;
-        // axis 0: position A (even) takes lane - 1's B and its own B; B takes its own A and
-        // lane + 1's A
-        float2 u[9];
+        const float na = sqrtf(lo2(s2)), nb = sqrtf(hi2(s2));
+        const f32x2 sc = pk(na > mu ? 1.0f - mu / na : 0.0f, nb > mu ? 1.0f - mu / nb : 0.0f);
+        const f32x2 sc2 = add2(sc, sc), scr = mul2(splat(SYN_R), sc), scn = mul2(splat(-SYN_R), sc);
+        // axis 0: the even position takes lane - 1's odd one and its own odd one; the odd position takes
+        // its own even one and lane + 1's even one
+        f32x2 u[9];
 #pragma unroll
         for (int mn = 0; mn < 9; ++mn) {
-            float2 a0 = P::f2(cur[3 * mn]), a1 = P::f2(cur[3 * mn + 1]), a2 = P::f2(cur[3 * mn + 2]);
-            if (mn) {
-                a0.x *= sa;
-                a0.y *= sb;
-            }
-            a1.x *= sa;
-            a1.y *= sb;
-            a2.x *= sa;
-            a2.y *= sb;
-            float upA, midA, dnA, upB, midB, dnB;
-            syn_shares(a0.x, a1.x, a2.x, upA, midA, dnA);
-            syn_shares(a0.y, a1.y, a2.y, upB, midB, dnB);
-            u[mn].x = __shfl_up_sync(0xffffffffu, upB, 1) + midA + dnB;
-            u[mn].y = upA + midB + __shfl_down_sync(0xffffffffu, dnA, 1);
+            f32x2 a0 = P::get(cur[3 * mn]), a1 = P::get(cur[3 * mn + 1]), a2 = P::get(cur[3 * mn + 2]);
+            if (mn == 0) a2 = mul2(sc, a2); // (channel 0 is not shrunk)
+            const f32x2 q = mn ? mul2(sc, sub2(a0, a2)) : sub2(a0, a2);
+            const f32x2 up = fma2(scr, a1, q), dn = fma2(scn, a1, q);
+            u[mn] = add2(fma2(mn ? sc2 : splat(2.0f), add2(a0, a2), pk(__shfl_up_sync(0xffffffffu, hi2(up), 1), lo2(up))),
+                         pk(hi2(dn), __shfl_down_sync(0xffffffffu, lo2(dn), 1)));
         }
         // axis 1 (warps) through shared memory
-        float2 midn[3];
+        f32x2 mid[3];
 #pragma unroll
         for (int n = 0; n < 3; ++n) {
-            float2 up, dn;
-            syn_shares(u[3 * n].x, u[3 * n + 1].x, u[3 * n + 2].x, up.x, midn[n].x, dn.x);
-            syn_shares(u[3 * n].y, u[3 * n + 1].y, u[3 * n + 2].y, up.y, midn[n].y, dn.y);
-            s_up[buf][w][n][lane] = up;
-            s_dn[buf][w][n][lane] = dn;
+            const f32x2 q = sub2(u[3 * n], u[3 * n + 2]);
+            mid[n] = add2(u[3 * n], u[3 * n + 2]);
+            s_up[buf][w][n][lane] = fma2(splat(SYN_R), u[3 * n + 1], q);
+            s_dn[buf][w][n][lane] = fma2(splat(-SYN_R), u[3 * n + 1], q);
         }
         __syncthreads();
         if (out_row) {
-            float2 wv[3];
+            f32x2 wv[3];
 #pragma unroll
-            for (int n = 0; n < 3; ++n) {
-                const float2 a = s_up[buf][w - 1][n][lane], b = s_dn[buf][w + 1][n][lane];
-                wv[n] = make_float2(a.x + midn[n].x + b.x, a.y + midn[n].y + b.y);
-            }
+            for (int n = 0; n < 3; ++n)
+                wv[n] = add2(fma2(splat(2.0f), mid[n], s_up[buf][w - 1][n][lane]), s_dn[buf][w + 1][n][lane]);
             if (cp >= c_begin + 1 && out_lane) {
-                float2 o;
-                o.x = syn3(w_m2[0].x, w_m1[0].x, wv[0].x, w_m2[1].x, wv[1].x, w_m2[2].x, w_m1[2].x, wv[2].x);
-                o.y = syn3(w_m2[0].y, w_m1[0].y, wv[0].y, w_m2[1].y, wv[1].y, w_m2[2].y, w_m1[2].y, wv[2].y);
+                const f32x2 ends = sub2(add2(w_m2[0], wv[0]), add2(w_m2[2], wv[2]));
+                const f32x2 o64 = add2(fma2(splat(2.0f), add2(w_m1[0], w_m1[2]), mul2(splat(SYN_R), sub2(w_m2[1], wv[1]))), ends);
+                float2 o = make_float2(lo2(o64) * (1.0f / 64.0f), hi2(o64) * (1.0f / 64.0f));
                 if (positivity) {
                     o.x = o.x < 0.0f ? 0.0f : o.x;
                     o.y = o.y < 0.0f ? 0.0f : o.y;
@@ -410,19 +533,19 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T16 *__restrict_
     }
 }
 
-template <typename T16>
-static cbct_status launch_tf_synth_shrink_pair(int n0, int n1, int n2, const T16 *alpha, float mu, int positivity,
+template <typename T>
+static cbct_status launch_tf_synth_shrink_pair(int n0, int n1, int n2, const T *alpha, float mu, int positivity,
                                                float *f, cudaStream_t st)
 {
+    constexpr int rows = SP_ROWS;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_synth_shrink_pair<T16>, SP_THREADS, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_synth_shrink_pair<T>, 32 * SP_WARPS, 0);
     if (e != cudaSuccess) return check_cuda(e, "tf_synth_shrink occupancy");
-    const long long tiles = (long long)((n0 + SP_OUT - 1) / SP_OUT) * ((n1 + SP_ROWS - 1) / SP_ROWS);
+    const long long tiles = (long long)((n0 + SP_OUT - 1) / SP_OUT) * ((n1 + rows - 1) / rows);
     const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
-    dim3 grid((n0 + SP_OUT - 1) / SP_OUT, (n1 + SP_ROWS - 1) / SP_ROWS, (n2 + chunk - 1) / chunk);
+    dim3 grid((n0 + SP_OUT - 1) / SP_OUT, (n1 + rows - 1) / rows, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
-               k_tf_synth_shrink_pair<T16><<<grid, dim3(32, SP_WARPS), 0, st>>>(n0, n1, n2, chunk, alpha, mu, positivity,
-                                                                                f));
+               k_tf_synth_shrink_pair<T><<<grid, dim3(32, SP_WARPS), 0, st>>>(n0, n1, n2, chunk, alpha, mu, positivity, f));
     return check_cuda(cudaGetLastError(), "tf_synth_shrink launch");
 }
 
@@ -490,47 +613,6 @@ constexpr int FR_WARPS = 16;
 constexpr int FR_ROWS = 2 * FR_WARPS - 4; // output rows per block along axis 1
 constexpr int FR_OUT = 28;                // output positions per warp along axis 0
 constexpr int FR_THREADS = 32 * FR_WARPS;
-
-// Two FP32 values in one 64-bit register: .x the even row's, .y the odd row's.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pk(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float lo2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return a;
-}
-__device__ __forceinline__ float hi2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return b;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 splat(float v) { return pk(v, v); }
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, splat(-1.0f), a); } // a - b, rounded once
 
 // The frame with plain taps: [1, 2, 1], [1, 0, -1] and [1, -2, 1] stand for 4 h_0, (4 / sqrt(2)) h_1
 // and -4 h_2, so that a triple takes four operations. A coefficient with j factors h_1 is then 64 /
