@@ -18,11 +18,12 @@
 // same plane coordinates and reciprocals as the projector's, so both operators use the same
 // weights to FP32 rounding. No atomics: the result is independent of scheduling.
 //
-// What bounds it on the paper's finest grid (512x512x70, 40 views, 1.25 ms, 14 voxels per
-// thread): L1 data wavefronts 69-74% (the table's lines: lanes of a patch read about ten
-// sectors), issue slots 71%. Before the straddling row became one saturating multiply and
-// the chunks whole it took 1.63 ms; with the warps of a block on the same patch taking
-// turns at the views, 128x128x18 takes 104 us (200 before), 64x64x16 25 us (61).
+// What bounds it on the paper's finest grid (512x512x70, 40 views, 1.16 ms, 14 voxels per
+// thread): issue slots 80% (1.15e9 warp instructions, three fifths of them the plane loop's) and
+// L1 data wavefronts 67% (the table's lines: lanes of a patch read about ten sectors). Before the
+// straddling row became one saturating multiply and the chunks whole it took 1.63 ms, with
+// the plane heights computed for each plane 1.25 ms; with the warps of a block on the same
+// patch taking turns at the views, 128x128x18 takes 99 us (200 before), 64x64x16 22 us (61).
 #include "cbct_internal.cuh"
 
 #include <cmath>
@@ -51,8 +52,9 @@ constexpr int BP_MAX_WARPS = 16;
 constexpr int BP_ZC[] = {8, 12, 14, 16, 18};
 
 // The voxels per thread that cover a column with the fewest planes (about one and a half more per
-// chunk for its first plane and set-up); measured at 512x512x70 (12 | 14 | 16 | 18): 1357 | 1254 | 1433 |
-// 1320 us, 256x256x35: 339 | 392 | 430 | 347 us. Where even 8 slices leave few warps, 8 voxels
+// chunk for its first plane and set-up); measured at 512x512x70 (12 | 14 | 16 | 18): 1268 | 1183 | 1321 |
+// 1249 us, 128x128x18 137 | 154 | 172 | 100 us, 256x256x35 320 | 350 | 400 | 340 us (three chunks of 12
+// have 36 planes like two of 18: the tail of the last wave is shorter). Where even 8 slices leave few warps, 8 voxels
 // (64x64x16: 24.6 us, with 16 32.8 us). Slices double until the chip has about 96 warps per
 // SM to draw from: 256x256x35 with 1 | 2 | 4 | 8 slices 403 | 354 | 339 | 356 us, 128x128x18 456 |
 // 240 | 131 | 104 us, 512x512x70 1254 | 1311 | 1393 | 1583 us (less of the table is shared in L1).
@@ -120,6 +122,7 @@ struct BpVisit {
 struct BpChunk {
     float zbot, zs_bot, dzs, c0;
     int nzc;
+    unsigned zpairs; // shared address of the heights of planes 1, 2, ..., ZC times SIDE
 };
 
 // Adds this visit's share of every voxel of the chunk. The rows that reach plane zp inside the
@@ -167,6 +170,34 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
     };
     float P0, g0, f0;
     plane(0, P0, g0, f0);
+    if constexpr (SIDE != 0 && FULL && !CLAMP) {
+        static_assert(ZC % 2 == 0);
+        constexpr bool LOOKUP = ZC > BP_ZC[0];
+        // Two planes at a time. Longer chunks read the pair's heights from shared memory, one load
+        // for both: the heights' arithmetic costs them issue slots and registers (512x512x70, 14
+        // voxels: 1181 us, computed 1251 us; 512x512x128: 1991 | 2166 us). Chunks of 8 have the
+        // registers and little to hide the load behind (64x64x16: 24.6 us, computed 22.6 us).
+        const float edge = SIDE > 0 ? -sa : sb;
+#pragma unroll
+        for (int z = 0; z < ZC; z += 2) {
+            const int a1 = __float_as_int(__fadd_ru(fmaf((float)(z + 1), xs, x0), 12582912.0f));
+            const int a2 = __float_as_int(__fadd_ru(fmaf((float)(z + 2), xs, x0), 12582912.0f));
+            const float2 T1 = __ldg(reinterpret_cast<const float2 *>(q.tab + (long long)a1 * q.row_bytes));
+            const float2 T2 = __ldg(reinterpret_cast<const float2 *>(q.tab + (long long)a2 * q.row_bytes));
+            float2 zp;
+            if constexpr (LOOKUP) zp = lds_float2(c.zpairs + 4u * (unsigned)z);
+            else zp = make_float2(SIDE * fmaf((float)(z + 1), G.dz, c.zbot), SIDE * fmaf((float)(z + 2), G.dz, c.zbot));
+            const float f1 = __saturatef(fmaf(zp.x, lds_float(q.iv + 4u * (unsigned)a1), edge) * winv);
+            const float f2 = __saturatef(fmaf(zp.y, lds_float(q.iv + 4u * (unsigned)a2), edge) * winv);
+            const float g1 = f1 > 0.0f ? T1.y : 0.0f, g2 = f2 > 0.0f ? T2.y : 0.0f;
+            acc[z] = fmaf(w, fmaf(-g0, f0, fmaf(g1, f1, T1.x - P0)), acc[z]);
+            acc[z + 1] = fmaf(w, fmaf(-g1, f1, fmaf(g2, f2, T2.x - T1.x)), acc[z + 1]);
+            P0 = T2.x;
+            g0 = g2;
+            f0 = f2;
+        }
+        return;
+    }
 #pragma unroll
     for (int z = 0; z < ZC; ++z) {
         if (!FULL && z >= c.nzc) break;
@@ -215,13 +246,20 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
     ch.zs_bot = ch.zbot * G.inv_dv;
     ch.dzs = G.dz * G.inv_dv;
     ch.c0 = fmaf(-G.v_first, G.inv_dv, -1e-3f);
+    __shared__ __align__(8) float s_z[2][ZC];
+    if (tid < ZC) {
+        const float z = plane_at(iz0 + 1 + tid, G.dz, G.z0);
+        s_z[0][tid] = z;
+        s_z[1][tid] = -z;
+    }
     const float ztop = plane_at(iz0 + ch.nzc, G.dz, G.z0), zs_top = ztop * G.inv_dv;
     const float zabs = fmaxf(fabsf(ch.zbot), fabsf(ztop));
     const float c1 = fmaf(-G.v_first, G.inv_dv, 1e-3f);
     const size_t view_stride = ((size_t)G.nv + 1) * G.nu;
     const unsigned iv0 = smem_u32(s_invv) - 4u * (unsigned)ROUND_BIAS;
 
-    // imager columns in the shadow of the voxel column in view k (its corners' u)
+    // imager columns in the shadow of the voxel column in view k (its corners' u); the least and
+    // greatest u / sdd, scaled once (scaled corner by corner 1181 us at 512x512x70, so 1163)
     auto shadow = [&](int k, int &lo, int &hi) {
         const float2 cs = G.cs[k];
         float umin = 3.0e38f, umax = -3.0e38f;
@@ -229,13 +267,13 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
         for (int c = 0; c < 4; ++c) {
             const float px = (c & 1) ? xh : xl, py = (c & 2) ? yh : yl;
             const float a = fmaf(-px, cs.y, py * cs.x);
-            const float w = G.sad - fmaf(px, cs.x, py * cs.y);
-            const float u = G.sdd * __fdividef(a, w);
-            umin = fminf(umin, u);
-            umax = fmaxf(umax, u);
+            const float w = fmaf(-px, cs.x, fmaf(-py, cs.y, G.sad));
+            const float t = __fdividef(a, w);
+            umin = fminf(umin, t);
+            umax = fmaxf(umax, t);
         }
-        lo = max(0, (int)ceilf(fmaf(umin - G.u_first, G.inv_du, -1e-3f)));
-        hi = min(G.nu - 1, (int)floorf(fmaf(umax - G.u_first, G.inv_du, 1e-3f)));
+        lo = max(0, (int)ceilf(fmaf(fmaf(umin, G.sdd, -G.u_first), G.inv_du, -1e-3f)));
+        hi = min(G.nu - 1, (int)floorf(fmaf(fmaf(umax, G.sdd, -G.u_first), G.inv_du, 1e-3f)));
     };
     // all rows of imager column iu in view k that cross this voxel column
     auto visit = [&](int k, int iu) {
@@ -271,6 +309,7 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
             q.row_bytes = 8 * G.nu;
             q.tab = reinterpret_cast<const char *>(ps + entry) - (long long)ROUND_BIAS * q.row_bytes;
             if (ch.nzc == ZC) {
+                ch.zpairs = smem_u32(s_z[side < 0]);
                 if (side > 0) bp_planes<ZC, 1, false, true>(G, q, ch, acc);
                 else if (side < 0) bp_planes<ZC, -1, false, true>(G, q, ch, acc);
                 else bp_planes<ZC, 0, true, true>(G, q, ch, acc);

@@ -76,9 +76,8 @@ __device__ __forceinline__ float tau_zplane(float p, float inv_v, float tc) { re
 __device__ __forceinline__ float imager_u(const GeomDev &G, int iu) { return fmaf((float)iu, G.du, G.u_first); }
 __device__ __forceinline__ float imager_v(const GeomDev &G, int iv) { return fmaf((float)iv, G.dv, G.v_first); }
 
-// Exact ceil / floor of |x| < 2^22 through the FP adder (no conversion instruction):
-// adding 1.5 * 2^23 with rounding up / down leaves the integer in the low mantissa bits.
-__device__ __forceinline__ int ceil_small(float x) { return __float_as_int(__fadd_ru(x, 12582912.0f)) - 0x4B400000; }
+// Exact floor of |x| < 2^22 through the FP adder (no conversion instruction):
+// adding 1.5 * 2^23 with rounding down leaves the integer in the low mantissa bits.
 __device__ __forceinline__ int floor_small(float x) { return __float_as_int(__fadd_rd(x, 12582912.0f)) - 0x4B400000; }
 
 // Shared memory by 32-bit address.
@@ -87,6 +86,12 @@ __device__ __forceinline__ float lds_float(unsigned a)
 {
     float v;
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 lds_float2(unsigned a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
     return v;
 }
 
