@@ -352,6 +352,7 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
         }
     };
 
+    chain_wait();
     __syncthreads();
     if (ok && FLAT) {
         // (the lane's list goes on across all views of its slice)
@@ -464,7 +465,7 @@ cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, l
     int isx = (int)sx, isy = (int)sy, isz = (int)sz;
     void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials, &sc, &fin_op, &scale_q};
     ProfToken tok = prof_start(CBCT_KERNEL_BACKPROJECT, st);
-    const cudaError_t e = cudaLaunchKernel(bp_kernel(p.zc, flat), p.grid, dim3(32u * p.warps), args, smem, st);
+    const cudaError_t e = launch_chained(bp_kernel(p.zc, flat), p.grid, dim3(32u * p.warps), args, smem, st);
     prof_stop(tok, st);
     note_launch();
     if (e != cudaSuccess) cudaGetLastError(); // the error is returned, not left pending
@@ -499,6 +500,7 @@ template <typename T, bool UPDATE>
 __global__ void __launch_bounds__(32 * PREFIX_WARPS)
 k_row_prefix(GeomDev G, T *g, const T *__restrict__ q, const Scalars *__restrict__ sc, float2 *__restrict__ ps, int prescale)
 {
+    chain_wait();
     __shared__ float2 s_tot[PREFIX_WARPS][32];
     const int lane = threadIdx.x, w = threadIdx.y;
     const int k = blockIdx.y, iu = blockIdx.x * 32 + lane;
@@ -562,10 +564,10 @@ static void row_prefix(const GeomDev &G, void *g, const void *q, const Scalars *
     const dim3 grid((G.nu + 31) / 32, G.nviews), block(32, PREFIX_WARPS);
     if (q)
         CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_row_prefix<T, true><<<grid, block, 0, st>>>(G, static_cast<T *>(g), static_cast<const T *>(q), sc, ps, prescale));
+                   launch_chained(k_row_prefix<T, true>, grid, block, 0, st, G, static_cast<T *>(g), static_cast<const T *>(q), sc, ps, prescale));
     else
         CBCT_TIMED(CBCT_KERNEL_OTHER, st,
-                   k_row_prefix<T, false><<<grid, block, 0, st>>>(G, static_cast<T *>(g), nullptr, nullptr, ps, prescale));
+                   launch_chained(k_row_prefix<T, false>, grid, block, 0, st, G, static_cast<T *>(g), nullptr, nullptr, ps, prescale));
 }
 
 cbct_status launch_update_prefix(const GeomDev &G, void *r, const void *q, const Scalars *sc, float2 *ps, int prescale,

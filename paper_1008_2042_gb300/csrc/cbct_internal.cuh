@@ -80,6 +80,12 @@ __device__ __forceinline__ float imager_v(const GeomDev &G, int iv) { return fma
 // adding 1.5 * 2^23 with rounding down leaves the integer in the low mantissa bits.
 __device__ __forceinline__ int floor_small(float x) { return __float_as_int(__fadd_rd(x, 12582912.0f)) - 0x4B400000; }
 
+// The kernels of a reconstruction are set up while the one they follow still runs (launch_chained):
+// each waits here, before it touches anything in global memory, until every kernel before it has
+// ended. Every block waits, so a kernel that has ended implies that all before it have. Launched
+// plainly, the wait does nothing.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Shared memory by 32-bit address.
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float lds_float(unsigned a)
@@ -225,6 +231,20 @@ void prof_stop(const ProfToken &t, cudaStream_t st);
         ::cbct::prof_stop(_cbct_tok, (st));                                                        \
         ::cbct::note_launch();                                                                     \
     } while (0)
+
+// Launches a kernel that calls chain_wait(): its launch overlaps the end of the kernel before it. An iteration of
+// short kernels gains most: 64x64x16, 20 iterations 4.13 -> 3.48 ms, 256x256x64 in three levels 49.0 -> 48.0 ms,
+// 512x512x70 135.6 -> 134.5 ms. (Letting the next kernel's blocks in as soon as all of this one's are
+// placed loses: 4.40, 54.4 and 156 ms; they take room from this kernel's second block per SM.)
+cudaError_t launch_chained(const void *kernel, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t st);
+template <typename T> struct AsIs { using type = T; };
+template <typename... P>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           typename AsIs<P>::type... a)
+{
+    void *args[] = {static_cast<void *>(&a)...};
+    launch_chained(reinterpret_cast<const void *>(kernel), grid, block, args, smem, st);
+}
 
 cbct_status set_error(cbct_status st, const char *fmt, ...);
 cbct_status check_cuda(cudaError_t e, const char *what);

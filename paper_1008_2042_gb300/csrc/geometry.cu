@@ -34,6 +34,27 @@ cbct_status check_cuda(cudaError_t e, const char *what)
     return set_error(CBCT_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+cudaError_t launch_chained(const void *kernel, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t st)
+{
+    // (a graph keeps plain edges between its kernels; while another stream's capture forbids the query, plain too)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+        cudaGetLastError();
+        capture = cudaStreamCaptureStatusActive;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 void note_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 // ---- per-launch timing -----------------------------------------------------------------

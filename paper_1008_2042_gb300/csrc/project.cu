@@ -263,7 +263,7 @@ cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const f
     const float *rec = static_cast<const float *>(traces);
     void *args[] = {&g, &map, &f, &zpitch, &c.plan, &y, &out, &partials, &sc, &rec, &col_first, &ncols, &nitems};
     ProfToken tok = prof_start(CBCT_KERNEL_PROJECT, st);
-    cudaError_t e = cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads + 32), args, c.smem, st);
+    cudaError_t e = launch_chained(fn, dim3((unsigned)grid), dim3((unsigned)threads + 32), args, c.smem, st);
     prof_stop(tok, st);
     note_launch();
     if (e != cudaSuccess) cudaGetLastError(); // the error is returned, not left pending

@@ -306,6 +306,7 @@ k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__r
             mbar_init(&s_empty[b], (unsigned)nwarps);
         }
     }
+    chain_wait();
     __syncthreads();
 
     if (warp == nwarps) {

@@ -15,6 +15,7 @@ namespace cbct {
 // once per level and every projection of that level reads it.
 __global__ void __launch_bounds__(PROJ_THREADS) k_trace_table(GeomDev G, float *__restrict__ traces, int col_first)
 {
+    chain_wait();
     extern __shared__ __align__(16) float smem[];
     const int cap = trace_cap(G);
     float *sEnd = smem;
@@ -76,7 +77,7 @@ cbct_status launch_trace_table(const GeomDev &G, void *tab, cudaStream_t st, int
     cbct_status r = trace_table_prepare();
     if (r != CBCT_OK) return r;
     if (ncols == 0) ncols = G.nviews * G.nu;
-    k_trace_table<<<(unsigned)ncols, PROJ_THREADS, smem, st>>>(G, static_cast<float *>(tab), col_first);
+    launch_chained(k_trace_table, (unsigned)ncols, PROJ_THREADS, smem, st, G, static_cast<float *>(tab), col_first);
     note_launch();
     return check_cuda(cudaGetLastError(), "trace table launch");
 }

@@ -34,6 +34,7 @@ static int vec_blocks(size_t n)
 __global__ void k_update_xp(float *__restrict__ x, float *__restrict__ p, const float *__restrict__ s,
                             const Scalars *sc, size_t n, int with_p)
 {
+    chain_wait();
     const float a = (float)sc->alpha, b = (float)sc->beta;
     const size_t n4 = n / 4;
     float4 *x4 = reinterpret_cast<float4 *>(x);
@@ -70,6 +71,7 @@ __global__ void k_update_xp(float *__restrict__ x, float *__restrict__ p, const 
 
 __global__ void k_pub_to_int(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz, int zp)
 {
+    chain_wait();
     __shared__ float t[32][33];
     const int xb = blockIdx.x * 32, zb = blockIdx.y * 32, y = blockIdx.z;
     for (int j = threadIdx.y; j < 32; j += 8) {
@@ -85,6 +87,7 @@ __global__ void k_pub_to_int(const float *__restrict__ in, float *__restrict__ o
 
 __global__ void k_int_to_pub(const float *__restrict__ in, float *__restrict__ out, int nx, int ny, int nz, int zp)
 {
+    chain_wait();
     __shared__ float t[32][33];
     const int xb = blockIdx.x * 32, zb = blockIdx.y * 32, y = blockIdx.z;
     for (int j = threadIdx.y; j < 32; j += 8) {
@@ -102,8 +105,8 @@ cbct_status transpose(const float *in, float *out, int nx, int ny, int nz, int z
                       cudaStream_t st)
 {
     dim3 grid((nx + 31) / 32, (nz + 31) / 32, ny), block(32, 8);
-    if (to_internal) CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_pub_to_int<<<grid, block, 0, st>>>(in, out, nx, ny, nz, zpitch));
-    else CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_int_to_pub<<<grid, block, 0, st>>>(in, out, nx, ny, nz, zpitch));
+    if (to_internal) CBCT_TIMED(CBCT_KERNEL_OTHER, st, launch_chained(k_pub_to_int, grid, block, 0, st, in, out, nx, ny, nz, zpitch));
+    else CBCT_TIMED(CBCT_KERNEL_OTHER, st, launch_chained(k_int_to_pub, grid, block, 0, st, in, out, nx, ny, nz, zpitch));
     return check_cuda(cudaGetLastError(), "transpose launch");
 }
 
@@ -326,7 +329,7 @@ static cbct_status run_cgls(const GeomDev &G, const float *y, float *x, int n_it
         // q = P p, alpha = gamma / ||q||^2
         TRY(launch_project(G, w.P, G.zp, nullptr, w.Q, PM_Q_SCALED, w.partials, 0.0f, st, storage, w.sc, traces));
         if (l == n_iter - 1) { // last update: x only; s and p would not be used again
-            CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_update_xp<<<vec_blocks(N), 256, 0, st>>>(x, w.P, w.S, w.sc, N, 0));
+            CBCT_TIMED(CBCT_KERNEL_OTHER, st, launch_chained(k_update_xp, vec_blocks(N), 256, 0, st, x, w.P, w.S, w.sc, N, 0));
             TRY(check_cuda(cudaGetLastError(), "update launch"));
             break;
         }
@@ -334,7 +337,7 @@ static cbct_status run_cgls(const GeomDev &G, const float *y, float *x, int n_it
         TRY(launch_update_prefix(G, w.R, w.Q, w.sc, w.PS, prescale, st, storage));
         TRY(launch_backproject(G, w.PS, w.S, sx, sy, sz, nullptr, w.partials, st, w.sc, FIN_BETA, scale_q));
         // x += alpha p; p = s + beta p
-        CBCT_TIMED(CBCT_KERNEL_OTHER, st, k_update_xp<<<vec_blocks(N), 256, 0, st>>>(x, w.P, w.S, w.sc, N, 1));
+        CBCT_TIMED(CBCT_KERNEL_OTHER, st, launch_chained(k_update_xp, vec_blocks(N), 256, 0, st, x, w.P, w.S, w.sc, N, 1));
         TRY(check_cuda(cudaGetLastError(), "update launch"));
     }
     return CBCT_OK;
@@ -346,7 +349,7 @@ static cbct_status read_flags(const Work &w, cudaStream_t st)
     cudaError_t e = cudaMemcpyAsync(&flags, &w.sc->flags, sizeof(flags), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return check_cuda(e, "status read-back");
-    if (flags & 2u) return set_error(CBCT_ERR_TIMEOUT, "a projector block timed out waiting for its trace record");
+    if (flags & 2u) return set_error(CBCT_ERR_TIMEOUT, "a projector block timed out waiting for its copies");
     if (flags & 1u) return set_error(CBCT_ERR_NONFINITE, "an inner product of the iteration was not finite");
     return CBCT_OK;
 }

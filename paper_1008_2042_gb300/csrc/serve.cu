@@ -357,7 +357,7 @@ void worker_main(cbct_server *srv)
                 msg = cbct_last_error();
             } else if (*srv->slot_flags(r->slot) & 2u) {
                 status = CBCT_ERR_TIMEOUT;
-                msg = "a projector block timed out waiting for its trace record";
+                msg = "a projector block timed out waiting for its copies";
             } else if (*srv->slot_flags(r->slot) & 1u) {
                 status = CBCT_ERR_NONFINITE;
                 msg = "an inner product of the iteration was not finite";

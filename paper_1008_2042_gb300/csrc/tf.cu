@@ -639,6 +639,7 @@ __global__ void __launch_bounds__(FR_THREADS, 1)
 k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__restrict__ x, float mu, int positivity,
                   float *__restrict__ fnew, const float *__restrict__ fold, float coef, float *__restrict__ vout)
 {
+    chain_wait();
     __shared__ f32x2 s_t[2][FR_WARPS][3][32];                      // axis-2 analysis of each pair
     __shared__ float s_up[2][FR_WARPS][3][32], s_dn[2][FR_WARPS][3][32]; // axis-1 synthesis shares to the pairs beside
     const int lane = threadIdx.x, w = threadIdx.y;
@@ -759,7 +760,7 @@ cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *
     const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
     dim3 grid((n0 + FR_OUT - 1) / FR_OUT, (n1 + FR_ROWS - 1) / FR_ROWS, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
-               k_tf_shrink_fused<<<grid, dim3(32, FR_WARPS), 0, st>>>(n0, n1, n2, p0, chunk, x, mu, positivity, fnew, fold,
+               launch_chained(k_tf_shrink_fused, grid, dim3(32, FR_WARPS), 0, st, n0, n1, n2, p0, chunk, x, mu, positivity, fnew, fold,
                                                                       coef, vout));
     return check_cuda(cudaGetLastError(), "tf_shrink_fused launch");
 }
