@@ -18,12 +18,12 @@
 // same plane coordinates and reciprocals as the projector's, so both operators use the same
 // weights to FP32 rounding. No atomics: the result is independent of scheduling.
 //
-// What bounds it on the paper's finest grid (512x512x70, 40 views, 1.16 ms, 14 voxels per
+// What bounds it on the paper's finest grid (512x512x70, 40 views, 1.18 ms, 14 voxels per
 // thread): issue slots 80% (1.15e9 warp instructions, three fifths of them the plane loop's) and
 // L1 data wavefronts 67% (the table's lines: lanes of a patch read about ten sectors). Before the
 // straddling row became one saturating multiply and the chunks whole it took 1.63 ms, with
 // the plane heights computed for each plane 1.25 ms; with the warps of a block on the same
-// patch taking turns at the views, 128x128x18 takes 99 us (200 before), 64x64x16 22 us (61).
+// patch taking turns at the views, 128x128x18 takes 100 us (200 before), 64x64x16 22 us (61).
 #include "cbct_internal.cuh"
 
 #include <cmath>
@@ -133,7 +133,8 @@ struct BpChunk {
 // and slab z receives the difference of its two planes,
 //     (tb - ta) ((P[a_{z+1}] - P[a_z]) + g_{z+1} f_{z+1} - g_z f_z),
 // with f the fraction of [ta, tb] that row a spends below the plane. f comes from the
-// crossing tau = zp / v - tc by one saturating multiply: where row a lies beyond the window, tau lies
+// crossing tau = zp / v - tc (rounded as the projector rounds it: subtracting tc + ta at once saves 1% of
+// the time, but its error grows by a tenth) by one saturating multiply: where row a lies beyond the window, tau lies
 // beyond [ta, tb] on the side where f is 0, so no test of the window's end is needed.
 // SIDE +1 / -1: row a of every plane has v > 0 / v < 0 (it rises / falls); 0: tested per row.
 // CLAMP: windows may leave the imager (rows clamped to [0, nv]; entry nv has value 0).
@@ -142,7 +143,6 @@ template <int ZC, int SIDE, bool CLAMP, bool FULL>
 __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, const BpChunk &c, float (&acc)[ZC])
 {
     const float w = q.tb - q.ta, winv = __fdividef(1.0f, w);
-    const float sa = G.tc + q.ta, sb = G.tc + q.tb;
     const float lo = SIDE < 0 ? q.A : q.B, x0 = fmaf(c.zs_bot, lo, c.c0), xs = c.dzs * lo;
     auto plane = [&](int z, float &P, float &g, float &f) {
         const float zp = fmaf((float)z, G.dz, c.zbot);
@@ -157,12 +157,12 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
         const int a = __float_as_int(__fadd_ru(x, 12582912.0f)); // ROUND_BIAS + ceil(x)
         const float2 T = __ldg(reinterpret_cast<const float2 *>(q.tab + (long long)a * q.row_bytes));
         const float iw = lds_float(q.iv + 4u * (unsigned)a);
-        if (SIDE > 0) {
-            f = __saturatef(fmaf(zp, iw, -sa) * winv);
-        } else if (SIDE < 0) {
-            f = __saturatef(fmaf(-zp, iw, sb) * winv);
+        if (SIDE < 0) {
+            f = __saturatef((q.tb - fmaf(zp, iw, -G.tc)) * winv);
         } else {
-            f = __saturatef(fmaf(zp, iw, -sa) * winv);
+            f = __saturatef((fmaf(zp, iw, -G.tc) - q.ta) * winv);
+        }
+        if (SIDE == 0) {
             if (!(iw > 0.0f)) f = 1.0f - f;
         }
         P = T.x;
@@ -177,7 +177,7 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
         // for both: the heights' arithmetic costs them issue slots and registers (512x512x70, 14
         // voxels: 1181 us, computed 1251 us; 512x512x128: 1991 | 2166 us). Chunks of 8 have the
         // registers and little to hide the load behind (64x64x16: 24.6 us, computed 22.6 us).
-        const float edge = SIDE > 0 ? -sa : sb;
+        const float tc = SIDE > 0 ? -G.tc : G.tc, edge = SIDE > 0 ? q.ta : -q.tb;
 #pragma unroll
         for (int z = 0; z < ZC; z += 2) {
             const int a1 = __float_as_int(__fadd_ru(fmaf((float)(z + 1), xs, x0), 12582912.0f));
@@ -187,8 +187,9 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
             float2 zp;
             if constexpr (LOOKUP) zp = lds_float2(c.zpairs + 4u * (unsigned)z);
             else zp = make_float2(SIDE * fmaf((float)(z + 1), G.dz, c.zbot), SIDE * fmaf((float)(z + 2), G.dz, c.zbot));
-            const float f1 = __saturatef(fmaf(zp.x, lds_float(q.iv + 4u * (unsigned)a1), edge) * winv);
-            const float f2 = __saturatef(fmaf(zp.y, lds_float(q.iv + 4u * (unsigned)a2), edge) * winv);
+            const float t1 = fmaf(zp.x, lds_float(q.iv + 4u * (unsigned)a1), tc);
+            const float t2 = fmaf(zp.y, lds_float(q.iv + 4u * (unsigned)a2), tc);
+            const float f1 = __saturatef((t1 - edge) * winv), f2 = __saturatef((t2 - edge) * winv);
             const float g1 = f1 > 0.0f ? T1.y : 0.0f, g2 = f2 > 0.0f ? T2.y : 0.0f;
             acc[z] = fmaf(w, fmaf(-g0, f0, fmaf(g1, f1, T1.x - P0)), acc[z]);
             acc[z + 1] = fmaf(w, fmaf(-g1, f1, fmaf(g2, f2, T2.x - T1.x)), acc[z + 1]);
