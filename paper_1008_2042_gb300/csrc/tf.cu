@@ -274,6 +274,25 @@ k_tf_analyze_pair(int n0, int n1, int n2, int chunk, const float *__restrict__ f
     }
 }
 
+// Resident blocks of a kernel on the whole device. The kernel's occupancy is asked for once per
+// device (`cache`, one per kernel): the query costs about as much host time as a launch.
+using Residency = std::atomic<int>[64];
+static cudaError_t resident_blocks(const void *kernel, int threads, Residency &cache, int *slots)
+{
+    int dev = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) per_sm = cache[dev].load(std::memory_order_relaxed);
+    if (!per_sm) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) per_sm = 1;
+        if (dev < 64) cache[dev].store(per_sm, std::memory_order_relaxed);
+    }
+    *slots = per_sm * device_sm_count();
+    return cudaSuccess;
+}
+
 // Planes per block along axis 2 (shrink + synthesis and the fused step): the split whose blocks fill whole
 // waves of the resident slots best, counting the two extra planes each block recomputes
 // at its start (a block's cost grows with chunk + 2).
@@ -411,11 +430,12 @@ static cbct_status launch_tf_analyze_t(int n0, int n1, int n2, const float *f, T
     const bool pair = n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & (2 * sizeof(TA_T) - 1)) == 0;
     const auto kernel = pair ? k_tf_analyze_pair<TA_T> : k_tf_analyze<TA_T>;
     const int ta = pair ? 64 : TA, tb = pair ? AP_B : TB;
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * tb, 0);
+    static Residency residency[2];
+    int slots = 0;
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(kernel), 32 * tb, residency[pair], &slots);
     if (e != cudaSuccess) return check_cuda(e, "tf_analyze occupancy");
     const long long tiles = (long long)((n0 + ta - 1) / ta) * ((n1 + tb - 1) / tb);
-    const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
+    const int chunk = fused_chunk(tiles, n2, slots);
     dim3 grid((n0 + ta - 1) / ta, (n1 + tb - 1) / tb, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_ANALYZE, st, kernel<<<grid, dim3(32, tb), 0, st>>>(n0, n1, n2, chunk, f, alpha));
     return check_cuda(cudaGetLastError(), "tf_analyze launch");
@@ -538,11 +558,12 @@ static cbct_status launch_tf_synth_shrink_pair(int n0, int n1, int n2, const T *
                                                float *f, cudaStream_t st)
 {
     constexpr int rows = SP_ROWS;
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_synth_shrink_pair<T>, 32 * SP_WARPS, 0);
+    static Residency residency;
+    int slots = 0;
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_synth_shrink_pair<T>), 32 * SP_WARPS, residency, &slots);
     if (e != cudaSuccess) return check_cuda(e, "tf_synth_shrink occupancy");
     const long long tiles = (long long)((n0 + SP_OUT - 1) / SP_OUT) * ((n1 + rows - 1) / rows);
-    const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
+    const int chunk = fused_chunk(tiles, n2, slots);
     dim3 grid((n0 + SP_OUT - 1) / SP_OUT, (n1 + rows - 1) / rows, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
                k_tf_synth_shrink_pair<T><<<grid, dim3(32, SP_WARPS), 0, st>>>(n0, n1, n2, chunk, alpha, mu, positivity, f));
@@ -558,11 +579,12 @@ static cbct_status launch_tf_synth_shrink_t(int n0, int n1, int n2, const TA_T *
     if constexpr (sizeof(TA_T) == 2)
         if (n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & 3) == 0 && (reinterpret_cast<uintptr_t>(f) & 7) == 0)
             return launch_tf_synth_shrink_pair(n0, n1, n2, alpha, mu, positivity, f, st);
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_synth_shrink<TA_T>, SY_THREADS, 0);
+    static Residency residency;
+    int slots = 0;
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_synth_shrink<TA_T>), SY_THREADS, residency, &slots);
     if (e != cudaSuccess) return check_cuda(e, "tf_synth_shrink occupancy");
     const long long tiles = (long long)((n0 + SY_OUT - 1) / SY_OUT) * ((n1 + SY_ROWS - 1) / SY_ROWS);
-    const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
+    const int chunk = fused_chunk(tiles, n2, slots);
     dim3 grid((n0 + SY_OUT - 1) / SY_OUT, (n1 + SY_ROWS - 1) / SY_ROWS, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
                k_tf_synth_shrink<TA_T><<<grid, dim3(32, SY_WARPS), 0, st>>>(n0, n1, n2, chunk, alpha, mu, positivity, f));
@@ -753,11 +775,12 @@ cbct_status tf_prepare() { return CBCT_OK; }
 cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *x, float mu, int positivity, float *fnew,
                                    const float *fold, float coef, float *vout, cudaStream_t st)
 {
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tf_shrink_fused, FR_THREADS, 0);
+    static Residency residency;
+    int slots = 0;
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_shrink_fused), FR_THREADS, residency, &slots);
     if (e != cudaSuccess) return check_cuda(e, "tf_shrink_fused occupancy");
     const long long tiles = (long long)((n0 + FR_OUT - 1) / FR_OUT) * ((n1 + FR_ROWS - 1) / FR_ROWS);
-    const int chunk = fused_chunk(tiles, n2, (per_sm > 0 ? per_sm : 1) * device_sm_count());
+    const int chunk = fused_chunk(tiles, n2, slots);
     dim3 grid((n0 + FR_OUT - 1) / FR_OUT, (n1 + FR_ROWS - 1) / FR_ROWS, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
                launch_chained(k_tf_shrink_fused, grid, dim3(32, FR_WARPS), 0, st, n0, n1, n2, p0, chunk, x, mu, positivity, fnew, fold,
