@@ -19,12 +19,15 @@
 // weights to FP32 rounding. No atomics: the result is independent of scheduling.
 //
 // What bounds it on the paper's finest grid (512x512x70, 40 views, 1.18 ms, 14 voxels per
-// thread): issue slots 80% (1.15e9 warp instructions, three fifths of them the plane loop's) and
+// thread): issue slots 80% (1.14e9 warp instructions, three fifths of them the plane loop's) and
 // L1 data wavefronts 67% (the table's lines: lanes of a patch read about ten sectors). Before the
 // straddling row became one saturating multiply and the chunks whole it took 1.63 ms, with
 // the plane heights computed for each plane 1.25 ms; with the warps of a block on the same
-// patch taking turns at the views, 128x128x18 takes 100 us (200 before), 64x64x16 22 us (61).
+// patch taking turns at the views, 128x128x18 takes 103 us (200 before), 64x64x16 21 us (61).
+// Chunks that begin or end at z = 0 take the loops of one side: 256x256x64 457 -> 395 us, 128x128x32 145 -> 119 us.
 #include "cbct_internal.cuh"
+
+#include <math_constants.h>
 
 #include <cmath>
 
@@ -51,10 +54,11 @@ struct BpPlan {
 constexpr int BP_MAX_WARPS = 16;
 constexpr int BP_ZC[] = {8, 12, 14, 16, 18};
 
-// The voxels per thread that cover a column with the fewest planes (about one and a half more per
-// chunk for its first plane and set-up); measured at 512x512x70 (12 | 14 | 16 | 18): 1268 | 1183 | 1321 |
-// 1249 us, 128x128x18 137 | 154 | 172 | 100 us, 256x256x35 320 | 350 | 400 | 340 us (three chunks of 12
-// have 36 planes like two of 18: the tail of the last wave is shorter). Where even 8 slices leave few warps, 8 voxels
+// The voxels per thread that cover a column at the least cost: its planes, about one and a half more per
+// chunk for its first plane and set-up, and a third more for a chunk that z = 0 cuts (its
+// rows are tested one by one). Measured (12 | 14 | 16 | 18): 512x512x70 1268 | 1183 | 1321 | 1249 us, 128x128x18
+// 137 | 154 | 172 | 100 us, 256x256x64 (meeting at z = 0 for 16 only) 503 | 470 | 395 | 493 us, 256x256x35 (one of three
+// chunks of 12 cut, both of 18) 320 | 350 | 400 | 349 us. Where even 8 slices leave few warps, 8 voxels
 // (64x64x16: 24.6 us, with 16 32.8 us). Slices double until the chip has about 96 warps per
 // SM to draw from: 256x256x35 with 1 | 2 | 4 | 8 slices 403 | 354 | 339 | 356 us, 128x128x18 456 |
 // 240 | 131 | 104 us, 512x512x70 1254 | 1311 | 1393 | 1583 us (less of the table is shared in L1).
@@ -63,9 +67,17 @@ static BpPlan bp_plan(const GeomDev &G)
     BpPlan p{};
     const long long patches = (long long)((G.nx + BP_WX - 1) / BP_WX) * ((G.ny + BP_WY - 1) / BP_WY);
     const long long sms = device_sm_count();
-    int chunks = 0, best = 1 << 30;
+    int chunks = 0;
+    double best = 1e30;
+    const double orbit = -(double)G.z0 / G.dz; // the plane z = 0
     for (int zc : BP_ZC) {
-        const int n = (G.nz + zc - 1) / zc, cost = n * (2 * zc + 3);
+        const int n = (G.nz + zc - 1) / zc;
+        double cost = 0.0;
+        for (int c = 0; c < n; ++c) {
+            const int z = G.nz < zc ? 0 : c * zc < G.nz - zc ? c * zc : G.nz - zc;
+            const bool cut = z < orbit && orbit < z + zc;
+            cost += (zc + 1.5) * (cut ? 4.0 / 3.0 : 1.0);
+        }
         if (cost < best) {
             best = cost;
             p.zc = zc;
@@ -220,13 +232,15 @@ __global__ void __launch_bounds__(32 * BP_MAX_WARPS, 2)
 k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz, int slices,
               float *__restrict__ out2, double *__restrict__ partials, Scalars *__restrict__ sc, int fin_op, int scale_q)
 {
-    extern __shared__ float smem[]; // 1 / v per imager row (one more for entry nv); then the slices' sums
+    // 1 / v per imager row (one more for entry nv); the same with -inf where v >= 0, for falling chunks; the slices' sums
+    extern __shared__ float smem[];
     __shared__ double s_warp[BP_MAX_WARPS];
-    float *s_invv = smem, *s_sum = smem + G.nv + 1;
+    float *s_invv = smem, *s_sum = smem + 2 * (G.nv + 1);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i <= G.nv; i += blockDim.x) {
         const float v = imager_v(G, i);
         s_invv[i] = v != 0.0f ? __frcp_rn(v) : 1e30f;
+        s_invv[G.nv + 1 + i] = v < 0.0f ? __frcp_rn(v) : -CUDART_INF_F;
     }
 
     const int npatch = (blockDim.x >> 5) / slices, slice = warp / npatch, patch = warp - slice * npatch;
@@ -258,6 +272,9 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
     const float c1 = fmaf(-G.v_first, G.inv_dv, 1e-3f);
     const size_t view_stride = ((size_t)G.nv + 1) * G.nu;
     const unsigned iv0 = smem_u32(s_invv) - 4u * (unsigned)ROUND_BIAS;
+    // Side +1: the window of the lowest plane, hence of every plane, starts at a row with
+    // v / dv >= zs B - 1e-3; where the first row from -1e-3 on has v > 0, z = 0 will do.
+    const float zs_rise = ch.zs_bot == 0.0f && imager_v(G, (int)ceilf(ch.c0)) > 0.0f ? 1.0f : ch.zs_bot;
 
     // imager columns in the shadow of the voxel column in view k (its corners' u); the least and
     // greatest u / sdd, scaled once (scaled corner by corner 1181 us at 512x512x70, so 1163)
@@ -302,18 +319,23 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
             // in the plane height, so these bound every plane's window)
             const bool inside = fmaf(ch.zs_bot, ch.zs_bot >= 0.0f ? B : A, ch.c0) >= 0.0f &&
                                 fmaf(zs_top, zs_top >= 0.0f ? A : B, c1) <= (float)(G.nv - 1);
-            // Side +1: the window of the lowest plane, hence of every plane, starts at a row
-            // with v / dv >= zs B - 1e-3 > 0, and so does every row at or above a window's start;
-            // side -1: every window ends more than a row below v = 0, so that the first row
-            // above a window's start has v < 0 even where it lies beyond the window.
-            const int side = !inside ? 0 : ch.zs_bot * B > 2e-3f ? 1 : zs_top * B < -1.002f ? -1 : 0;
+            // Side -1: every plane has z <= 0. A row at a window's start then has v < 0, or lies beyond the
+            // window with v >= 0, where -inf instead of 1 / v gives it no part (at z = 0 as well: 0 * inf
+            // saturates to 0).
+            const int side = !inside ? 0 : zs_rise * B > 2e-3f ? 1 : zs_top <= 0.0f ? -1 : 0;
             q.row_bytes = 8 * G.nu;
             q.tab = reinterpret_cast<const char *>(ps + entry) - (long long)ROUND_BIAS * q.row_bytes;
             if (ch.nzc == ZC) {
-                ch.zpairs = smem_u32(s_z[side < 0]);
-                if (side > 0) bp_planes<ZC, 1, false, true>(G, q, ch, acc);
-                else if (side < 0) bp_planes<ZC, -1, false, true>(G, q, ch, acc);
-                else bp_planes<ZC, 0, true, true>(G, q, ch, acc);
+                if (side > 0) {
+                    ch.zpairs = smem_u32(s_z[0]);
+                    bp_planes<ZC, 1, false, true>(G, q, ch, acc);
+                } else if (side < 0) {
+                    ch.zpairs = smem_u32(s_z[1]);
+                    q.iv += 4u * (unsigned)(G.nv + 1);
+                    bp_planes<ZC, -1, false, true>(G, q, ch, acc);
+                } else {
+                    bp_planes<ZC, 0, true, true>(G, q, ch, acc);
+                }
             } else {
                 bp_planes<ZC, 0, true, false>(G, q, ch, acc);
             }
@@ -438,14 +460,15 @@ static const void *bp_kernel(int zc, bool flat)
     }
 }
 
-// The shared-memory opt-in of every instantiation, once per device: at most 33 KB of rows (nv <= 8192)
+// The shared-memory opt-in of every instantiation, once per device: at most 66 KB of rows (nv <= 8192)
 // and 34 KB of the slices' sums (7/8 of 512 threads, 18 voxels).
+constexpr int BP_SMEM_LIMIT = 104 * 1024;
 cbct_status backproject_prepare()
 {
     static std::atomic<unsigned long long> done[sizeof(BP_ZC) / sizeof(int)][2];
     for (int i = 0; i < (int)(sizeof(BP_ZC) / sizeof(int)); ++i)
         for (int flat = 0; flat < 2; ++flat) {
-            const cudaError_t e = smem_optin_once(bp_kernel(BP_ZC[i], flat != 0), 72 * 1024, done[i][flat]);
+            const cudaError_t e = smem_optin_once(bp_kernel(BP_ZC[i], flat != 0), BP_SMEM_LIMIT, done[i][flat]);
             if (e != cudaSuccess) return check_cuda(e, "backproject attribute");
         }
     return CBCT_OK;
@@ -461,7 +484,7 @@ cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, l
     const bool flat = sqrtf(G.dx * G.dx + G.dy * G.dy) * (G.sdd / G.sad) < 1.5f * G.du;
     const cbct_status r = backproject_prepare();
     if (r != CBCT_OK) return r;
-    const size_t smem = sizeof(float) * ((size_t)G.nv + 1 + (size_t)(p.slices - 1) * p.zc * (p.warps / p.slices) * 32);
+    const size_t smem = sizeof(float) * (2 * ((size_t)G.nv + 1) + (size_t)(p.slices - 1) * p.zc * (p.warps / p.slices) * 32);
     GeomDev g = G;
     int isx = (int)sx, isy = (int)sy, isz = (int)sz;
     void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials, &sc, &fin_op, &scale_q};

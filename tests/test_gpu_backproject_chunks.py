@@ -47,6 +47,19 @@ def test_backproject_parity_at_chunk_edges(cb, nz, views):
     assert np.linalg.norm(b - ref) <= 1e-4 * np.linalg.norm(ref)
 
 
+# imager rows at v = 0 +- 0.0005 pitches, and away from it, against chunks that begin and end at z = 0
+@pytest.mark.parametrize("v_off", [0.65 - 0.00065, 0.65 + 0.00065, 0.1])
+@pytest.mark.parametrize("nz", [16, 24, 28, 32, 36, 64])
+def test_chunks_that_meet_at_the_orbit_plane(cb, nz, v_off):
+    g = synth.Geometry(nx=37, ny=21, nz=nz, dx=1.0, dy=1.1, dz=1.2, nu=33, nv=120, du=1.7, dv=1.3, u_off=0.6, v_off=v_off,
+                       n_views=5, angles=tuple(0.17 + 2 * np.pi * np.arange(5) / 5))
+    y = synth.random_projections(g, 80)
+    with cb.Geometry(g) as h:
+        b = cb.backproject(h, dev(y)).cpu().numpy()
+    ref = oracle.backproject(g, y)
+    assert np.linalg.norm(b - ref) <= 1e-4 * np.linalg.norm(ref)
+
+
 def test_wide_grid_of_whole_chunks(cb):
     """Enough columns for one slice per patch, 70 = 5 x 14 voxels, sampled voxels in the oracle."""
     g = synth.Geometry(nx=640, ny=600, nz=70, dx=0.4, dy=0.4, dz=1.0, nu=40, nv=60, du=9.7, dv=2.1, u_off=0.6, v_off=-0.35,
