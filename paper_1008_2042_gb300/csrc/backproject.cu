@@ -229,7 +229,7 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
 // shadows are about one column wide.
 template <int ZC, bool FLAT>
 __global__ void __launch_bounds__(32 * BP_MAX_WARPS, 2)
-k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz, int slices,
+k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out, int sx, int sy, int sz, int slices, float span_lim,
               float *__restrict__ out2, double *__restrict__ partials, Scalars *__restrict__ sc, int fin_op, int scale_q)
 {
     // 1 / v per imager row (one more for entry nv); the same with -inf where v >= 0, for falling chunks; the slices' sums
@@ -306,9 +306,10 @@ k_backproject(GeomDev G, const float2 *__restrict__ ps, float *__restrict__ out,
         const size_t entry = (size_t)k * view_stride + iu; // row m's entry: ps[entry + m * nu]
         // Plane z = zp is reached by the rows with v between zp*A and zp*B. While that
         // window is shorter than a row pitch and adjacent planes' windows are apart,
-        // every row crosses at most one plane inside the column (the usual case).
+        // every row crosses at most one plane inside the column (the usual case; span_lim is 1
+        // row, or 0 where the plane loop's row step does not fit, see the launcher).
         const float span = zabs * (A - B) * G.inv_dv;
-        if (span + 3e-3f < 1.0f && fmaf(G.dz * B, G.inv_dv, -span) > 3e-3f) {
+        if (span + 3e-3f < span_lim && fmaf(G.dz * B, G.inv_dv, -span) > 3e-3f) {
             BpVisit q;
             q.iv = iv0;
             q.ta = ta;
@@ -485,9 +486,12 @@ cbct_status launch_backproject(const GeomDev &G, const float2 *ps, float *out, l
     const cbct_status r = backproject_prepare();
     if (r != CBCT_OK) return r;
     const size_t smem = sizeof(float) * (2 * ((size_t)G.nv + 1) + (size_t)(p.slices - 1) * p.zc * (p.warps / p.slices) * 32);
+    // The plane loop steps through the table by rows of 8 nu bytes held in 32 bits. Rows of 2 GiB or
+    // more take the row-by-row loop at every visit, whose offsets count entries ((nv + 1) nu of them).
+    float span_lim = G.nu < 1 << 28 ? 1.0f : 0.0f;
     GeomDev g = G;
     int isx = (int)sx, isy = (int)sy, isz = (int)sz;
-    void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &out2, &partials, &sc, &fin_op, &scale_q};
+    void *args[] = {&g, &ps, &out, &isx, &isy, &isz, &p.slices, &span_lim, &out2, &partials, &sc, &fin_op, &scale_q};
     ProfToken tok = prof_start(CBCT_KERNEL_BACKPROJECT, st);
     const cudaError_t e = launch_chained(bp_kernel(p.zc, flat), p.grid, dim3(32u * p.warps), args, smem, st);
     prof_stop(tok, st);
