@@ -589,7 +589,7 @@ k_row_prefix(GeomDev G, T *g, const T *__restrict__ q, const Scalars *__restrict
 template <typename T>
 static void row_prefix(const GeomDev &G, void *g, const void *q, const Scalars *sc, float2 *ps, int prescale, cudaStream_t st)
 {
-    const dim3 grid((G.nu + 31) / 32, G.nviews), block(32, PREFIX_WARPS);
+    const dim3 grid((G.nu - 1) / 32 + 1, G.nviews), block(32, PREFIX_WARPS); // (nu + 31 may pass 2^31)
     if (q)
         CBCT_TIMED(CBCT_KERNEL_OTHER, st,
                    launch_chained(k_row_prefix<T, true>, grid, block, 0, st, G, static_cast<T *>(g), static_cast<const T *>(q), sc, ps, prescale));

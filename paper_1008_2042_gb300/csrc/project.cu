@@ -237,8 +237,8 @@ cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const f
     const int threads = proj_threads(G), fill = fill_of(G, zpitch);
     const int rows = fill == FILL_GATHER ? proj_rows_per_thread(G) : 2;
     if (ncols == 0) ncols = G.nviews * G.nu;
-    // (views x columns < 2^31 / nv, so the items fit an int)
-    int nitems = ncols * ((G.nv + rows * threads - 1) / (rows * threads));
+    // (views x columns < 2^31 / nv, so the items fit 31 bits)
+    unsigned nitems = (unsigned)ncols * ((G.nv + rows * threads - 1) / (rows * threads));
     // the packed layout takes the padded one's plan: the same tables, hence the same sums
     GroupChoice c{};
     cbct_status r = choose_group(G, threads, mode, storage, fill_of(G, G.zp), &c);
@@ -258,12 +258,13 @@ cbct_status launch_project(const GeomDev &G, const float *f, int zpitch, const f
         r = line_map(G, f, c.plan.pitch, &map);
         if (r != CBCT_OK) return r;
     }
-    const int grid = nitems < c.grid ? nitems : c.grid;
+    const unsigned grid = nitems < (unsigned)c.grid ? nitems : (unsigned)c.grid;
+    unsigned ucols = (unsigned)ncols;
     GeomDev g = G;
     const float *rec = static_cast<const float *>(traces);
-    void *args[] = {&g, &map, &f, &zpitch, &c.plan, &y, &out, &partials, &sc, &rec, &col_first, &ncols, &nitems};
+    void *args[] = {&g, &map, &f, &zpitch, &c.plan, &y, &out, &partials, &sc, &rec, &col_first, &ucols, &nitems};
     ProfToken tok = prof_start(CBCT_KERNEL_PROJECT, st);
-    cudaError_t e = launch_chained(fn, dim3((unsigned)grid), dim3((unsigned)threads + 32), args, c.smem, st);
+    cudaError_t e = launch_chained(fn, dim3(grid), dim3((unsigned)threads + 32), args, c.smem, st);
     prof_stop(tok, st);
     note_launch();
     if (e != cudaSuccess) cudaGetLastError(); // the error is returned, not left pending

@@ -264,7 +264,8 @@ __device__ __forceinline__ void build_part(unsigned at, unsigned lp4, unsigned a
 }
 
 // Items (view, imager column, chunk of rows) first_item + blockIdx.x, + gridDim.x, ...: item i is
-// chunk i / ncols of column col_first + i % ncols, whose record is rec[i % ncols].
+// chunk i / ncols of column col_first + i % ncols, whose record is rec[i % ncols]. (Unsigned: the last
+// step of a block may pass 2^31.)
 // Per group of sg segments of an item's trace the lines become the table in place,
 // T[c][k] = sum of f(column, slab k) * length over the columns of c's part up to and
 // including c, with the sums of the parts before in O[part][k] (O[PARTS] is the group's
@@ -279,7 +280,7 @@ template <int MODE, typename TP, int QW, int R, int FILL>
 __global__ void __launch_bounds__(PROJ_THREADS + 32, CBCT_PROJ_MIN_BLOCKS)
 k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__restrict__ f, int zpitch, ProjPlan pl,
           const float *__restrict__ y, TP *__restrict__ out, double *__restrict__ partials, Scalars *__restrict__ sc,
-          const float *__restrict__ rec, int col_first, int ncols, int nitems)
+          const float *__restrict__ rec, int col_first, unsigned ncols, unsigned nitems)
 {
     constexpr int PARTS = 32 / QW;
     extern __shared__ __align__(128) float smem[];
@@ -311,7 +312,8 @@ k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__r
 
     if (warp == nwarps) {
         // ---- producer: one group ahead of the consumers, through all items ----
-        int item = blockIdx.x, g = 0, nitem = 0, nseg = 0;
+        unsigned item = blockIdx.x;
+        int g = 0, nitem = 0, nseg = 0;
         const float *r = nullptr;
         int4 col = make_int4(0, 0, 0, 0);          // four columns of the next group ...
         float4 end = make_float4(0.f, 0.f, 0.f, 0.f); // ... the tau at which they end ...
@@ -395,7 +397,7 @@ k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__r
     double red = 0.0;
     bool lost = false; // a wait of the block ran out: NaN rows from here on
     int s = 0, nitem = 0; // groups and items so far
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++nitem) {
+    for (unsigned item = blockIdx.x; item < nitems; item += gridDim.x, ++nitem) {
         const int chunk = item / ncols;
         int kz[R];
         float inv_v[R], tzn[R], acc[R];
@@ -512,7 +514,7 @@ k_project(GeomDev G, const __grid_constant__ CUtensorMap lines, const float *__r
         }
 
         // ---- epilogue of the item ----
-        const int column = col_first + item - chunk * ncols, view = column / G.nu, iu = column - view * G.nu;
+        const int column = col_first + (int)(item - chunk * ncols), view = column / G.nu, iu = column - view * G.nu;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int iv = chunk * (R * nthr) + r * nthr + tid;

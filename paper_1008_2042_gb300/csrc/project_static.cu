@@ -82,8 +82,8 @@ extern "C" cbct_status cbct_project_static(const cbct_geometry *g, const float *
     st = transpose(f, scratch, G.nx, G.ny, G.nz, zpitch, true, s);
     if (st != CBCT_OK) return st;
     const int ncols = G.nviews * G.nu, batch = (int)(STATIC_TRACE_BYTES / (trace_table_bytes(G) / ncols));
-    for (int c0 = 0; c0 < ncols; c0 += batch) {
-        const int n = ncols - c0 < batch ? ncols - c0 : batch;
+    for (int c0 = 0, n; c0 < ncols; c0 += n) { // (c0 never passes ncols, which may be close to 2^31)
+        n = ncols - c0 < batch ? ncols - c0 : batch;
         st = launch_trace_table(G, traces, s, c0, n);
         if (st != CBCT_OK) return st;
         st = launch_project(G, scratch, zpitch, nullptr, g_out, PM_PLAIN, nullptr, 0.0f, s, ST_F32, nullptr, traces,

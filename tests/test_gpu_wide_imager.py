@@ -1,8 +1,9 @@
-"""The adjoint on an imager whose rows of the prefix table are 2 GiB long (2^28 columns).
+"""Imagers at the widths where counts pass 32 bits: rows of the adjoint's prefix table of 2 GiB (2^28
+columns), and nearly 2^31 columns, which the allocation-free projection takes in batches.
 
 The volume's shadow lies in the first 41 columns, which a narrow imager repeats; every other column
-misses it, so its ones have no part in the result. Bar: the operators' relative L2 of 1e-4 against
-the FP64 oracle on the narrow imager."""
+misses it. The adjoint's bar is the operators' relative L2 of 1e-4 against the FP64 oracle on the
+narrow imager; the projections run the same sums in the same order and are equal."""
 import numpy as np
 import pytest
 
@@ -13,11 +14,11 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-U_FIRST, NARROW, WIDE = -19.7, 41, 1 << 28
+U_FIRST, NARROW, WIDE = -19.75, 41, 1 << 28
 
 
-def geom(nu):
-    return synth.Geometry(nx=7, ny=5, nz=6, dx=1.0, dy=1.1, dz=1.2, nu=nu, nv=3, du=1.0, dv=2.3, v_off=0.4, n_views=1,
+def geom(nu, nv=3):
+    return synth.Geometry(nx=7, ny=5, nz=6, dx=1.0, dy=1.1, dz=1.2, nu=nu, nv=nv, du=1.0, dv=2.3, v_off=0.4, n_views=1,
                           u_off=U_FIRST + 0.5 * (nu - 1), angles=(0.3,))
 
 
@@ -36,3 +37,21 @@ def test_backproject_with_table_rows_of_2_gib():
     with cb.Geometry(geom(WIDE)) as h:
         b = cb.backproject(h, wide).cpu().numpy()
     assert np.linalg.norm(b - ref) <= 1e-4 * np.linalg.norm(ref)
+
+
+def test_static_projection_of_nearly_2_31_columns():
+    import paper_1008_2042_gb300 as cb
+
+    cb.load_library()
+    if torch.cuda.mem_get_info()[0] < 72 << 30:
+        pytest.skip("needs 63 GB of device memory")
+    g, nu = geom(NARROW, nv=1), 2**31 - 2
+    f = torch.tensor(synth.random_volume(g, 84), dtype=torch.float32, device="cuda")
+    with cb.Geometry(g) as h:
+        p = cb.project(h, f)
+    assert int(torch.count_nonzero(p)) >= 5
+    with cb.Geometry(geom(nu, nv=1)) as h:
+        q = torch.full((1, 1, nu), float("nan"), dtype=torch.float32, device="cuda")
+        cb.project_static(h, f, q)
+    assert torch.equal(p, q[:, :, :NARROW])
+    assert int(torch.count_nonzero(q[:, :, NARROW:])) == 0
