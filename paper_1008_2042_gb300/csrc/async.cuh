@@ -32,7 +32,9 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned 
 }
 // Every wait ends: after WAIT_CYCLES (about two seconds), or once another warp of the
 // block has given up, it returns false, and the block then ends with NaN results and bit 1
-// of the iteration's status word instead of a hang.
+// of the iteration's status word instead of a hang. The verdict is the warp's: lanes may leave
+// the loop for different reasons, and a warp that went on with some of them would wait at its
+// next full-mask shuffle for the others. Called by whole warps.
 constexpr long long WAIT_CYCLES = 4000000000ll;
 __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, volatile int *give_up)
 {
@@ -42,8 +44,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
         while (!(ok = mbar_try_wait(bar, parity)) && !*give_up)
             if (clock64() - t0 > WAIT_CYCLES) *give_up = 1;
     }
-    __syncwarp();
-    return ok;
+    return __all_sync(0xffffffffu, ok);
 }
 // generic accesses of this thread to shared memory before, bulk copies into it after
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
