@@ -19,6 +19,7 @@
 namespace cbct {
 
 constexpr int TA = 32, TB = 8, TF_THREADS = TA * TB;
+constexpr int MAX_GRID_Y = 65535;
 constexpr float R2_4 = 0.35355339059327373f; // sqrt(2) / 4
 
 __device__ __forceinline__ int wrapi(int i, int n)
@@ -427,7 +428,9 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
 template <typename TA_T>
 static cbct_status launch_tf_analyze_t(int n0, int n1, int n2, const float *f, TA_T *alpha, cudaStream_t st)
 {
-    const bool pair = n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & (2 * sizeof(TA_T) - 1)) == 0;
+    // (the pair kernel's tiles of AP_B rows reach the grid's limit along y at half the rows that are accepted)
+    const bool pair = n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & (2 * sizeof(TA_T) - 1)) == 0 &&
+                      (n1 + AP_B - 1) / AP_B <= MAX_GRID_Y;
     const auto kernel = pair ? k_tf_analyze_pair<TA_T> : k_tf_analyze<TA_T>;
     const int ta = pair ? 64 : TA, tb = pair ? AP_B : TB;
     static Residency residency[2];
