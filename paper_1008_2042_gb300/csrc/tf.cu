@@ -640,10 +640,10 @@ constexpr int FR_OUT = 28;                // output positions per warp along axi
 constexpr int FR_THREADS = 32 * FR_WARPS;
 
 // The frame with plain taps: [1, 2, 1], [1, 0, -1] and [1, -2, 1] stand for 4 h_0, (4 / sqrt(2)) h_1
-// and -4 h_2, so that a triple takes four operations. A coefficient with j factors h_1 is then 64 /
-// sqrt(2)^j times the frame's (its sign is its own on both ways), the squared norm is the sum of
-// 2^j A^2 over 4096, and synthesis counts the middle tap triple twice and divides by 4096: all
-// powers of two, which round nothing.
+// and -4 h_2, so that a triple takes four operations. Of x / 64, a coefficient with j factors h_1 is then
+// 1 / sqrt(2)^j times the frame's (its sign is its own on both ways), the squared norm is the sum of
+// 2^j A^2, and synthesis counts the middle tap triple twice, of A / 64: all powers of two, which
+// round nothing (values below 2^-114 lose their last bits), and no intermediate is larger than the frame's.
 __device__ __forceinline__ void ana3_plain(f32x2 p, f32x2 c, f32x2 n, f32x2 &o0, f32x2 &o1, f32x2 &o2)
 {
     const f32x2 s = add2(n, p);
@@ -682,9 +682,10 @@ k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__rest
         const float *src = x + (size_t)wrapi(c, n2) * plane;
         return pk(__ldg(src + in0), __ldg(src + in1));
     };
+    const f32x2 r64 = splat(1.0f / 64.0f);
 
-    // x of these positions at planes cp - 1, cp, cp + 1 (cp: the analysed plane)
-    f32x2 xm = load(c_begin - 2), x0 = load(c_begin - 1), xp = load(c_begin);
+    // x / 64 of these positions at planes cp - 1, cp, cp + 1 (cp: the analysed plane)
+    f32x2 xm = mul2(load(c_begin - 2), r64), x0 = mul2(load(c_begin - 1), r64), xp = mul2(load(c_begin), r64);
     f32x2 w_m2[3] = {0ull, 0ull, 0ull}, w_m1[3] = {0ull, 0ull, 0ull}; // axis-2 synthesis inputs at cp-2, cp-1
     int buf = 0;
     for (int cp = c_begin - 1; cp <= c_end; ++cp, buf ^= 1) {
@@ -720,8 +721,9 @@ k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__rest
             sj[j] = fma2(al[ch], al[ch], sj[j]);
         }
         const f32x2 s2 = fma2(splat(2.0f), fma2(splat(2.0f), fma2(splat(2.0f), sj[3], sj[2]), sj[1]), sj[0]);
-        const float na = sqrtf(lo2(s2)), nb = sqrtf(hi2(s2)), mu64 = 64.0f * mu;
-        const f32x2 scale = pk(na > mu64 ? 1.0f - mu64 / na : 0.0f, nb > mu64 ? 1.0f - mu64 / nb : 0.0f);
+        const float na = sqrtf(lo2(s2)), nb = sqrtf(hi2(s2));
+        const f32x2 scale = mul2(pk(na > mu ? 1.0f - mu / na : 0.0f, nb > mu ? 1.0f - mu / nb : 0.0f), r64);
+        al[0] = mul2(al[0], r64);
 #pragma unroll
         for (int ch = 1; ch < 27; ++ch) al[ch] = mul2(al[ch], scale);
         // synthesis along axis 0 (lanes), then the shares along axis 1
@@ -751,7 +753,7 @@ k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__rest
                 const size_t idx = (size_t)(cp - 1) * plane + (size_t)pb * p0 + pa;
                 const f32x2 ends = add2(add2(w_m2[0], w_m2[2]), add2(wv[0], wv[2]));
                 const f32x2 o2 = fma2(splat(2.0f), add2(sub2(w_m1[0], w_m1[2]), sub2(w_m2[1], wv[1])), ends);
-                float o[2] = {lo2(o2) * (1.0f / 4096.0f), hi2(o2) * (1.0f / 4096.0f)};
+                float o[2] = {lo2(o2), hi2(o2)};
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     if (pb + r >= n1) break; // an odd number of rows
@@ -769,7 +771,7 @@ k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__rest
         }
         xm = x0;
         x0 = xp;
-        xp = xn;
+        xp = mul2(xn, r64); // (here and not at the load, which this plane's work hides)
     }
 }
 

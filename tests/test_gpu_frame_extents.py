@@ -1,7 +1,9 @@
-"""Frame transforms at the largest second extents (the grid's limit of blocks along y).
+"""Frame transforms at the largest second extents (the grid's limit of blocks along y) and over the
+range of values.
 
-The analysis is compared with the oracle: three passes of at
-most three roundings each with taps of absolute sum <= 1."""
+The analysis is compared with the oracle: three passes of at most three roundings each with taps of absolute
+sum <= 1. Scaling the values and the threshold by a power of two scales the result by it, bit for bit,
+as long as no square of a coefficient passes FP32's range (1.8e19); without a threshold, up to its end."""
 import numpy as np
 import pytest
 
@@ -26,3 +28,16 @@ def test_analysis_of_tall_planes(cb, ny):
     f = np.random.default_rng(5).standard_normal((1, ny, 2)).astype(np.float32)
     a = cb.tf_analyze(torch.from_numpy(f).cuda()).cpu().numpy()
     assert np.abs(a - oracle.tf_analyze(f)).max() <= 10 * 2.0**-24 * np.abs(f).max()
+
+
+def scaled(shape, k):
+    f = torch.randn(shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(6))
+    return f, f * 2.0**k
+
+
+@pytest.mark.parametrize("k, mu", [(-40, 1.5), (56, 1.5), (60, 1.5), (122, 0.0)])
+def test_range_of_the_fused_step(cb, k, mu):
+    f, g = scaled((9, 31, 37), k)
+    out = cb.tf_shrink(f, mu, False)
+    assert mu == 0.0 or not torch.allclose(out, f, rtol=0.1)  # the threshold takes effect
+    assert torch.equal(cb.tf_shrink(g, mu * 2.0**k, False), out * 2.0**k)
