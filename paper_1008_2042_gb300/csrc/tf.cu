@@ -341,8 +341,9 @@ constexpr int SY_OUT = 30;                       // output positions per warp al
 constexpr int SY_WARPS = SY_ROWS + 2;
 constexpr int SY_THREADS = 32 * SY_WARPS;
 
-// Each pass leaves out a factor 1/4 of its taps, which rounds nothing: shares a_0 - a_2 +- sqrt(2) a_1 and
-// 2 (a_0 + a_2), and 64 times the result. The shrinkage factor is applied to a triple's sum and difference.
+// Each pass leaves out a factor 1/4 of its taps: shares a_0 - a_2 +- sqrt(2) a_1 and 2 (a_0 + a_2), of
+// coefficients that enter as 64ths (which rounds nothing, but for values below 2^-114, and leaves no intermediate
+// larger than the taps would). The shrinkage factor is applied to a triple's sum and difference.
 // Kernels for pairs of positions take the same operations and leave the same bits.
 constexpr float SYN_R = 4.0f * R2_4;
 
@@ -384,13 +385,14 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
 #pragma unroll
         for (int ch = 1; ch < 27; ++ch) s2 = fmaf(a[ch], a[ch], s2);
         const float nrm = sqrtf(s2);
-        const float scale = nrm > mu ? 1.0f - mu / nrm : 0.0f;
+        const float scale = (nrm > mu ? 1.0f - mu / nrm : 0.0f) * (1.0f / 64.0f);
         const float sc2 = scale + scale, scr = SYN_R * scale, scn = -SYN_R * scale;
         // axis 0 (lanes): u[m + 3n] = sum over l and the lane's neighbours
         float u[9];
 #pragma unroll
         for (int mn = 0; mn < 9; ++mn) {
-            const float a0 = a[3 * mn], a2 = mn ? a[3 * mn + 2] : __fmul_rn(scale, a[3 * mn + 2]); // (channel 0 is not shrunk)
+            // (channel 0 is not shrunk)
+            const float a0 = mn ? a[3 * mn] : a[0] * (1.0f / 64.0f), a2 = mn ? a[3 * mn + 2] : __fmul_rn(scale, a[2]);
             const float q = mn ? __fmul_rn(scale, a0 - a2) : a0 - a2;
             const float up = fmaf(scr, a[3 * mn + 1], q), dn = fmaf(scn, a[3 * mn + 1], q);
             u[mn] = fmaf(mn ? sc2 : 2.0f, a0 + a2, __shfl_up_sync(0xffffffffu, up, 1)) + __shfl_down_sync(0xffffffffu, dn, 1);
@@ -412,7 +414,7 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
             // axis 2 (planes): plane cp - 1 from planes cp - 2, cp - 1, cp
             if (cp >= c_begin + 1 && out_lane) {
                 const float ends = (w_m2[0] + wv[0]) - (w_m2[2] + wv[2]);
-                float o = (fmaf(2.0f, w_m1[0] + w_m1[2], SYN_R * (w_m2[1] - wv[1])) + ends) * (1.0f / 64.0f);
+                float o = fmaf(2.0f, w_m1[0] + w_m1[2], SYN_R * (w_m2[1] - wv[1])) + ends;
                 if (positivity && o < 0.0f) o = 0.0f;
                 f[(size_t)(cp - 1) * plane + (size_t)pb * n0 + pa] = o;
             }
@@ -508,7 +510,7 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T *__restrict__ 
             s2 = fma2(a, a, s2);
         }
         const float na = sqrtf(lo2(s2)), nb = sqrtf(hi2(s2));
-        const f32x2 sc = pk(na > mu ? 1.0f - mu / na : 0.0f, nb > mu ? 1.0f - mu / nb : 0.0f);
+        const f32x2 sc = mul2(pk(na > mu ? 1.0f - mu / na : 0.0f, nb > mu ? 1.0f - mu / nb : 0.0f), splat(1.0f / 64.0f));
         const f32x2 sc2 = add2(sc, sc), scr = mul2(splat(SYN_R), sc), scn = mul2(splat(-SYN_R), sc);
         // axis 0: the even position takes lane - 1's odd one and its own odd one; the odd position takes
         // its own even one and lane + 1's even one
@@ -516,7 +518,10 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T *__restrict__ 
 #pragma unroll
         for (int mn = 0; mn < 9; ++mn) {
             f32x2 a0 = P::get(cur[3 * mn]), a1 = P::get(cur[3 * mn + 1]), a2 = P::get(cur[3 * mn + 2]);
-            if (mn == 0) a2 = mul2(sc, a2); // (channel 0 is not shrunk)
+            if (mn == 0) { // (channel 0 is not shrunk)
+                a0 = mul2(splat(1.0f / 64.0f), a0);
+                a2 = mul2(sc, a2);
+            }
             const f32x2 q = mn ? mul2(sc, sub2(a0, a2)) : sub2(a0, a2);
             const f32x2 up = fma2(scr, a1, q), dn = fma2(scn, a1, q);
             u[mn] = add2(fma2(mn ? sc2 : splat(2.0f), add2(a0, a2), pk(__shfl_up_sync(0xffffffffu, hi2(up), 1), lo2(up))),
@@ -539,8 +544,8 @@ k_tf_synth_shrink_pair(int n0, int n1, int n2, int chunk, const T *__restrict__ 
                 wv[n] = add2(fma2(splat(2.0f), mid[n], s_up[buf][w - 1][n][lane]), s_dn[buf][w + 1][n][lane]);
             if (cp >= c_begin + 1 && out_lane) {
                 const f32x2 ends = sub2(add2(w_m2[0], wv[0]), add2(w_m2[2], wv[2]));
-                const f32x2 o64 = add2(fma2(splat(2.0f), add2(w_m1[0], w_m1[2]), mul2(splat(SYN_R), sub2(w_m2[1], wv[1]))), ends);
-                float2 o = make_float2(lo2(o64) * (1.0f / 64.0f), hi2(o64) * (1.0f / 64.0f));
+                const f32x2 o2 = add2(fma2(splat(2.0f), add2(w_m1[0], w_m1[2]), mul2(splat(SYN_R), sub2(w_m2[1], wv[1]))), ends);
+                float2 o = make_float2(lo2(o2), hi2(o2));
                 if (positivity) {
                     o.x = o.x < 0.0f ? 0.0f : o.x;
                     o.y = o.y < 0.0f ? 0.0f : o.y;

@@ -41,3 +41,13 @@ def test_range_of_the_fused_step(cb, k, mu):
     out = cb.tf_shrink(f, mu, False)
     assert mu == 0.0 or not torch.allclose(out, f, rtol=0.1)  # the threshold takes effect
     assert torch.equal(cb.tf_shrink(g, mu * 2.0**k, False), out * 2.0**k)
+
+
+# 38 and 37 columns: the kernels for one position per lane and, in 16 bits, for a pair
+@pytest.mark.parametrize("nx", [37, 38])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("k, mu", [(-40, 3.0), (60, 3.0), (122, 0.0)])
+def test_range_of_the_synthesis(cb, k, mu, dtype, nx):
+    a, b = (v.to(dtype) for v in scaled((27, 9, 31, nx), k))
+    out = cb.tf_synthesize_shrink(a, mu, False)
+    assert torch.equal(cb.tf_synthesize_shrink(b, mu * 2.0**k, False), out * 2.0**k)
