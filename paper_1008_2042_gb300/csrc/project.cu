@@ -125,10 +125,11 @@ static cbct_status choose_group(const GeomDev &G, int threads, int mode, int sto
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return check_cuda(e, "project device");
-    using Key = std::tuple<int, int, int, int, int, int, int>;
+    const int rows = fill == FILL_GATHER ? proj_rows_per_thread(G) : 2;
+    using Key = std::tuple<int, int, int, int, int, int, int, int>; // all that the occupancy and the plans depend on
     static std::mutex mu;
     static std::map<Key, GroupChoice> cache;
-    const Key key{dev, mode, storage, threads, G.nz, fill, forced};
+    const Key key{dev, mode, storage, threads, rows, G.nz, fill, forced};
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
@@ -144,7 +145,7 @@ static cbct_status choose_group(const GeomDev &G, int threads, int mode, int sto
         const int groups = i < PROJECT_N_GROUP_SIZES ? 1 : 2, sg = groups == 1 ? PROJECT_GROUP_SIZES[i] : 56;
         if ((use_forced && (sg != forced || groups > 1)) || !make_plan(G, threads, sg, groups, &c)) continue;
         const void *fn = nullptr;
-        cbct_status r = optin(c.qw, mode, storage, fill == FILL_GATHER ? proj_rows_per_thread(G) : 2, fill, &fn);
+        cbct_status r = optin(c.qw, mode, storage, rows, fill, &fn);
         if (r != CBCT_OK) return r;
         int nb = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads + 32, c.smem);
