@@ -54,14 +54,19 @@ struct BpPlan {
 constexpr int BP_MAX_WARPS = 16;
 constexpr int BP_ZC[] = {8, 12, 14, 16, 18};
 
-// The voxels per thread that cover a column at the least cost: its planes, about one and a half more per
-// chunk for its first plane and set-up, and a third more for a chunk that z = 0 cuts (its
-// rows are tested one by one). Measured (12 | 14 | 16 | 18): 512x512x70 1268 | 1183 | 1321 | 1249 us, 128x128x18
-// 137 | 154 | 172 | 100 us, 256x256x64 (meeting at z = 0 for 16 only) 503 | 470 | 395 | 493 us, 256x256x35 (one of three
-// chunks of 12 cut, both of 18) 320 | 350 | 400 | 349 us. Where even 8 slices leave few warps, 8 voxels
+// The voxels per thread that cover a column at the least cost: its planes, two more per chunk for
+// its first plane and set-up, a sixteenth more for a chunk that z = 0 cuts (its rows are tested one by
+// one) and 3% more for chunks of 16 and 18, which spill. Measured (8 | 12 | 14 | 16 | 18): 512x512x70
+// 1464 | 1241 | 1177 | 1286 | 1241 us, 256x256x64 (meeting at z = 0 for 8 and 16 only) 507 | 490 | 462 | 393 | 487 us,
+// 256x256x48 397 | 321 | 374 | 333 | 395 us, 512x512x30 356 | 342 | 380 | 327 | 358 us (20 views), 1000x1000x20 542 | 479 |
+// 524 | 567 | 612 us (12 views). Where even 8 slices leave few warps, 8 voxels
 // (64x64x16: 24.6 us, with 16 32.8 us). Slices double until the chip has about 96 warps per
 // SM to draw from: 256x256x35 with 1 | 2 | 4 | 8 slices 403 | 354 | 339 | 356 us, 128x128x18 456 |
 // 240 | 131 | 104 us, 512x512x70 1254 | 1311 | 1393 | 1583 us (less of the table is shared in L1).
+//
+// An even volume's middle plane is 0 only where nz / 2 dz and the corner round alike (always for pitches
+// of few bits, for about a third of the usual ones). Elsewhere it is +-1e-6 mm, and one or both of the
+// chunks that meet there count as cut: 256x256x56 360 us with dz = 1.0, 401 us with 1.7.
 static BpPlan bp_plan(const GeomDev &G)
 {
     BpPlan p{};
@@ -69,14 +74,15 @@ static BpPlan bp_plan(const GeomDev &G)
     const long long sms = device_sm_count();
     int chunks = 0;
     double best = 1e30;
-    const double orbit = -(double)G.z0 / G.dz; // the plane z = 0
     for (int zc : BP_ZC) {
         const int n = (G.nz + zc - 1) / zc;
         double cost = 0.0;
         for (int c = 0; c < n; ++c) {
             const int z = G.nz < zc ? 0 : c * zc < G.nz - zc ? c * zc : G.nz - zc;
-            const bool cut = z < orbit && orbit < z + zc;
-            cost += (zc + 1.5) * (cut ? 4.0 / 3.0 : 1.0);
+            // (the kernel's own planes; it takes a lowest plane just above 0 for a cut one)
+            const float bot = std::fmaf((float)z, G.dz, G.z0), top = std::fmaf((float)(z + zc), G.dz, G.z0);
+            const bool cut = top > 0.0f && bot != 0.0f && bot < 1e-2f * G.dz;
+            cost += (zc + 2.0) * (cut ? 17.0 / 16.0 : 1.0) * (zc >= 16 ? 1.03 : 1.0);
         }
         if (cost < best) {
             best = cost;
