@@ -430,8 +430,13 @@ k_tf_synth_shrink(int n0, int n1, int n2, int chunk, const TA_T *__restrict__ al
 template <typename TA_T>
 static cbct_status launch_tf_analyze_t(int n0, int n1, int n2, const float *f, TA_T *alpha, cudaStream_t st)
 {
-    // (the pair kernel's tiles of AP_B rows reach the grid's limit along y at half the rows that are accepted)
+    // The pair kernel's tiles are twice as wide, so that a row's last tile may do twice the columns in vain: taken
+    // up to 4/3 of the general kernel's (all widths above 32), and of FP32 rows of whole sectors, which the general
+    // kernel also writes well, up to 5/4 (pair | general: 18x512x64 24.6 | 18.9 us, 96x256x100 57.4 | 47.1 us, 160x256x100
+    // 72.4 | 82.5 us, 98x256x100 105 | 119 us; BF16 96x256x100 35.0 | 41.2 us). (Its AP_B rows reach the grid's limit along y at half the rows that are accepted.)
+    const int cols = (n0 + 63) / 64 * 64, general_cols = (n0 + TA - 1) / TA * TA;
     const bool pair = n0 % 2 == 0 && (reinterpret_cast<uintptr_t>(alpha) & (2 * sizeof(TA_T) - 1)) == 0 &&
+                      (sizeof(TA_T) == 4 && n0 % 8 == 0 ? 4LL * cols <= 5LL * general_cols : 3LL * cols <= 4LL * general_cols) &&
                       (n1 + AP_B - 1) / AP_B <= MAX_GRID_Y;
     const auto kernel = pair ? k_tf_analyze_pair<TA_T> : k_tf_analyze<TA_T>;
     const int ta = pair ? 64 : TA, tb = pair ? AP_B : TB;

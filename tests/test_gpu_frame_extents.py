@@ -51,3 +51,19 @@ def test_range_of_the_synthesis(cb, k, mu, dtype, nx):
     a, b = (v.to(dtype) for v in scaled((27, 9, 31, nx), k))
     out = cb.tf_synthesize_shrink(a, mu, False)
     assert torch.equal(cb.tf_synthesize_shrink(b, mu * 2.0**k, False), out * 2.0**k)
+
+
+# widths about a warp (32 and 34 columns), and FP32 rows of whole sectors that leave a pair tile half empty (72, 96)
+# or not (104, 160), each beside the next even width: both kernels agree bit for bit
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("nx", [32, 34, 72, 74, 96, 98, 104, 160, 162])
+def test_analysis_widths(cb, nx, dtype):
+    shape = (5, 13, nx)
+    f = torch.randn(shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(7))
+    a = cb.tf_analyze(f, dtype=dtype)
+    single = torch.empty(a.numel() + 1, dtype=dtype, device="cuda")[1:].view(a.shape)
+    assert torch.equal(a, cb.tf_analyze(f, out=single))
+    ref = oracle.tf_analyze(f.cpu().numpy())
+    eps = 0.0 if dtype == torch.float32 else 2.0**-8
+    err = np.abs(a.float().cpu().numpy() - ref)
+    assert np.all(err <= 10 * 2.0**-24 * float(f.abs().max()) + eps * np.abs(ref) * 1.001 + 2.0**-25)
