@@ -297,13 +297,14 @@ static cudaError_t resident_blocks(const void *kernel, int threads, Residency &c
 // Planes per block along axis 2 (shrink + synthesis and the fused step): the split whose blocks fill whole
 // waves of the resident slots best, counting the two extra planes each block recomputes
 // at its start (a block's cost grows with chunk + 2).
-static int fused_chunk(long long tiles, int n2, int slots)
+// *cost, if given: the waves times the planes of a block.
+static int fused_chunk(long long tiles, int n2, int slots, long long *cost = nullptr)
 {
     int best = n2;
     double best_eff = -1.0;
-    for (int nch = 1; nch <= n2; ++nch) {
-        const int chunk = (n2 + nch - 1) / nch;
-        if (nch > 1 && chunk == (n2 + nch - 2) / (nch - 1)) continue; // same split as nch - 1
+    // (every split into equal chunks once: from one length to the next shorter one)
+    for (int nch = 1, chunk = n2;; nch = (n2 + chunk - 2) / (chunk - 1)) {
+        chunk = (n2 + nch - 1) / nch;
         const long long nb = tiles * ((n2 + chunk - 1) / chunk);
         const long long waves = (nb + slots - 1) / slots;
         const double eff = (double)n2 / ((double)((n2 + chunk - 1) / chunk) * (chunk + 2)) * (double)nb /
@@ -311,7 +312,9 @@ static int fused_chunk(long long tiles, int n2, int slots)
         if (eff > best_eff + 1e-9) {
             best_eff = eff;
             best = chunk;
+            if (cost) *cost = waves * (chunk + 2);
         }
+        if (chunk == 1) break;
     }
     return best;
 }
@@ -640,14 +643,13 @@ namespace cbct {
 // lanes by shuffles, of neighbouring rows within the pair or through shared memory, of
 // neighbouring planes in registers, finishing the output plane one behind the analysed one.
 //
-// Bound by instruction issue (57%), the packed-FP32 pipe and the shuffles; 16 warps (118
+// Bound by instruction issue (57%), the packed-FP32 pipe and the shuffles; 16 warps (120
 // registers) per SM. 512x512x70: 334 us (one row per warp, 22 warps: 377 us), z-fastest as in
-// the iteration 363 us (421 us); 12 warps with more registers 484 us.
+// the iteration 363 us (421 us). Volumes whose tiles of 16 warps end in a poor last wave take 12 warps (rule at
+// the launcher).
 // ------------------------------------------------------------------------------------
-constexpr int FR_WARPS = 16;
-constexpr int FR_ROWS = 2 * FR_WARPS - 4; // output rows per block along axis 1
-constexpr int FR_OUT = 28;                // output positions per warp along axis 0
-constexpr int FR_THREADS = 32 * FR_WARPS;
+constexpr int FR_OUT = 28; // output positions per warp along axis 0
+constexpr int fr_rows(int warps) { return 2 * warps - 4; } // output rows per block along axis 1
 
 // The frame with plain taps: [1, 2, 1], [1, 0, -1] and [1, -2, 1] stand for 4 h_0, (4 / sqrt(2)) h_1
 // and -4 h_2, so that a triple takes four operations. Of x / 64, a coefficient with j factors h_1 is then
@@ -670,10 +672,12 @@ __device__ __forceinline__ void syn_shares_plain(f32x2 a0, f32x2 a1, f32x2 a2, f
     half = sub2(a0, a2);
 }
 
-__global__ void __launch_bounds__(FR_THREADS, 1)
+template <int FR_WARPS>
+__global__ void __launch_bounds__(32 * FR_WARPS, 1)
 k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__restrict__ x, float mu, int positivity,
                   float *__restrict__ fnew, const float *__restrict__ fold, float coef, float *__restrict__ vout)
 {
+    constexpr int FR_ROWS = fr_rows(FR_WARPS);
     chain_wait();
     __shared__ f32x2 s_t[2][FR_WARPS][3][32];                      // axis-2 analysis of each pair
     __shared__ float s_up[2][FR_WARPS][3][32], s_dn[2][FR_WARPS][3][32]; // axis-1 synthesis shares to the pairs beside
@@ -787,19 +791,42 @@ k_tf_shrink_fused(int n0, int n1, int n2, int p0, int chunk, const float *__rest
 
 cbct_status tf_prepare() { return CBCT_OK; }
 
-cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *x, float mu, int positivity, float *fnew,
-                                   const float *fold, float coef, float *vout, cudaStream_t st)
+// A launch of the fused step with WARPS warps per block, and its cost in planes of a block, one after another.
+struct FusedPlan {
+    dim3 grid;
+    int chunk;
+    long long cost;
+};
+template <int WARPS> static cudaError_t fused_plan(int n0, int n1, int n2, FusedPlan *p)
 {
     static Residency residency;
     int slots = 0;
-    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_shrink_fused), FR_THREADS, residency, &slots);
+    const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_shrink_fused<WARPS>), 32 * WARPS, residency, &slots);
+    if (e != cudaSuccess) return e;
+    const int tx = (n0 + FR_OUT - 1) / FR_OUT, ty = (n1 + fr_rows(WARPS) - 1) / fr_rows(WARPS);
+    p->chunk = fused_chunk((long long)tx * ty, n2, slots, &p->cost);
+    p->grid = dim3(tx, ty, (n2 + p->chunk - 1) / p->chunk);
+    return cudaSuccess;
+}
+
+// 16 warps share their halo rows best, but their few large blocks may leave most of a wave empty (256x256x8: 100
+// blocks on 152 SMs). A plane costs a block of 16 warps 1.85 us and one of 12 warps 1.40 us (nearly the same at every
+// size), so 12 warps where their planes are fewer than 1.32 times as many. Measured (16 | 12 warps, planes): 256x256x8 19.2 | 15.0 us (10 |
+// 10), 256x256x20 33.9 | 31.3 us (18 | 22), 450x430x60 223.7 | 220.5 us (124 | 160), 512x512x20 110 | 118 us (60 | 84),
+// 512x512x70 332 | 354 us (185 | 259). 8, 10, 11 and 14 warps were no better where 12 win, but for a few per cent.
+cbct_status launch_tf_shrink_fused(int n0, int n1, int n2, int p0, const float *x, float mu, int positivity, float *fnew,
+                                   const float *fold, float coef, float *vout, cudaStream_t st)
+{
+    FusedPlan p{}, q{};
+    cudaError_t e = fused_plan<16>(n0, n1, n2, &p);
+    if (e == cudaSuccess) e = fused_plan<12>(n0, n1, n2, &q);
     if (e != cudaSuccess) return check_cuda(e, "tf_shrink_fused occupancy");
-    const long long tiles = (long long)((n0 + FR_OUT - 1) / FR_OUT) * ((n1 + FR_ROWS - 1) / FR_ROWS);
-    const int chunk = fused_chunk(tiles, n2, slots);
-    dim3 grid((n0 + FR_OUT - 1) / FR_OUT, (n1 + FR_ROWS - 1) / FR_ROWS, (n2 + chunk - 1) / chunk);
+    const bool few = 100 * q.cost < 132 * p.cost;
+    const auto kernel = few ? k_tf_shrink_fused<12> : k_tf_shrink_fused<16>;
+    if (few) p = q;
     CBCT_TIMED(CBCT_KERNEL_TF_SYNTH, st,
-               launch_chained(k_tf_shrink_fused, grid, dim3(32, FR_WARPS), 0, st, n0, n1, n2, p0, chunk, x, mu, positivity, fnew, fold,
-                                                                      coef, vout));
+               launch_chained(kernel, p.grid, dim3(32, few ? 12 : 16), 0, st, n0, n1, n2, p0, p.chunk, x, mu, positivity, fnew,
+                              fold, coef, vout));
     return check_cuda(cudaGetLastError(), "tf_shrink_fused launch");
 }
 

@@ -67,3 +67,13 @@ def test_analysis_widths(cb, nx, dtype):
     eps = 0.0 if dtype == torch.float32 else 2.0**-8
     err = np.abs(a.float().cpu().numpy() - ref)
     assert np.all(err <= 10 * 2.0**-24 * float(f.abs().max()) + eps * np.abs(ref) * 1.001 + 2.0**-25)
+
+
+# blocks of 12 warps (20 rows; 256x256x8 leaves blocks of 16 warps a third of the SMs idle) and of 16 warps (28 rows):
+# whole tiles, one row and one column more, the z-fastest order of a thin volume
+@pytest.mark.parametrize("shape", [(1, 20, 28), (5, 21, 29), (30, 40, 57), (8, 256, 256), (40, 84, 128), (40, 85, 127), (128, 128, 18), (120, 130, 33)])
+def test_fused_step_block_sizes(cb, shape):
+    f = np.random.default_rng(8).standard_normal(shape).astype(np.float32)
+    out = cb.tf_shrink(torch.from_numpy(f).cuda(), 1.5, False).cpu().numpy()
+    ref = oracle.tf_synthesize(oracle.tf_shrink(oracle.tf_analyze(f), 1.5))
+    assert np.linalg.norm(out - ref) <= 1e-5 * np.linalg.norm(ref)
