@@ -294,11 +294,10 @@ static cudaError_t resident_blocks(const void *kernel, int threads, Residency &c
     return cudaSuccess;
 }
 
-// Planes per block along axis 2 (shrink + synthesis and the fused step): the split whose blocks fill whole
-// waves of the resident slots best, counting the two extra planes each block recomputes
-// at its start (a block's cost grows with chunk + 2).
+// Planes per block along axis 2: the split whose blocks fill whole waves of the resident slots best, counting the
+// two extra planes each block computes at its ends as `extra` (a block's cost grows with chunk + extra).
 // *cost, if given: the waves times the planes of a block.
-static int fused_chunk(long long tiles, int n2, int slots, long long *cost = nullptr)
+static int fused_chunk(long long tiles, int n2, int slots, double extra = 2.0, long long *cost = nullptr)
 {
     int best = n2;
     double best_eff = -1.0;
@@ -307,7 +306,7 @@ static int fused_chunk(long long tiles, int n2, int slots, long long *cost = nul
         chunk = (n2 + nch - 1) / nch;
         const long long nb = tiles * ((n2 + chunk - 1) / chunk);
         const long long waves = (nb + slots - 1) / slots;
-        const double eff = (double)n2 / ((double)((n2 + chunk - 1) / chunk) * (chunk + 2)) * (double)nb /
+        const double eff = (double)n2 / ((double)((n2 + chunk - 1) / chunk) * (chunk + extra)) * (double)nb /
                            ((double)waves * slots);
         if (eff > best_eff + 1e-9) {
             best_eff = eff;
@@ -448,7 +447,10 @@ static cbct_status launch_tf_analyze_t(int n0, int n1, int n2, const float *f, T
     const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(kernel), 32 * tb, residency[pair], &slots);
     if (e != cudaSuccess) return check_cuda(e, "tf_analyze occupancy");
     const long long tiles = (long long)((n0 + ta - 1) / ta) * ((n1 + tb - 1) / tb);
-    const int chunk = fused_chunk(tiles, n2, slots);
+    // The extra planes of the pair kernel are read and passed along two axes but not stored, which is what an FP32
+    // plane costs: 0.6 of one (with 2 | 0.6: 288x512x64 218 | 171 us, 82x256x100 95 | 71 us, 256x256x20 28.7 |
+    // 25.9 us, 512x512x70 328 | 322 us). 16-bit planes cost as much to compute as to store (256x256x20 BF16 16.9 | 18.2 us).
+    const int chunk = fused_chunk(tiles, n2, slots, pair && sizeof(TA_T) == 4 ? 0.6 : 2.0);
     dim3 grid((n0 + ta - 1) / ta, (n1 + tb - 1) / tb, (n2 + chunk - 1) / chunk);
     CBCT_TIMED(CBCT_KERNEL_TF_ANALYZE, st, kernel<<<grid, dim3(32, tb), 0, st>>>(n0, n1, n2, chunk, f, alpha));
     return check_cuda(cudaGetLastError(), "tf_analyze launch");
@@ -804,7 +806,7 @@ template <int WARPS> static cudaError_t fused_plan(int n0, int n1, int n2, Fused
     const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(k_tf_shrink_fused<WARPS>), 32 * WARPS, residency, &slots);
     if (e != cudaSuccess) return e;
     const int tx = (n0 + FR_OUT - 1) / FR_OUT, ty = (n1 + fr_rows(WARPS) - 1) / fr_rows(WARPS);
-    p->chunk = fused_chunk((long long)tx * ty, n2, slots, &p->cost);
+    p->chunk = fused_chunk((long long)tx * ty, n2, slots, 2.0, &p->cost);
     p->grid = dim3(tx, ty, (n2 + p->chunk - 1) / p->chunk);
     return cudaSuccess;
 }
