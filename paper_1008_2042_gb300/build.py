@@ -38,7 +38,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     """Compile every CUDA source and link the shared library; returns its path."""
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
-    headers = [os.path.join(CSRC, h) for h in ("cbct_internal.cuh", "async.cuh", "project.cuh", "project_kernel.cuh")]
+    headers = [os.path.join(CSRC, h) for h in ("cbct_internal.cuh", "async.cuh", "f32x2.cuh", "project.cuh", "project_kernel.cuh")]
     headers.append(os.path.join(ROOT, "include", "cbcttf.h"))
     jobs = []
     for src in SOURCES:

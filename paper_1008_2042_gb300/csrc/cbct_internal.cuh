@@ -138,8 +138,6 @@ template <> __device__ __forceinline__ void store_stream<__nv_bfloat16>(__nv_bfl
 }
 template <> __device__ __forceinline__ void store_stream<__half>(__half *p, float v) { __stcs(p, __float2half_rn(v)); }
 
-static inline size_t storage_bytes(int storage) { return storage == ST_F32 ? 4 : 2; }
-
 // Opts a kernel into more than 48 KB of dynamic shared memory. The attribute belongs to
 // the function on one device, so it is set once per device (`done` holds one bit each).
 template <typename Kernel>
@@ -256,11 +254,6 @@ int device_sm_count();
 int project_num_blocks(const GeomDev &G);
 // Elements of a volume in the internal layout.
 static inline size_t internal_elems(const GeomDev &G) { return (size_t)G.nx * G.ny * G.zp; }
-// Bytes past the end of a volume that the projector may read (the unpadded layout's last
-// z-line is read up to a multiple of 4 values): every volume buffer passed to
-// launch_project is allocated with at least this much slack, and its base is 16-byte aligned.
-constexpr size_t PROJECT_VOLUME_SLACK = 64;
-
 // Dynamic shared memory a projector block may use (opted in per kernel).
 constexpr size_t PROJECT_SMEM_LIMIT = 200 * 1024;
 

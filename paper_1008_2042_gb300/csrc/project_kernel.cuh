@@ -29,31 +29,10 @@
 // project_q*.cu units (compiled in parallel) and launched from project.cu.
 #pragma once
 #include "async.cuh"
+#include "f32x2.cuh"
 #include "project.cuh"
 
 namespace cbct {
-
-// Two FP32 operations in one instruction, on pairs held as 64-bit registers; each half is
-// rounded like the scalar operation.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 
 // Shared-memory accesses by 32-bit address (byte offsets are added to it in one instruction).
 __device__ __forceinline__ ulonglong2 lds_quad(unsigned a)

@@ -12,10 +12,9 @@
 
 namespace cbct {
 
-// Fixed scratch: the z-contiguous copy of the input volume, plus the slack the projector
-// may read past a volume's end. Every GPU that loads the library holds this array (16 MiB)
-// until the process exits.
-static __device__ __align__(256) float g_static_volume[CBCT_PROJECT_STATIC_MAX_VOXELS + PROJECT_VOLUME_SLACK / 4];
+// Fixed scratch: the z-contiguous copy of the input volume. Every GPU that loads the library
+// holds this array (16 MiB) until the process exits.
+static __device__ __align__(256) float g_static_volume[CBCT_PROJECT_STATIC_MAX_VOXELS];
 // Fixed scratch for trace records (8 MiB): a call whose table is larger projects its (view,
 // imager column) pairs batch by batch. The largest record (nx + ny = 4096) is 33 KB.
 constexpr size_t STATIC_TRACE_BYTES = 8u << 20;

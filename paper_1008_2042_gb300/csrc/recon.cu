@@ -246,7 +246,7 @@ static size_t max_partials(const cbct_geometry *g)
 {
     GeomDev G = level_geom(g, 0);
     size_t a = (size_t)project_num_blocks(G);
-    // backprojection blocks are most numerous with one z voxel per thread at the finest grid
+    // (both are largest on the finest grid; the adjoint's with the smallest tile and chunk)
     size_t b = (size_t)backproject_max_blocks(G);
     return a > b ? a : b;
 }
@@ -261,7 +261,7 @@ static size_t work_layout(const cbct_geometry *g, char *base, Work *w)
         off += align256(bytes);
         return p;
     };
-    const size_t VB = 4 * N + PROJECT_VOLUME_SLACK; // volumes the projector may read past the end
+    const size_t VB = 4 * N;
     float *X = (float *)take(VB), *X2 = (float *)take(VB), *P = (float *)take(VB), *S = (float *)take(VB);
     float *Fa = (float *)take(VB), *Fb = (float *)take(VB);
     void *R = take(4 * M), *Q = take(4 * M); // sized for FP32, the widest storage type
@@ -536,7 +536,7 @@ extern "C" cbct_status cbct_project_ex(const cbct_geometry *gc, const float *f, 
     if (!valid_dtype(g_type)) return set_error(CBCT_ERR_INVALID_ARG, "project: unknown storage type %d", (int)g_type);
     cbct_geometry *g = const_cast<cbct_geometry *>(gc);
     const GeomDev G = level_geom(g, 0);
-    const size_t vol_bytes = align256(sizeof(float) * internal_elems(G) + PROJECT_VOLUME_SLACK);
+    const size_t vol_bytes = align256(sizeof(float) * internal_elems(G));
     TRY(ensure_scratch(g, vol_bytes + trace_table_bytes(G)));
     cudaStream_t st = (cudaStream_t)stream;
     float *fz = g->d_scratch;

@@ -15,6 +15,7 @@
 // described at their kernels. The public transforms are bandwidth bound: 4 B in + 108 B
 // out per voxel for W, 108 B in + 4 B out for the shrink/synthesis (FP32 coefficients).
 #include "cbct_internal.cuh"
+#include "f32x2.cuh"
 
 namespace cbct {
 
@@ -27,47 +28,6 @@ __device__ __forceinline__ int wrapi(int i, int n)
     i %= n;
     return i < 0 ? i + n : i;
 }
-
-// Two FP32 values in one 64-bit register; each half rounds like the scalar operation.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pk(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float lo2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return a;
-}
-__device__ __forceinline__ float hi2(f32x2 v)
-{
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-    return b;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 splat(float v) { return pk(v, v); }
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, splat(-1.0f), a); } // a - b, rounded once
 
 // Analysis along one axis for the window (f(x-1), f(x), f(x+1)) = (p, c, n):
 // alpha_l(x) = h_l[-1] f(x+1) + h_l[0] f(x) + h_l[1] f(x-1).

@@ -32,7 +32,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 
 KERNEL_SOURCES = {
-    "k_project": ("project.cu", "project.cuh", "project_kernel.cuh", "project_trace.cu", "async.cuh"),
+    "k_project": ("project.cu", "project.cuh", "project_kernel.cuh", "project_trace.cu", "async.cuh",
+                  "f32x2.cuh"),
     "k_backproject": ("backproject.cu",),
 }
 OPS = {"k_project": "project", "k_backproject": "backproject"}
