@@ -24,7 +24,8 @@
 // straddling row became one saturating multiply and the chunks whole it took 1.63 ms, with
 // the plane heights computed for each plane 1.25 ms; with the warps of a block on the same
 // patch taking turns at the views, 128x128x18 takes 103 us (200 before), 64x64x16 21 us (61).
-// Chunks that begin or end at z = 0 take the loops of one side: 256x256x64 457 -> 395 us, 128x128x32 145 -> 119 us.
+// Chunks that begin or end at z = 0 take the loops of one side where the middle plane rounds to 0 (see bp_plan):
+// 256x256x64 457 -> 395 us, 128x128x32 145 -> 119 us.
 #include "cbct_internal.cuh"
 
 #include <math_constants.h>
@@ -229,7 +230,7 @@ __device__ __forceinline__ void bp_planes(const GeomDev &G, const BpVisit &q, co
     }
 }
 
-// Register budget: 64, two resident blocks of 512 threads.
+// Register budget: 64, two resident blocks of 512 threads (chunks of 18 voxels spill 56-64 bytes, those of 16 four).
 // FLAT: each lane walks its own list of candidates (view, imager column), so a warp runs for the
 // longest per-lane total instead of the widest shadow in every view: fewer idle lanes where
 // shadows are about one column wide.

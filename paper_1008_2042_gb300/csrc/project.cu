@@ -33,7 +33,8 @@ size_t project_smem_bytes(const GeomDev &G)
 // the columns, so fewer passes end in a scan (each pass costs about 8 instructions per column
 // and 60 around them), but the longest chain doubles. The split with the least total work plus
 // longest chain. Measured with groups of 80 (4 | 8): 18 quads on 6 warps 661 | 703 us, 16 quads
-// 206 | 187 us, 9 quads 315 | 355 us, 5 quads 185 | 211 us (the orders hold for the sizes used).
+// 206 | 187 us, 9 quads 315 | 355 us, 5 quads 185 | 211 us, as the costs order them; in between
+// the costs may lie within 3-6% of each other, and the order was not measured there.
 static int quads_per_warp(const GeomDev &G, int threads, int sg)
 {
     const int nq = G.zp / 4, warps = threads / 32;

@@ -11,7 +11,8 @@ namespace cbct {
 
 constexpr int PROJ_THREADS = 192; // consumer threads per block at most; each owns one or two imager rows
 #ifndef CBCT_PROJ_MIN_BLOCKS
-// resident blocks per SM the register budget is sized for (72 registers a thread)
+// resident blocks per SM the register budget is sized for (72 registers a thread; the kernels with 8 quads per warp
+// and two rows per thread spill 24 bytes, in the modes of CGLS up to 44)
 #define CBCT_PROJ_MIN_BLOCKS 4
 #endif
 // fewest threads of a block: short imagers would leave the table build to one warp

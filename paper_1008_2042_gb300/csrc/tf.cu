@@ -157,8 +157,9 @@ k_tf_analyze(int n0, int n1, int n2, int chunk, const float *__restrict__ f, TA_
 // and axis-1 passes of each plane done once (those of the two planes before stay in registers).
 // Bound by the 27 written channels: 512x512x70 FP32 334 us (6.2 TB/s; one position per lane and three
 // planes in shared memory 360 us), BF16 198 us (240), 256x256x64 74 (76) and 44 us (62). Blocks of
-// 4 rows and 102 registers, five per SM; with 80 registers 336 | 245 us, blocks of 8 rows 330 | 221 us but
-// 84 us at 256x256x64 FP32 (the last wave), 2 rows 341 | 256 us. An odd n0 takes the general kernel.
+// 4 rows, 96 registers, five per SM; with 80 registers 336 | 245 us, blocks of 8 rows 330 | 221 us but
+// 84 us at 256x256x64 FP32 (the last wave), 2 rows 341 | 256 us. An odd n0 takes the general kernel, and so do the
+// widths that leave too much of its tiles idle (rule at the launcher).
 constexpr int AP_B = 4, AP_THREADS = 32 * AP_B, AP_BLOCKS = 5;
 template <typename T>
 __global__ void __launch_bounds__(AP_THREADS, AP_BLOCKS)
@@ -606,8 +607,8 @@ namespace cbct {
 // neighbouring planes in registers, finishing the output plane one behind the analysed one.
 //
 // Bound by instruction issue (57%), the packed-FP32 pipe and the shuffles; 16 warps (120
-// registers) per SM. 512x512x70: 334 us (one row per warp, 22 warps: 377 us), z-fastest as in
-// the iteration 363 us (421 us). Volumes whose tiles of 16 warps end in a poor last wave take 12 warps (rule at
+// registers) per SM. 512x512x70: 333 us (one row per warp, 22 warps: 377 us), z-fastest as in
+// the iteration 358 us (416 us). Volumes whose tiles of 16 warps end in a poor last wave take 12 warps (rule at
 // the launcher).
 // ------------------------------------------------------------------------------------
 constexpr int FR_OUT = 28; // output positions per warp along axis 0
